@@ -166,11 +166,12 @@ int msat_step(msat_ctx *ctx, int32_t n_steps, float *loss_out, int64_t *cost_out
  * stream); the results are bit for bit those of the plain launches.  It is
  * ignored while kernel timing (msat_profile_enable) is on.  A graph holds
  * the context's device pointers; it is released with the context.
- * Small instances (B <= 64, 4 n B + m B floats within 200 KiB of shared
- * memory, no variable with more than 32736 occurrences) run all their steps
- * in one single-CTA launch holding the state in shared memory, again with
- * the same bits; MSAT_STEP_PER_PASS keeps them on the per-pass kernels (for
- * comparison), as does kernel timing.
+ * Small instances (one restart's x, moments, tanh(x) and clause values
+ * within one SM's shared memory: n up to about 6000 at 4.3 clauses a
+ * variable) run all their steps and the final evaluation in one launch of
+ * one block per restart, again with the same bits, where that is the faster
+ * route for the instance, B and n_steps; MSAT_STEP_PER_PASS keeps them on
+ * the per-pass kernels (for comparison), as does kernel timing.
  */
 #define MSAT_STEP_NO_FINAL_EVAL 1u
 #define MSAT_STEP_GRAPH 2u
@@ -349,8 +350,10 @@ typedef struct {
     int32_t max_degree;   /* most occurrences of one variable                  */
     int32_t n_heavy;      /* variables whose occurrence sum is split across warps */
     int32_t uniform_len;  /* common clause length, or 0 if lengths differ      */
-    int32_t small_kernel; /* 1: msat_step runs the single-CTA kernel (all steps
-                             of a call in one launch, state in shared memory) */
+    int32_t small_kernel; /* 1: msat_step runs the one-block-per-restart kernel
+                             (all steps of a call in one launch, state in
+                             shared memory; calls of a few steps with many
+                             restarts may still take the per-pass kernels)     */
 } msat_info;
 
 int msat_get_info(msat_ctx *ctx, msat_info *info);
@@ -483,8 +486,8 @@ typedef struct {
 
 typedef struct {
     int64_t submitted, completed, failed, cancelled;
-    int32_t queued, running, peak_running;
-    int32_t small_direct;  /* requests small enough for the single-CTA kernel: they
+    int32_t queued, running, peak_running;  /* running: in the slot table or direct */
+    int32_t small_direct;  /* requests small enough for the one-block-per-restart kernel: they
                               take all their steps in one launch on a side stream
                               as soon as they are admitted, outside the slot table */
     int64_t hbm_in_use, hbm_budget, rounds, graph_captures;

@@ -256,7 +256,31 @@ int msat::ctx_create(msat_ctx **out, int32_t n_vars, int64_t n_clauses, const in
         const int rrc = build_block_rows(n_vars, m, kfix, coff, lit, weights, lblk, ro);
         if (rrc) return rrc;
     }
-    scatter_occurrences(n_vars, m, hc, block_rows ? &ro.row : nullptr);
+    // a forced row order is a request for the per-pass kernels
+    SoloHost solo;
+    bool use_solo = cfg.row_order != 2 && build_solo(n_vars, m, kfix, max_len, max_deg, hc, solo);
+    if (use_solo) {
+        int dev = 0;
+        cudaGetDevice(&dev);
+        if (cudaDeviceGetAttribute(&solo.dev.sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
+            cudaGetLastError();
+            solo.dev.sms = 152;
+        }
+        DevInst shape{};
+        shape.n = n_vars;
+        shape.B = B;
+        shape.kfix = kfix;
+        use_solo = solo_pays(solo.dev, shape, nnz, max_len, 1 << 30);  // for a long call
+    }
+    // the serving engine runs such an instance on that kernel alone: its
+    // context holds none of the per-pass kernels' lists and buffers
+    const bool solo_only = use_solo && pool_alloc;
+    if (!solo_only) scatter_occurrences(n_vars, m, hc, block_rows ? &ro.row : nullptr);
+    std::vector<int64_t> solo_w;
+    if (use_solo && weights && !solo.slot.empty()) {
+        solo_w.resize((size_t)m);
+        for (int64_t j = 0; j < m; ++j) solo_w[(size_t)solo.slot[(size_t)j]] = weights[j];
+    }
     std::vector<int2> occx;
     if (expand) {
         occx.resize((size_t)nnz);
@@ -298,16 +322,21 @@ int msat::ctx_create(msat_ctx **out, int32_t n_vars, int64_t n_clauses, const in
     int32_t *d_plit = nullptr, *d_pcoff = nullptr;
     int64_t *d_pw = nullptr;
     int64_t *d_w = nullptr;
+    unsigned char *d_slists = nullptr;
+    int32_t *d_sperm = nullptr;
+    int64_t *d_sw = nullptr;
 #define TRY_ALLOC(ptr, count)                          \
     do {                                               \
         rc = dalloc_t(c, &(ptr), (size_t)(count));     \
         if (rc) { free_all(c); delete c; return rc; }  \
     } while (0)
-    TRY_ALLOC(d_coff, m + 1);
-    TRY_ALLOC(d_lit, nnz);
+    if (!solo_only) {
+        TRY_ALLOC(d_coff, m + 1);
+        TRY_ALLOC(d_lit, nnz);
+        TRY_ALLOC(d_voff, (int64_t)n_vars + 1);
+        TRY_ALLOC(d_occ, nnz);
+    }
     if (weights) TRY_ALLOC(d_w, m);
-    TRY_ALLOC(d_voff, (int64_t)n_vars + 1);
-    TRY_ALLOC(d_occ, nnz);
     TRY_ALLOC(d_hvar, (int64_t)hvar.size());
     TRY_ALLOC(d_hch, (int64_t)hchunk0.size());
     TRY_ALLOC(d_hofc, std::max<int64_t>(1, hchunk0.back()));
@@ -318,13 +347,18 @@ int msat::ctx_create(msat_ctx **out, int32_t n_vars, int64_t n_clauses, const in
         if (kfix == 0) TRY_ALLOC(d_pcoff, m + 1);
         if (weights) TRY_ALLOC(d_pw, m);
     }
-    if (use_fstore) TRY_ALLOC(c->S.fstore, m * B);
+    if (use_solo) {
+        TRY_ALLOC(d_slists, solo.lists.size());
+        TRY_ALLOC(d_sperm, n_vars);
+        if (!solo_w.empty()) TRY_ALLOC(d_sw, m);
+    }
+    if (use_fstore && !solo_only) TRY_ALLOC(c->S.fstore, m * B);
     TRY_ALLOC(c->S.x, nB);
     TRY_ALLOC(c->S.mom, nB);
     TRY_ALLOC(c->S.vel, nB);
     TRY_ALLOC(c->S.t0, nB);
     TRY_ALLOC(c->S.t1, nB);
-    TRY_ALLOC(c->S.ubits, (m * B + 31) / 32 + 1);
+    if (!solo_only) TRY_ALLOC(c->S.ubits, (m * B + 31) / 32 + 1);
     TRY_ALLOC(c->S.bestx, nB);
 
     DevInst &I = c->I;
@@ -353,6 +387,13 @@ int msat::ctx_create(msat_ctx **out, int32_t n_vars, int64_t n_clauses, const in
     I.plit = d_plit;
     I.pcoff = d_pcoff;
     I.pw = d_pw;
+
+    if (use_solo) {
+        c->solo = solo.dev;
+        c->solo.lists = d_slists;
+        c->solo.perm = d_sperm;
+        c->solo.w = d_sw ? d_sw : d_w;
+    }
 
     DevStep &D = c->D;
     D.fwd_blocks = cfg.fwd_blocks > 0 ? cfg.fwd_blocks : fwd_grid_blocks(I);
@@ -393,11 +434,11 @@ int msat::ctx_create(msat_ctx **out, int32_t n_vars, int64_t n_clauses, const in
     sc.loss_norm = cfg.loss_norm;
     std::vector<long long> best((size_t)B, (long long)wsum);
     cudaError_t e = cudaSuccess;
-    if (!e) e = up(d_coff, coff.data(), sizeof(int32_t) * coff.size());
-    if (!e) e = up(d_lit, lit.data(), sizeof(int32_t) * lit.size());
+    if (!e && !solo_only) e = up(d_coff, coff.data(), sizeof(int32_t) * coff.size());
+    if (!e && !solo_only) e = up(d_lit, lit.data(), sizeof(int32_t) * lit.size());
     if (!e && weights) e = up(d_w, weights, sizeof(int64_t) * (size_t)m);
-    if (!e) e = up(d_voff, voff.data(), sizeof(int32_t) * voff.size());
-    if (!e) e = up(d_occ, occ.data(), sizeof(int32_t) * occ.size());
+    if (!e && !solo_only) e = up(d_voff, voff.data(), sizeof(int32_t) * voff.size());
+    if (!e && !solo_only) e = up(d_occ, occ.data(), sizeof(int32_t) * occ.size());
     if (!e) e = up(d_hvar, hvar.data(), sizeof(int32_t) * hvar.size());
     if (!e) e = up(d_hch, hchunk0.data(), sizeof(int32_t) * hchunk0.size());
     // the heavy variable of every chunk (one load per chunk block)
@@ -410,6 +451,9 @@ int msat::ctx_create(msat_ctx **out, int32_t n_vars, int64_t n_clauses, const in
     if (!e && block_rows) e = up(d_plit, ro.plit.data(), sizeof(int32_t) * ro.plit.size());
     if (!e && d_pcoff) e = up(d_pcoff, ro.pcoff.data(), sizeof(int32_t) * ro.pcoff.size());
     if (!e && d_pw) e = up(d_pw, ro.pw.data(), sizeof(int64_t) * ro.pw.size());
+    if (!e && use_solo) e = up(d_slists, solo.lists.data(), solo.lists.size());
+    if (!e && use_solo) e = up(d_sperm, solo.perm.data(), sizeof(int32_t) * solo.perm.size());
+    if (!e && d_sw) e = up(d_sw, solo_w.data(), sizeof(int64_t) * solo_w.size());
     if (!e) e = up(D.sc, &sc, sizeof(sc));
     if (!e) e = up(D.best, best.data(), sizeof(long long) * best.size());
     if (!e) e = cudaMemsetAsync(D.best_step, 0, sizeof(long long) * (size_t)B, st);
@@ -418,7 +462,7 @@ int msat::ctx_create(msat_ctx **out, int32_t n_vars, int64_t n_clauses, const in
     if (!e) e = cudaMemsetAsync(D.cost, 0, sizeof(long long) * (size_t)B, st);
     if (!e) e = cudaMemsetAsync(D.loss, 0, sizeof(float) * (size_t)B, st);
     if (!e) e = cudaMemsetAsync(D.hcount, 0, sizeof(unsigned) * std::max<size_t>(1, hvar.size() * (size_t)G), st);
-    if (!e) e = cudaMemsetAsync(c->S.ubits, 0, sizeof(uint32_t) * (size_t)((m * B + 31) / 32 + 1), st);
+    if (!e && !solo_only) e = cudaMemsetAsync(c->S.ubits, 0, sizeof(uint32_t) * (size_t)((m * B + 31) / 32 + 1), st);
     if (!e) e = launch_init(I, c->S, cfg.seed_x, st);
     if (!e) e = cudaStreamSynchronize(st);  // host vectors above are freed on return
     if (e) {
@@ -515,18 +559,25 @@ static cudaError_t plain_steps(msat_ctx *c, int64_t n_steps) {
     return e;
 }
 
-// k steps by the fastest route that gives the same bits: the single-CTA
-// kernel for small instances, captured graphs when asked, else plain
-// launches (always plain while kernel timing is on, so every pass is timed).
-static cudaError_t run_steps(msat_ctx *c, int64_t k, uint32_t flags) {
-    if (c->prof_on) return plain_steps(c, k);
-    if (!(flags & MSAT_STEP_PER_PASS) && small_fits(c->I, c->max_deg)) {
-        cudaError_t e = cudaSuccess;
-        for (int64_t done = 0; done < k && !e; done += (1 << 30))
-            e = launch_small_steps(c->I, c->S, c->D, (int)std::min<int64_t>(k - done, 1 << 30), c->stream);
+// k steps and, if asked, the evaluation of the final x by the fastest route
+// that gives the same bits: the one-block-per-restart kernel for small
+// instances, captured graphs when asked, else plain launches (always plain
+// while kernel timing is on, so every pass is timed).
+static cudaError_t run_steps(msat_ctx *c, int64_t k, uint32_t flags, bool final_eval) {
+    cudaError_t e = cudaSuccess;
+    if (!c->prof_on && !(flags & MSAT_STEP_PER_PASS) && c->solo.lists &&
+        solo_pays(c->solo, c->I, c->nnz, c->max_len, k)) {
+        for (int64_t done = 0; !e;) {
+            const int64_t now = std::min<int64_t>(k - done, 1 << 30);
+            done += now;
+            e = launch_solo_steps(c->solo, c->I, c->S, c->D, (int)now, final_eval && done == k, c->stream);
+            if (done == k) break;
+        }
         return e;
     }
-    return (flags & MSAT_STEP_GRAPH) ? graph_steps(c, k) : plain_steps(c, k);
+    e = !c->prof_on && (flags & MSAT_STEP_GRAPH) ? graph_steps(c, k) : plain_steps(c, k);
+    if (!e && final_eval) e = eval_current(c);
+    return e;
 }
 
 extern "C" int msat_step_ex(msat_ctx *c, int32_t n_steps, uint32_t flags, float *loss_out,
@@ -536,8 +587,7 @@ extern "C" int msat_step_ex(msat_ctx *c, int32_t n_steps, uint32_t flags, float 
     if (flags & ~(MSAT_STEP_NO_FINAL_EVAL | MSAT_STEP_GRAPH | MSAT_STEP_PER_PASS))
         return fail(MSAT_EINVAL, "msat_step: unknown flags");
     NvtxRange nv("msat_step");
-    cudaError_t e = run_steps(c, n_steps, flags);
-    if (!e && !(flags & MSAT_STEP_NO_FINAL_EVAL)) e = eval_current(c);
+    const cudaError_t e = run_steps(c, n_steps, flags, !(flags & MSAT_STEP_NO_FINAL_EVAL));
     if (e) return cuda_fail(e, "msat_step: kernel launch");
     c->steps_done_host += n_steps;
     if (loss_out)
@@ -588,7 +638,7 @@ extern "C" int msat_solve(msat_ctx *c, int64_t max_steps, double time_limit_s, i
     for (;;) {
         const int64_t k = std::min<int64_t>(chunk, max_steps - done);
         cudaError_t e = cudaSuccess;
-        if (k > 0) e = run_steps(c, k, MSAT_STEP_GRAPH);
+        if (k > 0) e = run_steps(c, k, MSAT_STEP_GRAPH, false);
         done += k;
         long long bmin = 0;
         if (!e) e = read_best(&bmin);
@@ -598,7 +648,7 @@ extern "C" int msat_solve(msat_ctx *c, int64_t max_steps, double time_limit_s, i
     }
     // the final x is evaluated once, as msat_step does
     long long bmin = 0;
-    cudaError_t e = eval_current(c);
+    cudaError_t e = run_steps(c, 0, 0u, true);
     if (!e) e = read_best(&bmin);
     if (e) return cuda_fail(e, "msat_solve: final evaluation");
     trace(bmin);
@@ -866,7 +916,7 @@ extern "C" int msat_get_info(msat_ctx *c, msat_info *info) {
     info->max_degree = c->max_deg;
     info->n_heavy = c->I.n_heavy;
     info->uniform_len = c->kfix;
-    info->small_kernel = small_fits(c->I, c->max_deg) ? 1 : 0;
+    info->small_kernel = c->solo.lists ? 1 : 0;
     return MSAT_OK;
 }
 

@@ -27,6 +27,7 @@ struct msat_ctx {
     msat::DevInst I{};
     msat::DevState S{};
     msat::DevStep D{};
+    msat::SoloDev solo{};  // lists of the one-block-per-restart kernel (small instances)
 
     // probe (autograd) path, allocated on first use
     bool probe_ready = false;

@@ -7,6 +7,8 @@
 #include <memory>
 #include <vector>
 
+#include "msat_internal.cuh"
+
 namespace msat {
 
 // An int32 array that is not zero-filled when sized (its filler threads
@@ -75,5 +77,17 @@ int build_block_rows(int32_t n, int64_t m, int32_t kfix, const I32Buf &coff, con
 // (clause, position) order): words row << 1 | neg, with row = row[j] of
 // clause j when `row` is given (the grouped store), else j.
 void scatter_occurrences(int32_t n, int64_t m, HostCnf &hc, const I32Buf *row);
+
+// Lists of the one-block-per-restart step kernel (k_solo.cu) of a canonical
+// CNF; false where the instance does not fit one SM's shared memory.  dev
+// holds the sizes and offsets (its pointers are set after the upload).
+struct SoloHost {
+    SoloDev dev;
+    std::vector<unsigned char> lists;
+    std::vector<int32_t> perm;  // internal variable order -> variable
+    std::vector<int32_t> slot;  // clause -> slot, empty: clause order
+};
+bool build_solo(int32_t n, int64_t m, int32_t kfix, int32_t max_len, int32_t max_deg, const HostCnf &hc,
+                SoloHost &out);
 
 }  // namespace msat

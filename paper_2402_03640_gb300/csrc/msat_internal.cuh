@@ -102,6 +102,26 @@ struct DevState {
                            // nullptr: the variable pass recomputes f from the unsat bits
 };
 
+// Lists of the one-block-per-restart step kernel (k_solo.cu): 16-bit literal
+// and occurrence words in 32-lane slices and their tables, in one array.
+struct SoloDev {
+    const unsigned char *lists = nullptr;  // nullptr: the instance does not fit one SM
+    uint32_t list_bytes = 0;
+    uint32_t off_lit = 0, off_occ = 0;            // rows of 32 lanes x four words
+    uint32_t off_lit_base = 0, off_occ_base = 0;  // first row of each slice
+    uint32_t off_sgn = 0;                         // sign bits of each leaf task
+    uint32_t off_mbeg = 0;                        // first leaf task of each variable of several leaves
+    const int *perm = nullptr;                    // internal variable order -> variable
+    const int64_t *w = nullptr;                   // clause weights in slot order, or all 1
+    int n_single = 0;  // variables of at most one leaf (the first of the internal order)
+    int n_multi = 0;   // variables of several leaves
+    int n_wide = 0;    // of these, the ones a warp combines (first)
+    int n_mtask = 0;   // leaf tasks of the variables of several leaves
+    int kind = 0;      // 0: every clause has 3 literals, 1: at most 32, 2: any length
+    bool pairs = false;          // w*f held as {q, -q}
+    int sms = 1;                 // multiprocessors of the device
+};
+
 // Dense tensor-core evaluation (k_dense.cu): clause matrix W^T
 // [m_pad][n_pad] in packed e2m1 (n_pad / 2 bytes a row), per-row target
 // -len_j (NaN: never unsat), 32-bit weights, the packed e2m1 assignment
@@ -286,15 +306,12 @@ cudaError_t launch_step_batch(const SlotDesc *slots, int nslot, const int *fwd_s
 int heavy_blocks_of(const DevInst &I);
 int light_blocks_of(const DevInst &I);
 cudaError_t launch_loss_reduce(const DevStep &D, int B, cudaStream_t st);
-// Small instances: every step in one single-CTA launch with the state in
-// shared memory (same bits as the per-pass kernels).
-constexpr int kSmallThreads = 1024;
-constexpr int kSmallMaxB = 64;
-constexpr size_t kSmallSmemMax = 200 * 1024;
-size_t small_smem_bytes(const DevInst &I);
-bool small_fits(const DevInst &I, int max_deg);
-cudaError_t launch_small_steps(const DevInst &I, const DevState &S, const DevStep &D, int n_steps,
-                               cudaStream_t st);
+// Small instances: one block per restart takes every step of a call (and, if
+// asked, the evaluation of the final x) with the restart's state in shared
+// memory (k_solo.cu; same bits as the per-pass kernels).
+cudaError_t launch_solo_steps(const SoloDev &V, const DevInst &I, const DevState &S, const DevStep &D,
+                              int n_steps, bool final_eval, cudaStream_t st);
+bool solo_pays(const SoloDev &V, const DevInst &I, int64_t nnz, int max_len, int64_t steps);
 cudaError_t launch_eval_sparse(const DevInst &I, const int8_t *a, int nb, long long *cost,
                                cudaStream_t st);
 cudaError_t launch_round_pm1(const float *x, int8_t *a, long long count, cudaStream_t st);

@@ -15,8 +15,8 @@
 // its best costs and assignment are copied to pinned host memory behind an
 // event, and its memory is released in stream order once the copy has
 // landed; the freed budget admits queued requests.
-// An instance small enough for the single-CTA kernel (state in shared
-// memory) skips the slot table: it takes all its steps in one launch on one
+// An instance small enough for the one-block-per-restart kernel (state in
+// shared memory) skips the slot table: it takes all its steps in one launch on one
 // of several side streams as soon as it is built and retires the same
 // way, so it is not held back by the large instances of the batch.
 //
@@ -80,6 +80,7 @@ struct SrvBuilt {
 struct SrvFinishing {
     SrvSlot slot;
     cudaEvent_t ev = nullptr;
+    bool direct = false;        // a small instance, running until the event
     int64_t *h_best = nullptr;  // pinned [B]
     uint8_t *h_bits = nullptr;  // pinned [n][B]
     int64_t *h_bstep = nullptr; // pinned [B]
@@ -198,14 +199,15 @@ void finish_failed(msat_server *S, uint64_t ticket, int code, Clock::time_point 
     S->cv_done.notify_all();
 }
 
-// Evaluate a finished instance once more and copy its best costs and
+// Evaluate a finished instance once more (unless its last launch did) and copy its best costs and
 // assignment to pinned host memory behind an event, all on the instance's
 // stream; reap() collects it when the event has completed.
-cudaError_t start_retire(msat_server *S, const SrvSlot &sl) {
+cudaError_t start_retire(msat_server *S, const SrvSlot &sl, bool evaluated) {
     msat_ctx *c = sl.ctx;
     SrvFinishing fin;
     fin.slot = sl;
-    cudaError_t e = ctx_eval_current(c);
+    fin.direct = evaluated;
+    cudaError_t e = evaluated ? cudaSuccess : ctx_eval_current(c);
     if (!e) e = pinned_get(S, sizeof(int64_t) * (size_t)c->B, (void **)&fin.h_best, &fin.cap_best);
     if (!e) e = pinned_get(S, (size_t)c->n * c->B, (void **)&fin.h_bits, &fin.cap_bits);
     if (!e) e = pinned_get(S, sizeof(int64_t) * (size_t)c->B, (void **)&fin.h_bstep, &fin.cap_bstep);
@@ -287,13 +289,14 @@ void place(msat_server *S, SrvBuilt &b) {
     sl.t_admit = b.t_admit;
     sl.bytes = (size_t)c->device_bytes;
     S->in_use += sl.bytes;
-    if (small_fits(c->I, c->max_deg)) {
-        // a small instance takes all its steps in one single-CTA launch on a
-        // side stream (same bits as the batched kernels), then retires
+    if (c->solo.lists) {
+        // a small instance takes all its steps and its final evaluation in
+        // one launch (a block per restart) on a side stream, with the same
+        // bits as the batched kernels, then retires
         c->stream = S->small_st[S->small_next];
         S->small_next = (S->small_next + 1) % msat_server::kSmallStreams;
-        cudaError_t e = launch_small_steps(c->I, c->S, c->D, req.steps, c->stream);
-        if (!e) e = start_retire(S, sl);
+        cudaError_t e = launch_solo_steps(c->solo, c->I, c->S, c->D, req.steps, true, c->stream);
+        if (!e) e = start_retire(S, sl, true);
         if (e) {
             cuda_fail(e, "msat server: small instance");
             finish_failed(S, req.ticket, MSAT_ECUDA, req.t_submit);
@@ -401,7 +404,7 @@ int run_round_body(msat_server *S) {
             keep.push_back(sl);
             continue;
         }
-        const cudaError_t e = start_retire(S, sl);
+        const cudaError_t e = start_retire(S, sl, false);
         if (e) return cuda_fail(e, "msat server: result copy");
         S->work -= sl.work;
         S->dirty = true;
@@ -522,7 +525,9 @@ void worker_main(msat_server *S) {
         got.clear();
         {
             std::lock_guard<std::mutex> lk(S->mu);
+            // the slot table's instances and those running on the side streams
             S->st.running = (int32_t)S->slots.size();
+            for (const SrvFinishing &f : S->finishing) S->st.running += f.direct ? 1 : 0;
             S->st.peak_running = std::max(S->st.peak_running, S->st.running);
             S->st.queued = (int32_t)S->queue.size();
             S->st.hbm_in_use = (int64_t)S->in_use;

@@ -1,0 +1,86 @@
+"""The one-block-per-restart kernel at the edges of its slices, list layouts
+and sums: bit-exact trajectories against the FP32-mode oracle, continued on
+the per-pass kernels."""
+import numpy as np
+import pytest
+
+from synth import Cnf, uniform_ksat, zipf_weighted
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def pkg():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    import paper_2402_03640_gb300 as p
+    from paper_2402_03640_gb300 import build
+    build.build()
+    p.load()
+    return p
+
+
+def _mixed(seed, n, m, lo, hi, w_max=0):
+    """Clauses of lo..hi literals (repeats and x-or-not-x clauses among them)."""
+    rng = np.random.default_rng(seed)
+    cl = [((rng.integers(0, n, size=k) + 1) * rng.choice([-1, 1], size=k)).tolist()
+          for k in rng.integers(lo, hi + 1, size=m)]
+    w = rng.integers(1, w_max, size=m) if w_max else None
+    return Cnf.from_clauses(n, cl, weights=w)
+
+
+CASES = {
+    "one_clause": lambda: (uniform_ksat(3, 1, 3, seed=1), 1),
+    "slice_less_one": lambda: (uniform_ksat(31, 31, 3, seed=2), 2),
+    "slice_full": lambda: (uniform_ksat(32, 32, 3, seed=3), 2),
+    "slice_plus_one": lambda: (uniform_ksat(33, 33, 3, seed=4), 4),
+    "two_blocks_an_sm": lambda: (uniform_ksat(301, 1290, 3, seed=5), 256),
+    "lists_in_l2": lambda: (uniform_ksat(2500, 10750, 3, seed=6), 2),
+    "signs_apart": lambda: (uniform_ksat(5000, 21500, 3, seed=7), 1),
+    "k5": lambda: (uniform_ksat(97, 2067, 5, seed=8), 4),
+    "mixed": lambda: (_mixed(9, 61, 500, 0, 9), 2),
+    "units_64bit_weights": lambda: (_mixed(10, 40, 300, 1, 4, w_max=1 << 40), 2),
+    "long_weighted": lambda: (_mixed(11, 300, 400, 20, 90, w_max=50), 2),
+    "many_leaves": lambda: (uniform_ksat(12, 9000, 3, seed=12), 1),
+    "skewed": lambda: (zipf_weighted(900, 4100, seed=13), 4),
+}
+
+
+@pytest.mark.parametrize("name", sorted(CASES))
+def test_solo_kernel_matches_oracle(pkg, oracle, name):
+    cnf, B = CASES[name]()
+    S, lr = 40, 2e-2
+    ref = oracle.solve(cnf, B, 1, S + 3, mode=oracle.MODE_F32, lr=lr)
+    with pkg.Solver.from_cnf(cnf, restarts=B, lr=lr) as s:
+        assert s.info()["small_kernel"] == 1
+        # 33 steps cross a chunk of the Adam scalars; the cost after each call
+        # is that of the final x
+        _, c0 = s.step(0, want_loss=False)
+        _, c1 = s.step(33, want_loss=False)
+        _, c2 = s.step(7, want_loss=False)
+        _, c3 = s.step(3, want_loss=False, per_pass=True)
+        x = s.x()
+        assign, best = s.best()
+        assert s.info()["steps_done"] == S + 3
+    assert np.array_equal(np.stack([c0, c1, c2, c3]), ref["cost_hist"][[0, 33, 40, 43]])
+    assert np.array_equal(x.astype(np.float64), ref["x_final"])
+    assert np.array_equal(best, ref["best_cost"]) and np.array_equal(assign, ref["best_assign"])
+
+
+def test_solo_kernel_keeps_nan_in_its_restart(pkg):
+    """A NaN in one restart's x stays in that variable: its clauses add
+    nothing, as on the per-pass kernels."""
+    cnf = uniform_ksat(60, 240, 3, seed=14)
+    out = []
+    for per_pass in (False, True):
+        with pkg.Solver.from_cnf(cnf, restarts=2, lr=1e-2) as s:
+            st = s.get_state()
+            st["x"][7, 0] = np.nan
+            st["x"][9, 1] = 0.0
+            st["x"][11, 1] = -0.0
+            s.set_state(st)
+            _, cost = s.step(20, want_loss=False, per_pass=per_pass)
+            out.append((cost, s.x(), s.best()[1]))
+    for a, b in zip(*out):
+        assert np.array_equal(a, b, equal_nan=True)
