@@ -98,6 +98,9 @@ static void free_all(msat_ctx *c) {
         if (c->pool_alloc) cudaFreeAsync(p, c->stream); else cudaFree(p);
     }
     c->allocs.clear();
+    if (c->ebits) cudaFree(c->ebits);
+    c->ebits = nullptr;
+    c->ebits_bytes = 0;
     if (c->dense.Xt) cudaFree(c->dense.Xt);
     c->dense.Xt = nullptr;
     c->dense.xt_bytes = 0;
@@ -313,6 +316,7 @@ int msat::ctx_create(msat_ctx **out, int32_t n_vars, int64_t n_clauses, const in
     c->clen = std::move(hc.clen);
     c->taut = std::move(hc.taut);
     if (weights) c->wts.assign(weights, weights + m);
+    while (hc.wor >> c->wbits) ++c->wbits;
 
     const int64_t nB = (int64_t)n_vars * B;
     int rc = MSAT_OK;
@@ -746,18 +750,69 @@ extern "C" int msat_check(msat_ctx *c) {
 
 static int dense_eval(msat_ctx *c, const int8_t *a, const float *x, int32_t nb, int64_t *cost_out);
 
+// Clause-list evaluation of a batch given as int8 +-1 (a) or as relaxed x
+// read through its rounding.  The packed batch lies in a buffer kept with the
+// context, at most 256 MiB (a larger batch goes through it in parts) or, where
+// that cannot be had, 128 assignments' worth.  A call captured into a graph
+// takes it from the stream-ordered pool instead, allocated and freed by the
+// graph: the graph may outlive the context's buffer.
+static int sparse_eval(msat_ctx *c, const int8_t *a, const float *x, int32_t nb, int64_t *cost_out) {
+    if (eval_is_direct(c->nnz, nb)) {
+        prof_begin(c, PROF_EVAL);
+        const cudaError_t e = launch_eval_sparse(c->I, a, x, nb, nb, c->wbits, nullptr, (long long *)cost_out, c->stream);
+        prof_end(c);
+        return e ? cuda_fail(e, "msat_evaluate: sparse kernel") : MSAT_OK;
+    }
+    constexpr int kGroup = 128;
+    const int64_t groups = (256LL << 20) / (int64_t)eval_sparse_bytes(c->n, kGroup);
+    int chunk = (int)std::min<int64_t>(nb, std::max<int64_t>(1, groups) * kGroup);
+    size_t need = eval_sparse_bytes(c->n, chunk);
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(c->stream, &cap) != cudaSuccess) cudaGetLastError();
+    const bool own = cap != cudaStreamCaptureStatusNone;
+    uint32_t *bits = c->ebits;
+    cudaError_t e = cudaSuccess;
+    if (own) {
+        e = cudaMallocAsync(&bits, need, c->stream);
+    } else if (need > c->ebits_bytes) {
+        if (c->ebits) {
+            cudaStreamSynchronize(c->stream);
+            cudaFree(c->ebits);
+            c->ebits = nullptr;
+            c->ebits_bytes = 0;
+        }
+        e = cudaMalloc(&c->ebits, need);
+        if (e && chunk > kGroup) {
+            cudaGetLastError();
+            chunk = kGroup;
+            need = eval_sparse_bytes(c->n, chunk);
+            e = cudaMalloc(&c->ebits, need);
+        }
+        if (!e) c->ebits_bytes = need;
+        else c->ebits = nullptr;
+        bits = c->ebits;
+    }
+    if (e) {
+        cudaGetLastError();
+        return fail(MSAT_ENOMEM, "msat_evaluate: packed assignment buffer allocation failed");
+    }
+    prof_begin(c, PROF_EVAL);
+    e = launch_eval_sparse(c->I, a, x, nb, chunk, c->wbits, bits, (long long *)cost_out, c->stream);
+    prof_end(c);
+    if (own) {
+        const cudaError_t f = cudaFreeAsync(bits, c->stream);
+        if (!e) e = f;
+    }
+    if (e) return cuda_fail(e, "msat_evaluate: sparse kernel");
+    return MSAT_OK;
+}
+
 extern "C" int msat_evaluate(msat_ctx *c, const int8_t *assign_pm1, int32_t nb, int64_t *cost_out,
                              int32_t backend) {
     if (!c) return fail(MSAT_EINVAL, "msat_evaluate: ctx is NULL");
     if (nb < 1 || !assign_pm1 || !cost_out)
         return fail(MSAT_EINVAL, "msat_evaluate: need nb >= 1 and non-NULL buffers");
-    if (backend == MSAT_BACKEND_SPARSE) {
-        prof_begin(c, PROF_EVAL);
-        cudaError_t e = launch_eval_sparse(c->I, assign_pm1, nb, (long long *)cost_out, c->stream);
-        prof_end(c);
-        if (e) return cuda_fail(e, "msat_evaluate: sparse kernel");
-        return MSAT_OK;
-    }
+    if (backend == MSAT_BACKEND_SPARSE) return sparse_eval(c, assign_pm1, nullptr, nb, cost_out);
     if (backend == MSAT_BACKEND_DENSE) return dense_eval(c, assign_pm1, nullptr, nb, cost_out);
     return fail(MSAT_EINVAL, "msat_evaluate: unknown backend");
 }
@@ -845,16 +900,8 @@ extern "C" int msat_evaluate_x(msat_ctx *c, int32_t backend, int64_t *cost_out) 
     if (!c || !cost_out) return fail(MSAT_EINVAL, "msat_evaluate_x: NULL argument");
     // the tensor-core operand is built from x directly (rounding and transposition in one kernel)
     if (backend == MSAT_BACKEND_DENSE) return dense_eval(c, nullptr, c->S.x, c->B, cost_out);
-    const long long nB = (long long)c->n * c->B;
-    if (!c->xpm1) {
-        int rc = dalloc_t(c, &c->xpm1, (size_t)nB);
-        if (rc) return rc;
-    }
-    prof_begin(c, PROF_OTHER);
-    cudaError_t e = launch_round_pm1(c->S.x, c->xpm1, nB, c->stream);
-    prof_end(c);
-    if (e) return cuda_fail(e, "msat_evaluate_x: rounding kernel");
-    return msat_evaluate(c, c->xpm1, c->B, cost_out, backend);
+    if (backend == MSAT_BACKEND_SPARSE) return sparse_eval(c, nullptr, c->S.x, c->B, cost_out);
+    return fail(MSAT_EINVAL, "msat_evaluate_x: unknown backend");
 }
 
 extern "C" int msat_heuristic_gap(msat_ctx *c, int64_t *heur_unsat, int64_t *disagree) {

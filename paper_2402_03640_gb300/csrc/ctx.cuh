@@ -40,7 +40,11 @@ struct msat_ctx {
     std::vector<int64_t> wts;     // clause weights (empty: all 1)
     bool dense_ready = false;
     msat::DenseDev dense;
-    int8_t *xpm1 = nullptr;       // rounded x as a +-1 batch, allocated on first use
+    // sparse evaluation: the packed batch (grown on use) and the bits of the
+    // largest clause weight (0: all 1)
+    uint32_t *ebits = nullptr;
+    size_t ebits_bytes = 0;
+    int wbits = 0;
     long long *hgap = nullptr;    // [2][B] counts of msat_heuristic_gap, allocated on first use
 
     // CUDA graphs of 1 and kGraphSteps steps (MSAT_STEP_GRAPH), captured on first use

@@ -108,7 +108,7 @@ int build_host_cnf(int32_t n, int64_t m, const int64_t *off, const int32_t *lits
     // variables in the thread's own arrays (marked with the clause index).
     struct Part {
         std::vector<int32_t> lit;
-        int64_t wsum = 0;
+        int64_t wsum = 0, wor = 0;
         int32_t max_len = 0;
         int32_t first_len = -1;  // length of the part's first clause
         bool same_len = true;    // every clause of the part has first_len literals
@@ -159,6 +159,7 @@ int build_host_cnf(int32_t n, int64_t m, const int64_t *off, const int32_t *lits
             out.clen[(size_t)j] = len;
             out.taut[(size_t)j] = taut ? 1 : 0;
             P.wsum += w ? w[j] : 1;
+            if (w) P.wor |= w[j];
         }
     });
     for (const Part &P : parts)
@@ -173,6 +174,7 @@ int build_host_cnf(int32_t n, int64_t m, const int64_t *off, const int32_t *lits
     for (int t = 0; t < Tm; ++t) {
         lbase[(size_t)t + 1] = lbase[(size_t)t] + (int64_t)parts[(size_t)t].lit.size();
         out.wsum += parts[(size_t)t].wsum;
+        out.wor |= parts[(size_t)t].wor;
         out.max_len = std::max(out.max_len, parts[(size_t)t].max_len);
     }
     out.nnz = lbase[(size_t)Tm];

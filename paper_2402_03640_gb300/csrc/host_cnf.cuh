@@ -41,6 +41,7 @@ struct HostCnf {
     std::vector<uint8_t> taut;  // [m] clause holds some x and not x
     int64_t nnz = 0;
     int64_t wsum = 0;           // total clause weight
+    int64_t wor = 0;            // or of the caller's weights (0: all 1)
     int32_t max_len = 0, max_deg = 0;
     int32_t kfix = 0;           // common clause length, or 0
     // between build_host_cnf and scatter_occurrences: thread t's first

@@ -1,49 +1,220 @@
-// Exact cost of a batch of +-1 assignments by the clause CSR (sm_103a).
+// Exact cost of a batch of assignments by the clause CSR (sm_103a).
 //
 // A clause is unsatisfied iff none of its literals is true (the paper's
 // test x'.W == -len with x' read as +-1, Sec. 4 "Unsatisfiable Cores").
-// Layout: a[i * nb + b] is variable i of assignment b, so the 32 lanes of a
-// warp read 32 consecutive assignments of one variable (one 32-byte sector).
-// Each warp walks clauses with a stride; per-lane integer sums are combined
-// across the block's warps in shared memory and added to cost[b] with one
-// 64-bit atomic per (block, assignment) -- integer addition, so the result
-// does not depend on the order.
+// Kernels:
+//
+//   k_pack_bits    the batch a[n][nb] (one byte or float an entry, true
+//                  where > 0) to one bit an entry, 32 assignments a word
+//   k_eval_sparse  a lane owns one clause for VW words of 32 assignments:
+//                  per literal one gather of VW words, an exclusive or with
+//                  the sign and an or; the unsat words of a warp's 32
+//                  clauses are transposed, so that lane b counts the unsat
+//                  clauses of assignment b with one popcount (per bit of
+//                  the weights where there are weights)
+//   k_eval_direct  small calls, one assignment a lane, without the packing
+//
+// What bounds it: the gathers, one 4 VW-byte read per literal, VW = 4 where
+// the batch has more than 64 assignments (a 16-byte row holds 128 of them).
+// The form before it gave each lane one assignment and read 32 bytes of a
+// per literal and 32 assignments, about 42 instructions for 32 (clause,
+// assignment) pairs where this one takes about 150 for 4096.  Weighted Zipf
+// n=2e5, m=1e6, 100 assignments: 695 -> 53
+// us a call (14 packing, 36 evaluation, the rest launches).
 
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <algorithm>
+
+#include "bits.cuh"
 #include "msat_internal.cuh"
 
 namespace msat {
 
 namespace {
+
 constexpr int kEvalWarps = kThreads / 32;
+constexpr int kLitBatch = 4;  // literals whose loads and gathers are in flight together
+
+// What the evaluation reads of an instance (a launch copies its arguments).
+struct EvalInst {
+    int m, kfix;
+    const int32_t *coff, *lit;
+    const int64_t *w;
+};
+
+__device__ __forceinline__ bool is_true(int8_t v) { return v > 0; }
+__device__ __forceinline__ bool is_true(float v) { return v > 0.0f; }
+
+// VW consecutive words of one row.
+template <int VW>
+__device__ __forceinline__ void ld_words(const uint32_t *__restrict__ p, uint32_t (&o)[VW]) {
+    if constexpr (VW == 4) {
+        const uint4 v = __ldg(reinterpret_cast<const uint4 *>(p));
+        o[0] = v.x;
+        o[1] = v.y;
+        o[2] = v.z;
+        o[3] = v.w;
+    } else if constexpr (VW == 2) {
+        const uint2 v = __ldg(reinterpret_cast<const uint2 *>(p));
+        o[0] = v.x;
+        o[1] = v.y;
+    } else {
+        o[0] = __ldg(p);
+    }
 }
 
+}  // namespace
+
+// One warp packs rows: RW words of 32 entries of a row an iteration, RPI =
+// 4 / RW rows at a time.  row: entries of a row of the source, of which the
+// first nb are packed; wpr: words per row of the result, a multiple of RW
+// (words past the batch are zero).  V4 (int8 rows and batch of multiples of
+// four bytes): a lane reads four entries at a time, their bits meet by
+// shuffles of eight lanes; otherwise a lane reads one entry and a ballot
+// makes the word.  Clears the costs the evaluation adds to.
+// 2e5 rows of 100 bytes: 14 us (51 with one byte a lane and a division per word).
+template <typename T, int RW, bool V4>
 __global__ void __launch_bounds__(kThreads)
-    k_eval_sparse(DevInst I, const int8_t *__restrict__ a, int nb,
+    k_pack_bits(const T *__restrict__ a, int n, int row, int nb, int wpr, uint32_t *__restrict__ bits,
+                unsigned long long *__restrict__ cost) {
+    constexpr int RPI = 4 / RW;
+    const int lane = threadIdx.x & 31;
+    if (blockIdx.x == 0)
+        for (int b = threadIdx.x; b < nb; b += kThreads) cost[b] = 0ull;
+    const long long stride = (long long)gridDim.x * kEvalWarps * RPI;
+    for (long long i0 = ((long long)blockIdx.x * kEvalWarps + (threadIdx.x >> 5)) * RPI; i0 < n; i0 += stride) {
+        for (int w0 = 0; w0 < wpr; w0 += RW) {
+            if constexpr (V4) {
+                // RW words are 8 RW lanes of four entries: the rows of the
+                // iteration side by side in the warp's lanes
+                const int r = lane / (8 * RW), c = w0 * 32 + (lane % (8 * RW)) * 4;
+                uint32_t x = 0u;
+                if (i0 + r < n && c < nb) x = __ldg(reinterpret_cast<const uint32_t *>(a + (i0 + r) * row + c));
+                // bit 7 of each byte where it is > 0, then the four bits together
+                const uint32_t pos = ((x & 0x7f7f7f7fu) + 0x7f7f7f7fu) & ~x & 0x80808080u;
+                uint32_t word = ((((pos >> 7) * 0x01020408u) >> 24) & 0xfu) << (4 * (lane & 7));
+#pragma unroll
+                for (int o = 1; o < 8; o <<= 1) word |= __shfl_xor_sync(0xffffffffu, word, o);
+                if ((lane & 7) == 0 && i0 + r < n) bits[(i0 + r) * wpr + w0 + (lane % (8 * RW)) / 8] = word;
+            } else {
+                T v[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    const int c = (w0 + u % RW) * 32 + lane;
+                    v[u] = i0 + u / RW < n && c < nb ? __ldg(a + (i0 + u / RW) * row + c) : T(0);
+                }
+                uint32_t mine = 0u;
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    const uint32_t word = __ballot_sync(0xffffffffu, is_true(v[u]));
+                    if (lane == u) mine = word;
+                }
+                if (lane < 4 && i0 + lane / RW < n) bits[(i0 + lane / RW) * wpr + w0 + lane % RW] = mine;
+            }
+        }
+    }
+}
+
+// wbits: bits of the largest clause weight (0: every weight is 1).
+template <int VW>
+__global__ void __launch_bounds__(kThreads)
+    k_eval_sparse(EvalInst I, const uint32_t *__restrict__ bits, int wpr, int nb, int wbits,
                   unsigned long long *__restrict__ cost) {
+    __shared__ unsigned long long s_acc[kEvalWarps][32 * VW];
+    const int lane = threadIdx.x & 31;
+    const int warp = threadIdx.x >> 5;
+    const int word0 = blockIdx.y * VW;
+    unsigned long long acc[VW];
+#pragma unroll
+    for (int v = 0; v < VW; ++v) acc[v] = 0;
+    for (long long j0 = ((long long)blockIdx.x * kEvalWarps + warp) * 32; j0 < I.m;
+         j0 += (long long)gridDim.x * kEvalWarps * 32) {
+        const long long j = j0 + lane;
+        const bool live = j < I.m;
+        int beg = 0, end = 0;
+        if (live) {
+            if (I.kfix > 0) {
+                beg = (int)j * I.kfix;
+                end = beg + I.kfix;
+            } else {
+                beg = __ldg(I.coff + j);
+                end = __ldg(I.coff + j + 1);
+            }
+        }
+        uint32_t sat[VW];
+#pragma unroll
+        for (int v = 0; v < VW; ++v) sat[v] = live ? 0u : 0xffffffffu;
+        for (int p0 = beg; p0 < end; p0 += kLitBatch) {
+            int L[kLitBatch];
+            uint32_t row[kLitBatch][VW];
+#pragma unroll
+            for (int k = 0; k < kLitBatch; ++k) L[k] = p0 + k < end ? __ldg(I.lit + p0 + k) : -1;
+#pragma unroll
+            for (int k = 0; k < kLitBatch; ++k)
+                if (L[k] >= 0) ld_words<VW>(bits + (long long)(L[k] >> 1) * wpr + word0, row[k]);
+#pragma unroll
+            for (int k = 0; k < kLitBatch; ++k) {
+                if (L[k] < 0) continue;
+                const uint32_t neg = (L[k] & 1) ? 0xffffffffu : 0u;
+#pragma unroll
+                for (int v = 0; v < VW; ++v) sat[v] |= row[k][v] ^ neg;
+            }
+        }
+        __syncwarp();
+        uint32_t un[VW];  // lane b: the unsat bits of the warp's 32 clauses under assignment b
+#pragma unroll
+        for (int v = 0; v < VW; ++v) un[v] = transpose_bits32(~sat[v], lane);
+        if (wbits == 0) {
+#pragma unroll
+            for (int v = 0; v < VW; ++v) acc[v] += (unsigned)__popc(un[v]);
+        } else {
+            const unsigned long long w = live ? (unsigned long long)__ldg(I.w + j) : 0ull;
+            for (int p = 0; p < min(wbits, 32); ++p) {
+                const uint32_t plane = __ballot_sync(0xffffffffu, ((uint32_t)w >> p) & 1u);
+#pragma unroll
+                for (int v = 0; v < VW; ++v) acc[v] += (unsigned long long)__popc(un[v] & plane) * (1u << p);
+            }
+            for (int p = 32; p < wbits; ++p) {
+                const uint32_t plane = __ballot_sync(0xffffffffu, (w >> p) & 1ull);
+#pragma unroll
+                for (int v = 0; v < VW; ++v) acc[v] += (unsigned long long)__popc(un[v] & plane) << p;
+            }
+        }
+    }
+#pragma unroll
+    for (int v = 0; v < VW; ++v) s_acc[warp][32 * v + lane] = acc[v];
+    __syncthreads();
+    for (int b = threadIdx.x; b < 32 * VW; b += kThreads) {
+        unsigned long long s = 0;
+#pragma unroll
+        for (int k = 0; k < kEvalWarps; ++k) s += s_acc[k][b];
+        const int at = word0 * 32 + b;
+        if (at < nb && s) atomicAdd(cost + at, s);
+    }
+}
+
+// Small batches of small instances, in one launch without scratch: a lane is
+// one assignment and a warp walks clauses, reading 32 entries of a variable's
+// row per literal.
+template <typename T>
+__global__ void __launch_bounds__(kThreads)
+    k_eval_direct(EvalInst I, const T *__restrict__ a, int nb, unsigned long long *__restrict__ cost) {
     __shared__ unsigned long long s_acc[kEvalWarps][32];
     const int lane = threadIdx.x & 31;
     const int warp = threadIdx.x >> 5;
     const int b = blockIdx.y * 32 + lane;
     const bool live = b < nb;
     unsigned long long acc = 0;
-    for (long long j = (long long)blockIdx.x * kEvalWarps + warp; j < I.m;
-         j += (long long)gridDim.x * kEvalWarps) {
-        int beg, end;
-        if (I.kfix > 0) {
-            beg = (int)j * I.kfix;
-            end = beg + I.kfix;
-        } else {
-            beg = __ldg(I.coff + j);
-            end = __ldg(I.coff + j + 1);
-        }
+    for (long long j = (long long)blockIdx.x * kEvalWarps + warp; j < I.m; j += (long long)gridDim.x * kEvalWarps) {
+        const int beg = I.kfix > 0 ? (int)j * I.kfix : __ldg(I.coff + j);
+        const int end = I.kfix > 0 ? beg + I.kfix : __ldg(I.coff + j + 1);
         bool sat = false;
         for (int p = beg; p < end; ++p) {
             const int L = __ldg(I.lit + p);
-            const int8_t v = live ? __ldg(a + (long long)(L >> 1) * nb + b) : 0;
-            sat |= ((v > 0) != (bool)(L & 1));
+            const T v = live ? __ldg(a + (long long)(L >> 1) * nb + b) : T(0);
+            sat |= is_true(v) != (bool)(L & 1);
         }
         if (!sat) acc += I.w ? (unsigned long long)__ldg(I.w + j) : 1ull;
     }
@@ -57,27 +228,77 @@ __global__ void __launch_bounds__(kThreads)
     }
 }
 
-cudaError_t launch_eval_sparse(const DevInst &I, const int8_t *a, int nb, long long *cost,
-                               cudaStream_t st) {
-    cudaError_t e = cudaMemsetAsync(cost, 0, sizeof(long long) * (size_t)nb, st);
-    if (e != cudaSuccess) return e;
-    if (I.m == 0) return cudaSuccess;
-    const int gy = (nb + 31) / 32;
-    long long gx = (I.m + kEvalWarps - 1) / kEvalWarps;
-    long long cap = (152LL * 8 + gy - 1) / gy;  // about 8 blocks per SM in total
-    if (gx > cap) gx = cap;
-    if (gx < 1) gx = 1;
-    dim3 grid((unsigned)gx, (unsigned)gy);
-    k_eval_sparse<<<grid, kThreads, 0, st>>>(I, a, nb, reinterpret_cast<unsigned long long *>(cost));
-    return cudaGetLastError();
+// Up to this many literal evaluations the direct kernel: below it a call is
+// bound by its launches on the host, where a clear and one kernel (5.2 us)
+// beat two kernels (8.2 us); 3-SAT m=21500 with 64 assignments, 4.1 million,
+// takes 12.3 us directly and 11.7 packed.
+constexpr long long kDirectEvals = 1 << 20;
+
+bool eval_is_direct(int64_t nnz, int nb) { return nnz * nb <= kDirectEvals; }
+
+// Words a lane carries: rows of up to 128 assignments are one load.
+static int eval_vw(int nb) { return nb > 64 ? 4 : nb > 32 ? 2 : 1; }
+
+static int eval_wpr(int nb) {
+    const int vw = eval_vw(nb);
+    return ((nb + 31) / 32 + vw - 1) / vw * vw;
 }
 
-// Rounded batch of the relaxed variables: a[q] = +1 if x[q] > 0 else -1
-// (the de-relaxation of Sec. 4, read as +-1), same [n][B] layout.
-__global__ void k_round_pm1(const float *__restrict__ x, int8_t *__restrict__ a, long long count) {
-    for (long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x; q < count;
-         q += (long long)gridDim.x * blockDim.x)
-        a[q] = __ldg(x + q) > 0.0f ? (int8_t)1 : (int8_t)-1;
+// Scratch of one pass over nb assignments.
+size_t eval_sparse_bytes(int n, int nb) { return sizeof(uint32_t) * (size_t)n * (size_t)eval_wpr(nb); }
+
+template <int VW>
+static void launch_eval_vw(const DevInst &I, const int8_t *a, const float *x, int row, int nb, int wbits,
+                           uint32_t *bits, unsigned long long *cost, cudaStream_t st) {
+    const int wpr = eval_wpr(nb);
+    const long long rows4 = ((long long)I.n * VW + 3) / 4;  // warp iterations of the packing
+    const unsigned pb = (unsigned)std::min<long long>((rows4 + kEvalWarps - 1) / kEvalWarps, 152LL * 8);
+    // four-byte reads: every row of the batch starts on four bytes
+    const bool v4 = a && row % 4 == 0 && nb % 4 == 0 && reinterpret_cast<uintptr_t>(a) % 4 == 0;
+    if (v4) k_pack_bits<int8_t, VW, true><<<pb, kThreads, 0, st>>>(a, I.n, row, nb, wpr, bits, cost);
+    else if (a) k_pack_bits<int8_t, VW, false><<<pb, kThreads, 0, st>>>(a, I.n, row, nb, wpr, bits, cost);
+    else k_pack_bits<float, VW, false><<<pb, kThreads, 0, st>>>(x, I.n, row, nb, wpr, bits, cost);
+    const int gy = wpr / VW;
+    // about eight blocks per SM in all, or fewer when the clauses do not fill them
+    const long long need = ((long long)I.m + kThreads - 1) / kThreads;
+    const long long gx = std::max<long long>(1, std::min<long long>(need, (152LL * 8 + gy - 1) / gy));
+    k_eval_sparse<VW><<<dim3((unsigned)gx, (unsigned)gy), kThreads, 0, st>>>(
+        EvalInst{I.m, I.kfix, I.coff, I.lit, I.w}, bits, wpr, nb, wbits, cost);
+}
+
+// The batch is a (int8 [n][nb]) or, where a is nullptr, x (float [n][nb],
+// rounded by x > 0), taken at most `chunk` assignments at a time; bits:
+// eval_sparse_bytes(n, min(nb, chunk)) of scratch, or nullptr for the direct
+// kernel.
+cudaError_t launch_eval_sparse(const DevInst &I, const int8_t *a, const float *x, int nb, int chunk, int wbits,
+                               uint32_t *bits, long long *cost_out, cudaStream_t st) {
+    cudaError_t e = cudaSuccess;
+    if (I.m == 0 || !bits) {
+        e = cudaMemsetAsync(cost_out, 0, sizeof(long long) * (size_t)nb, st);
+        if (e != cudaSuccess || I.m == 0) return e;
+        const int gy = (nb + 31) / 32;
+        const long long need = ((long long)I.m + kEvalWarps - 1) / kEvalWarps;
+        const dim3 grid((unsigned)std::max<long long>(1, std::min<long long>(need, (152LL * 8 + gy - 1) / gy)),
+                        (unsigned)gy);
+        const EvalInst E{I.m, I.kfix, I.coff, I.lit, I.w};
+        unsigned long long *cost = reinterpret_cast<unsigned long long *>(cost_out);
+        if (a) k_eval_direct<int8_t><<<grid, kThreads, 0, st>>>(E, a, nb, cost);
+        else k_eval_direct<float><<<grid, kThreads, 0, st>>>(E, x, nb, cost);
+        return cudaGetLastError();
+    }
+    for (int b0 = 0; b0 < nb && e == cudaSuccess; b0 += chunk) {
+        const int k = std::min(chunk, nb - b0);
+        const int8_t *ak = a ? a + b0 : nullptr;
+        const float *xk = a ? nullptr : x + b0;
+        unsigned long long *cost = reinterpret_cast<unsigned long long *>(cost_out) + b0;
+        switch (eval_vw(k)) {
+            case 4: launch_eval_vw<4>(I, ak, xk, nb, k, wbits, bits, cost, st); break;
+            case 2: launch_eval_vw<2>(I, ak, xk, nb, k, wbits, bits, cost, st); break;
+            default: launch_eval_vw<1>(I, ak, xk, nb, k, wbits, bits, cost, st); break;
+        }
+        e = cudaGetLastError();
+    }
+    return e;
 }
 
 // The paper's quick reading of a clause as satisfied when f_j > 0 (Sec. 4,
@@ -139,14 +360,6 @@ cudaError_t launch_heuristic_gap(const DevInst &I, const float *x, long long *he
     if (blocks < 1) blocks = 1;
     k_heuristic_gap<<<(unsigned)blocks, kThreads, 0, st>>>(I, x, reinterpret_cast<unsigned long long *>(heur_unsat),
                                                            reinterpret_cast<unsigned long long *>(disagree));
-    return cudaGetLastError();
-}
-
-cudaError_t launch_round_pm1(const float *x, int8_t *a, long long count, cudaStream_t st) {
-    long long blocks = (count + kThreads - 1) / kThreads;
-    if (blocks > 152 * 16) blocks = 152 * 16;
-    if (blocks < 1) blocks = 1;
-    k_round_pm1<<<(unsigned)blocks, kThreads, 0, st>>>(x, a, count);
     return cudaGetLastError();
 }
 

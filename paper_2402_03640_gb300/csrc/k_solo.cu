@@ -538,7 +538,6 @@ bool build_solo(int32_t n, int64_t m, int32_t kfix, int32_t max_len, int32_t max
     // variables: one leaf first (longest first), then several leaves (those a
     // warp combines first)
     auto leaves = [&](int32_t i) { return (voff[i + 1] - voff[i] + 31) / 32; };
-    std::vector<int32_t> vid((size_t)n);          // variable -> internal id
     out.perm.resize((size_t)n);
     SoloShape sh;
     {
@@ -559,7 +558,6 @@ bool build_solo(int32_t n, int64_t m, int32_t kfix, int32_t max_len, int32_t max
         for (int32_t i = 0; i < n; ++i) {
             const int32_t d = voff[i + 1] - voff[i];
             const int32_t id = d <= 32 ? at[8 - (d + 3) / 4]++ : leaves(i) > kNarrowLeaves ? wide++ : narrow++;
-            vid[(size_t)i] = id;
             out.perm[(size_t)id] = i;
         }
     }
@@ -646,20 +644,39 @@ bool build_solo(int32_t n, int64_t m, int32_t kfix, int32_t max_len, int32_t max
     std::copy(mbeg.begin(), mbeg.end(), reinterpret_cast<int32_t *>(out.lists.data() + V.off_mbeg));
     std::fill(lw, lw + sh.lit_rows * 128, (uint16_t)(n << 1));
     std::fill(ow, ow + sh.occ_rows * 128, (uint16_t)(V.pairs ? 2 * m : m));
-    std::vector<int32_t> fill((size_t)n, 0);  // occurrences placed per internal id
+    // per variable: its word, where its current leaf's words go, the leaf
+    // task and the occurrences and signs placed in it
+    struct Fill {
+        uint32_t word, at, task, cnt, sgn;
+    };
+    std::vector<Fill> fill((size_t)n);
+    auto leaf_at = [&](uint32_t k) { return ((uint32_t)obase[k >> 5] * 32u + (k & 31u)) * 4u; };
+    for (int32_t id = 0; id < n; ++id) {
+        const uint32_t k = (uint32_t)tfirst[(size_t)id];
+        fill[(size_t)out.perm[(size_t)id]] = Fill{(uint32_t)id << 1, leaf_at(k), k, 0u, 0u};
+    }
+    const uint32_t pairs = V.pairs ? 1u : 0u;
     for (int64_t j = 0; j < m; ++j) {
-        const int32_t s = kfix > 0 ? (int32_t)j : slot[(size_t)j];
-        const int64_t row = lbase[(size_t)(s >> 5)];
-        for (int32_t p = coff[j]; p < coff[j + 1]; ++p) {
-            const int32_t Lw = lit[p], id = vid[(size_t)(Lw >> 1)], r = p - coff[j];
-            lw[((row + r / 4) * 32 + (s & 31)) * 4 + (r & 3)] = (uint16_t)((id << 1) | (Lw & 1));
-            const int32_t e = fill[(size_t)id]++;
-            const int32_t k = tfirst[(size_t)id] + e / 32, q = e & 31;
-            ow[((obase[(size_t)(k >> 5)] + q / 4) * 32 + (k & 31)) * 4 + (q & 3)] =
-                (uint16_t)(V.pairs ? (s << 1) | (Lw & 1) : s);
-            sg[k] |= (uint32_t)(Lw & 1) << q;
+        const uint32_t s = (uint32_t)(kfix > 0 ? j : slot[(size_t)j]);
+        uint16_t *l0 = lw + ((size_t)lbase[s >> 5] * 32 + (s & 31u)) * 4;
+        const int32_t *c = lit + coff[j];
+        const int32_t len = coff[j + 1] - coff[j];
+        for (int32_t r = 0; r < len; ++r) {
+            const uint32_t neg = (uint32_t)c[r] & 1u;
+            Fill &F = fill[(size_t)(c[r] >> 1)];
+            if (F.cnt == 32u) {
+                sg[F.task] = F.sgn;
+                ++F.task;
+                F.at = leaf_at(F.task);
+                F.cnt = F.sgn = 0u;
+            }
+            l0[(r >> 2) * 128 + (r & 3)] = (uint16_t)(F.word | neg);
+            ow[F.at + (F.cnt >> 2) * 128u + (F.cnt & 3u)] = (uint16_t)((s << pairs) | (neg & pairs));
+            F.sgn |= neg << F.cnt;
+            ++F.cnt;
         }
     }
+    for (const Fill &F : fill) sg[F.task] = F.sgn;
     out.slot = std::move(slot);
     V.n_single = sh.n_single;
     V.n_multi = sh.n_multi;

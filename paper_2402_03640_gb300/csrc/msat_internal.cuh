@@ -312,9 +312,10 @@ cudaError_t launch_loss_reduce(const DevStep &D, int B, cudaStream_t st);
 cudaError_t launch_solo_steps(const SoloDev &V, const DevInst &I, const DevState &S, const DevStep &D,
                               int n_steps, bool final_eval, cudaStream_t st);
 bool solo_pays(const SoloDev &V, const DevInst &I, int64_t nnz, int max_len, int64_t steps);
-cudaError_t launch_eval_sparse(const DevInst &I, const int8_t *a, int nb, long long *cost,
-                               cudaStream_t st);
-cudaError_t launch_round_pm1(const float *x, int8_t *a, long long count, cudaStream_t st);
+size_t eval_sparse_bytes(int n, int nb);
+bool eval_is_direct(int64_t nnz, int nb);
+cudaError_t launch_eval_sparse(const DevInst &I, const int8_t *a, const float *x, int nb, int chunk, int wbits,
+                               uint32_t *bits, long long *cost_out, cudaStream_t st);
 cudaError_t launch_heuristic_gap(const DevInst &I, const float *x, long long *heur_unsat,
                                  long long *disagree, cudaStream_t st);
 int dense_tile_n(int nb);
