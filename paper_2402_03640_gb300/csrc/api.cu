@@ -180,7 +180,7 @@ int msat::ctx_create(msat_ctx **out, int32_t n_vars, int64_t n_clauses, const in
     const int G = B / VW;
     // launch shapes
     auto pow2_le = [](int32_t v, int32_t cap) { return v >= 1 && v <= cap && (v & (v - 1)) == 0; };
-    const int32_t fwd_vw = cfg.fwd_vw ? cfg.fwd_vw : auto_fwd_vw(B);
+    const int32_t fwd_vw = cfg.fwd_vw ? cfg.fwd_vw : auto_fwd_vw(B, m);
     const int32_t stage_vw = cfg.stage_vw ? cfg.stage_vw : auto_stage_vw(B);
     if (!pow2_le(fwd_vw, std::min(8, B)) || !pow2_le(stage_vw, std::min(16, B)))
         return fail(MSAT_EINVAL, "msat_create: fwd_vw / stage_vw must be powers of two <= min(8 or 16, B)");
@@ -273,7 +273,9 @@ int msat::ctx_create(msat_ctx **out, int32_t n_vars, int64_t n_clauses, const in
         shape.n = n_vars;
         shape.B = B;
         shape.kfix = kfix;
-        use_solo = solo_pays(solo.dev, shape, nnz, max_len, 1 << 30);  // for a long call
+        // for a long call, with room for what the estimate does not know; each
+        // call then takes the faster route (the serving engine has only one)
+        use_solo = solo_pays(solo.dev, shape, nnz, max_len, 1 << 30, pool_alloc ? 1.0 : 1.5);
     }
     // the serving engine runs such an instance on that kernel alone: its
     // context holds none of the per-pass kernels' lists and buffers
@@ -570,7 +572,7 @@ static cudaError_t plain_steps(msat_ctx *c, int64_t n_steps) {
 static cudaError_t run_steps(msat_ctx *c, int64_t k, uint32_t flags, bool final_eval) {
     cudaError_t e = cudaSuccess;
     if (!c->prof_on && !(flags & MSAT_STEP_PER_PASS) && c->solo.lists &&
-        solo_pays(c->solo, c->I, c->nnz, c->max_len, k)) {
+        solo_pays(c->solo, c->I, c->nnz, c->max_len, k, 1.0)) {
         for (int64_t done = 0; !e;) {
             const int64_t now = std::min<int64_t>(k - done, 1 << 30);
             done += now;

@@ -755,19 +755,23 @@ cudaError_t launch_solo_steps(const SoloDev &V, const DevInst &I, const DevState
 
 // Whether `steps` steps are taken faster by this kernel than by the per-pass
 // kernels, from what both measured on one GB300 (microseconds a step).  A
-// block takes 1 + 0.24 per thousand literals (n=301 1.9, n=5000 14.5; 0.3
-// where the clause lengths differ: weighted Zipf n=2000 14.8), one wave of
+// block takes 1 + 0.24 per thousand literals of 3-literal clauses (n=301
+// 1.9, n=5000 14.5), 0.33 where lengths differ (weighted Zipf n=3000 20.6)
+// and 0.43 with clauses of more than 32 literals (PHP(40) 30), one wave of
 // SMs at a time (n=5000, B=256: 29), and gathers and scatters its column of
 // the state once a call (7e-5 per variable and restart: n=5000, B=256 90).
-// The two passes take 18 (launch and dependent latency), 1.4 per million
+// The two passes take 16 (launches and dependent latency), 1.4 per million
 // literal evaluations (n=5000, B=256: 43) and, for clauses that are not all
-// of three literals with four or more restarts, 4 + 0.35 per literal of the
-// longest (the ordering principle on 31 elements, B=8: 33 against 19 here).
-bool solo_pays(const SoloDev &V, const DevInst &I, int64_t nnz, int max_len, int64_t steps) {
+// of three literals, 0.2 per literal of the longest (PHP(40), B=1: 25) or,
+// with four or more restarts, 4 + 0.35 (the ordering principle on 31
+// elements, B=8: 31 against 19 here).  slack: factor allowed to this kernel.
+bool solo_pays(const SoloDev &V, const DevInst &I, int64_t nnz, int max_len, int64_t steps, double slack) {
     const double waves = (I.B + V.sms - 1) / V.sms;
-    const double solo = 1.0 + (I.kfix ? 0.24e-3 : 0.3e-3) * (double)nnz * waves;
-    const double passes = 18.0 + 1.4e-6 * (double)nnz * I.B + (I.kfix == 3 || I.B < 4 ? 0.0 : 4.0 + 0.35 * max_len);
-    return (double)steps * solo + 7e-5 * (double)I.n * I.B <= (double)std::max<int64_t>(steps, 1) * passes;
+    const double per_lit = V.kind == 0 ? 0.24e-3 : V.kind == 1 ? 0.33e-3 : 0.43e-3;
+    const double solo = 1.0 + per_lit * (double)nnz * waves;
+    const double passes = 16.0 + 1.4e-6 * (double)nnz * I.B +
+                          (I.kfix == 3 ? 0.0 : I.B < 4 ? 0.2 * max_len : 4.0 + 0.35 * max_len);
+    return (double)steps * solo + 7e-5 * (double)I.n * I.B <= slack * (double)std::max<int64_t>(steps, 1) * passes;
 }
 
 }  // namespace msat

@@ -174,11 +174,11 @@ __device__ __forceinline__ void clause_value(const DevInst &I, const float *__re
     float stk[kClauseLevels][VW];
     unsigned nleaf = 0;
     int in_leaf = 0;
-    if constexpr (WANT_SAT && VW <= 2) {
-        // the clause pass with one or two restarts a thread: NB literals at
+    if constexpr (WANT_SAT && VW <= 4) {
+        // the clause pass with up to four restarts a thread: NB literals at
         // a time -- their loads, then their row gathers, then the terms in
         // literal order (the same additions as one literal at a time)
-        constexpr int NB = 8 / VW;
+        constexpr int NB = VW == 1 ? 8 : 4;
         for (int p0 = beg; p0 < end; p0 += NB) {
             int L[NB];
             float tv[NB][VW];
@@ -334,63 +334,14 @@ __device__ __forceinline__ void term_from_f(const DevInst &I, int o, uint32_t ni
     }
 }
 
-// Terms of C occurrences (words o, expanded records ox, valid where ok) of
-// variable own_var for VW restarts at col, all loads of the C occurrences in
-// flight together.  With the clause pass's store, q = (float)w_j * f_j (NaN
-// where satisfied) gives the term +-(q * 2/W_U) or +0; otherwise the unsat
-// bits select the restarts whose f is recomputed (fetched together with the
-// bits when unsat clauses are dense).
-template <int VW, int KFIX, int C, bool STORE>
-__device__ __forceinline__ void occ_terms(const DevInst &I, const DevState &S, int kfix,
-                                          const float *__restrict__ tcur, const int (&o)[C],
-                                          const int2 (&ox)[C], const bool (&ok)[C], int own_var,
-                                          int col, const float (&cs)[VW], bool dense,
-                                          float (&term)[C][VW]) {
-    const int B = I.B;
-    if constexpr (STORE) {
-        float q[C][VW];
-#pragma unroll
-        for (int u = 0; u < C; ++u) {
-            if (ok[u]) {
-                ldv<VW>(S.fstore + (int64_t)(o[u] >> I.occ_shift) * B + col, q[u]);
-            } else {
-#pragma unroll
-                for (int e = 0; e < VW; ++e) q[u][e] = 0.0f;
-            }
-        }
-#pragma unroll
-        for (int u = 0; u < C; ++u) {
-            const bool neg = o[u] & 1;
-#pragma unroll
-            for (int e = 0; e < VW; ++e) {
-                const float g = q[u][e] * cs[e];
-                term[u][e] = (q[u][e] != q[u][e]) ? 0.0f : (neg ? -g : g);
-            }
-        }
-    } else {
-        uint32_t wd[C];
-        float f[C][VW];
-#pragma unroll
-        for (int u = 0; u < C; ++u) {
-            wd[u] = ok[u] ? __ldg(ubits_word(I, S.ubits, o[u], col)) : 0u;
-            if (dense && ok[u]) fetch_f<VW, KFIX>(I, kfix, tcur, o[u], ox[u], own_var, col, f[u]);
-        }
-#pragma unroll
-        for (int u = 0; u < C; ++u) {
-            const uint32_t nib = ok[u] ? occ_nib<VW>(I, o[u], wd[u], col) : 0u;
-#pragma unroll
-            for (int e = 0; e < VW; ++e) term[u][e] = 0.0f;
-            if (nib) {
-                if (!dense) fetch_f<VW, KFIX>(I, kfix, tcur, o[u], ox[u], own_var, col, f[u]);
-                term_from_f<VW>(I, o[u], nib, f[u], cs, term[u]);
-            }
-        }
-    }
-}
-
-// The same terms of C consecutive occurrences of one leaf, added in order
-// to the leaf sum (first: the chunk opens the leaf, so its first term
-// starts the sum instead of being added to +0).
+// Adds the terms of C consecutive occurrences (words o, expanded records ox,
+// valid where ok) of variable own_var for VW restarts at col to the sum of
+// their leaf, in order, all their loads in flight together (first: they open
+// the leaf, so the first term starts the sum instead of being added to +0).
+// With the clause pass's store, q = (float)w_j * f_j (NaN where satisfied)
+// gives the term +-(q * 2/W_U) or +0; otherwise the unsat bits select the
+// restarts whose f is recomputed (fetched together with the bits when unsat
+// clauses are dense).
 template <int VW, int KFIX, int C, bool STORE>
 __device__ __forceinline__ void occ_accumulate(const DevInst &I, const DevState &S, int kfix,
                                                const float *__restrict__ tcur, const int (&o)[C],
@@ -446,17 +397,31 @@ __device__ __forceinline__ void occ_accumulate(const DevInst &I, const DevState 
 
 // --------------------------------------------------------------- update
 
+// x, moments and t of one (variable, restart group).
+template <int VW>
+struct VarState {
+    float x[VW], m[VW], v[VW], t[VW];
+    __device__ __forceinline__ void load(const DevState &S, const float *__restrict__ tcur, int64_t q0) {
+        ldv_stream<VW>(S.x + q0, x);
+        ldv_stream<VW>(S.mom + q0, m);
+        ldv_stream<VW>(S.vel + q0, v);
+        ldv<VW>(tcur + q0, t);
+    }
+};
+
 // Update of one (variable, restart group) from its occurrence sum S: the
 // gradient S * (1 - t^2) with t = tanh(x) of the evaluated x, then Adam
 // (unless the restart has stopped), the best-assignment capture and tanh of
-// the new x; or, in the gradient-only mode, the scaled gradient.
+// the new x; or, in the gradient-only mode, the scaled gradient.  pre: the
+// state loaded earlier, or nullptr.
 template <int VW>
 __device__ __forceinline__ void finish_variable(const DevState &S, const DevStep &D,
                                                 const AdamView &A, int mode, int64_t q0,
                                                 int col, const float *__restrict__ tcur,
                                                 const float (&Ssum)[VW], float *tnext,
                                                 const float *__restrict__ gscale,
-                                                float *__restrict__ grad_out) {
+                                                float *__restrict__ grad_out,
+                                                const VarState<VW> *pre = nullptr) {
     if constexpr (VW > 4) {  // slices of four restarts keep the live registers down
 #pragma unroll
         for (int h = 0; h < VW; h += 4) {
@@ -467,33 +432,35 @@ __device__ __forceinline__ void finish_variable(const DevState &S, const DevStep
         }
         return;
     }
-    float tv[VW], gr[VW];
-    ldv<VW>(tcur + q0, tv);
-#pragma unroll
-    for (int e = 0; e < VW; ++e) gr[e] = Ssum[e] * fmaf(-tv[e], tv[e], 1.0f);
     if (mode == BWD_GRAD_ONLY) {
+        float tv[VW], gr[VW];
+        ldv<VW>(tcur + q0, tv);
 #pragma unroll
-        for (int e = 0; e < VW; ++e) gr[e] = gscale ? gr[e] * gscale[col + e] : gr[e];
+        for (int e = 0; e < VW; ++e) {
+            gr[e] = Ssum[e] * fmaf(-tv[e], tv[e], 1.0f);
+            gr[e] = gscale ? gr[e] * gscale[col + e] : gr[e];
+        }
         stv<VW>(grad_out + q0, gr);
         return;
     }
-    float xv[VW], mv[VW], vv[VW], tn[VW];
-    ldv_stream<VW>(S.x + q0, xv);
-    ldv_stream<VW>(S.mom + q0, mv);
-    ldv_stream<VW>(S.vel + q0, vv);
+    VarState<VW> w;
+    if (pre) w = *pre;
+    else w.load(S, tcur, q0);
+    float tn[VW];
 #pragma unroll
     for (int e = 0; e < VW; ++e) {
-        if (D.improved[col + e]) S.bestx[q0 + e] = xv[e] > 0.0f;
+        const float gr = Ssum[e] * fmaf(-w.t[e], w.t[e], 1.0f);
+        if (D.improved[col + e]) S.bestx[q0 + e] = w.x[e] > 0.0f;
         if (D.cost[col + e] != 0) {
-            xv[e] = adam_update(A, xv[e], mv[e], vv[e], gr[e]);
-            tn[e] = tanh_fixed(xv[e]);
+            w.x[e] = adam_update(A, w.x[e], w.m[e], w.v[e], gr);
+            tn[e] = tanh_fixed(w.x[e]);
         } else {
-            tn[e] = tv[e];
+            tn[e] = w.t[e];
         }
     }
-    stv_stream<VW>(S.x + q0, xv);
-    stv_stream<VW>(S.mom + q0, mv);
-    stv_stream<VW>(S.vel + q0, vv);
+    stv_stream<VW>(S.x + q0, w.x);
+    stv_stream<VW>(S.mom + q0, w.m);
+    stv_stream<VW>(S.vel + q0, w.v);
     stv<VW>(tnext + q0, tn);
 }
 
@@ -556,6 +523,20 @@ cudaError_t launch_tanh(const float *x, float *t, int64_t count, cudaStream_t st
     return cudaGetLastError();
 }
 
+// Replicas of the per-restart cost accumulator that are in use: the blocks'
+// additions to one address wait for one another (n=5000, B=256: 22 us with 32
+// replicas, 38 with one), and the last block reads them all, a warp a restart
+// where there are few restarts, else a thread a restart, eight loads in
+// flight (sixteen raise the kernel's registers: 143 -> 153 us at n=1e6, B=16).
+template <int VW>
+__device__ __forceinline__ int cost_replicas(int B) {
+    return VW < 8 && B <= 8 ? kRep : kRep / 2;
+}
+
+// Items a lane of the clause pass has in flight: two where their rows (VW
+// values a literal) leave the registers for it.
+__host__ __device__ constexpr int fwd_items(int VW, int KFIX) { return VW <= 4 && VW * KFIX <= 12 ? 2 : 1; }
+
 // --------------------------------------------------------------- k_forward
 // One item = (clause j, restart group g of VW restarts).  For VW <= 4 the
 // grid-stride loop is unrolled by two (items base + lane and base + stride +
@@ -571,9 +552,8 @@ __device__ __forceinline__ void forward_body(const DevInst &I, const float *__re
                                              uint32_t *__restrict__ ubits,
                                              float *__restrict__ fstore, int mode, int blk,
                                              int nblk) {
-    constexpr int NU = VW <= 4 ? 2 : 1;  // items per lane per iteration
-    __shared__ unsigned long long s_w[kThreads];
-    __shared__ float s_l[kThreads];
+    constexpr int NU = fwd_items(VW, KFIX);  // items per lane per iteration
+    extern __shared__ float4 dyn_smem[];
     __shared__ int s_last;
 
     const int B = I.B;
@@ -673,53 +653,96 @@ __device__ __forceinline__ void forward_body(const DevInst &I, const float *__re
 
     // per restart: block sums.  The threads of restart group g are those
     // with threadIdx.x % G == g (G divides the block).  Lanes of one warp in
-    // the same group are combined by xor shuffles, then thread g adds the
-    // blockDim / max(G, 32) partials of its group.  The weights are integers
-    // (any order is exact); the loss partial's order is free because the
-    // loss is reported and never fed back into x.
-    unsigned long long *acc = D.wu_acc + (long long)(blk % kRep) * B;
-    const int per_group = blockDim.x / (G < 32 ? 32 : G);
+    // the same group are combined by xor shuffles, each row (a warp, or G
+    // threads where G > 32) puts its sums into shared memory, and threads add
+    // the rows: all VW restarts of the groups at once behind one barrier, or,
+    // with eight restarts a thread, one at a time (eight pairs of sums in
+    // shuffles at once take the kernel from 64 to 69 registers, three blocks
+    // per SM instead of four: 3-SAT n=1e6, B=16 143 -> 148 us).  The weights
+    // are integers (any order is exact); the loss partial's order is free
+    // because the loss is reported and never fed back into x.
+    const int nrep = cost_replicas<VW>(B);
+    unsigned long long *acc = D.wu_acc + (long long)(blk % nrep) * B;
+    unsigned long long *s_w = reinterpret_cast<unsigned long long *>(dyn_smem);
+    const int step = G < 32 ? 32 : G;  // threads of a row
+    const int rows = blockDim.x / step;
+    if constexpr (VW == 8) {
+        float *s_l = reinterpret_cast<float *>(s_w + kThreads);
 #pragma unroll
-    for (int e = 0; e < VW; ++e) {
-        unsigned long long sw = wacc[e];
-        float sl = lacc[e];
-        for (int o = G; o < 32; o <<= 1) {
-            sw += __shfl_xor_sync(0xffffffffu, sw, o);
-            sl += __shfl_xor_sync(0xffffffffu, sl, o);
-        }
-        s_w[threadIdx.x] = sw;
-        s_l[threadIdx.x] = sl;
-        __syncthreads();
-        if (threadIdx.x < G) {
-            sw = 0;
-            sl = 0.0f;
-            const int step = G < 32 ? 32 : G;
-            for (int k = 0; k < per_group; ++k) {
-                sw += s_w[threadIdx.x + k * step];
-                sl += s_l[threadIdx.x + k * step];
+        for (int e = 0; e < VW; ++e) {
+            unsigned long long sw = wacc[e];
+            float sl = lacc[e];
+            for (int o = G; o < 32; o <<= 1) {
+                sw += __shfl_xor_sync(0xffffffffu, sw, o);
+                sl += __shfl_xor_sync(0xffffffffu, sl, o);
             }
-            const int b = threadIdx.x * VW + e;
+            s_w[threadIdx.x] = sw;
+            s_l[threadIdx.x] = sl;
+            __syncthreads();
+            if (threadIdx.x < G) {
+                sw = 0;
+                sl = 0.0f;
+                for (int k = 0; k < rows; ++k) {
+                    sw += s_w[threadIdx.x + k * step];
+                    sl += s_l[threadIdx.x + k * step];
+                }
+                const int b = threadIdx.x * VW + e;
+                if (sw) atomicAdd(acc + b, sw);
+                D.lpart[(long long)blk * B + b] = sl;
+            }
+            __syncthreads();
+        }
+    } else {
+        float *s_l = reinterpret_cast<float *>(s_w + rows * B);
+        const int row = threadIdx.x / step;
+#pragma unroll
+        for (int e = 0; e < VW; ++e) {
+            unsigned long long sw = wacc[e];
+            float sl = lacc[e];
+            for (int o = G; o < 32; o <<= 1) {
+                sw += __shfl_xor_sync(0xffffffffu, sw, o);
+                sl += __shfl_xor_sync(0xffffffffu, sl, o);
+            }
+            if (G >= 32 || lane < G) {
+                s_w[row * B + col + e] = sw;
+                s_l[row * B + col + e] = sl;
+            }
+        }
+        __syncthreads();
+        for (int b = threadIdx.x; b < B; b += blockDim.x) {
+            unsigned long long sw = 0;
+            float sl = 0.0f;
+            for (int k = 0; k < rows; ++k) {
+                sw += s_w[k * B + b];
+                sl += s_l[k * B + b];
+            }
             if (sw) atomicAdd(acc + b, sw);
             D.lpart[(long long)blk * B + b] = sl;
         }
-        __syncthreads();
     }
     __threadfence();
+    __syncthreads();
     if (threadIdx.x == 0) s_last = (atomicAdd(&D.sc->counter, 1u) == nblk - 1);
     __syncthreads();
     if (!s_last) return;
     __threadfence();
-    unsigned long long my_tot = 0;  // this thread's restarts' costs
-    for (int b = threadIdx.x; b < B; b += blockDim.x) {
-        // every block's additions are complete (fence before the counter):
-        // read the replicas from L2, then clear them for the next pass
-        unsigned long long wu = 0;
-#pragma unroll 8
-        for (int r = 0; r < kRep; ++r) wu += __ldcg(D.wu_acc + (long long)r * B + b);
-#pragma unroll 8
-        for (int r = 0; r < kRep; ++r) D.wu_acc[(long long)r * B + b] = 0ull;
+    // the last block's finish: every block's additions are complete (fence
+    // before the counter).  The last thread makes the step's Adam scalars
+    // (double division and root) while the others sum the replicas.
+    if (mode == FWD_STEP && threadIdx.x == blockDim.x - 1) {
+        StepScalars *sc = D.sc;
+        const double p1 = sc->p1 * sc->beta1;
+        const double p2 = sc->p2 * sc->beta2;
+        sc->p1 = p1;
+        sc->p2 = p2;
+        sc->a_t = (float)(sc->lr / (1.0 - p1));
+        sc->r_t = (float)(1.0 / sqrt(1.0 - p2));
+        sc->steps_done = steps + 1;
+    }
+    // restart b's cost from L2, the replicas cleared for the next pass: one
+    // thread a restart, or for a few restarts one thread a replica
+    auto finish = [&](int b, unsigned long long wu) {
         const long long c = (long long)wu;
-        my_tot += wu;
         D.cost[b] = c;
         if (mode != FWD_PROBE) {
             const long long bb = D.best[b];
@@ -735,27 +758,47 @@ __device__ __forceinline__ void forward_body(const DevInst &I, const float *__re
         const int ln = D.sc->loss_norm;
         const float den = ln == 1 ? 1.0f : (float)(ln == 2 ? D.sc->wsum : c);
         D.cscale[b] = c > 0 ? 2.0f / den : 0.0f;
-    }
-    // the sum over the restarts from shared memory (integers: any order is
-    // exact); the costs just written to global memory are not read back
-    s_w[threadIdx.x] = my_tot;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        StepScalars *sc = D.sc;
-        sc->counter = 0;
-        unsigned long long tot = 0;
-        for (int k = 0; k < (int)blockDim.x; ++k) tot += s_w[k];
-        sc->dense = (double)tot * 16.0 > (double)sc->wsum * (double)B;
-        if (mode == FWD_STEP) {
-            const double p1 = sc->p1 * sc->beta1;
-            const double p2 = sc->p2 * sc->beta2;
-            sc->p1 = p1;
-            sc->p2 = p2;
-            sc->a_t = (float)(sc->lr / (1.0 - p1));
-            sc->r_t = (float)(1.0 / sqrt(1.0 - p2));
-            sc->steps_done = steps + 1;
+    };
+    unsigned long long my_tot = 0;  // this thread's restarts' costs
+    if (VW < 8 && nrep == kRep) {
+        for (int b = threadIdx.x >> 5; b < B; b += blockDim.x >> 5) {
+            unsigned long long wu = __ldcg(D.wu_acc + (long long)lane * B + b);
+            D.wu_acc[(long long)lane * B + b] = 0ull;
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) wu += __shfl_xor_sync(0xffffffffu, wu, o);
+            if (lane == 0) {
+                my_tot += wu;
+                finish(b, wu);
+            }
+        }
+    } else {
+        for (int b = threadIdx.x; b < B; b += blockDim.x) {
+            unsigned long long wu = 0;
+#pragma unroll 8
+            for (int r = 0; r < kRep / 2; ++r) wu += __ldcg(D.wu_acc + (long long)r * B + b);
+#pragma unroll 8
+            for (int r = 0; r < kRep / 2; ++r) D.wu_acc[(long long)r * B + b] = 0ull;
+            my_tot += wu;
+            finish(b, wu);
         }
     }
+    if (threadIdx.x == 0) D.sc->counter = 0;
+    if (fstore) return;  // uniform: only a recomputing variable pass reads the density
+    s_w = reinterpret_cast<unsigned long long *>(dyn_smem);
+    __syncthreads();
+    if (threadIdx.x == 0) s_w[0] = 0ull;
+    __syncthreads();
+    if (my_tot) atomicAdd(s_w, my_tot);
+    __syncthreads();
+    if (threadIdx.x == 0) D.sc->dense = (double)s_w[0] * 16.0 > (double)D.sc->wsum * (double)B;
+}
+
+// Dynamic shared memory of the clause pass: its per-restart block sums.
+template <int VW>
+static size_t fwd_smem(int B) {
+    const int G = B / VW;
+    return (VW == 8 ? (size_t)kThreads : (size_t)(kThreads / (G < 32 ? 32 : G)) * B) *
+           (sizeof(unsigned long long) + sizeof(float));
 }
 
 template <int VW, int KFIX>
@@ -766,16 +809,27 @@ __global__ void __launch_bounds__(kThreads)
     forward_body<VW, KFIX>(I, t0, t1, t_ovr, D, ubits, fstore, mode, blockIdx.x, gridDim.x);
 }
 
-int auto_fwd_vw(int B) { return B < 8 ? B : 8; }
+// Four restarts a thread in the clause pass; eight where the store is past
+// 64 MiB: its rows then come from HBM and are better taken whole (3-SAT
+// n=1e6, B=16: 140 us with eight, 172 with four; n=3e5, B=8, 41 MB: 38 / 31;
+// ordering principle on 31 elements, B=8: 21 / 15).
+int auto_fwd_vw(int B, int64_t m) {
+    return std::min(B, (double)m * B * sizeof(float) > 64.0 * (1 << 20) ? 8 : 4);
+}
 int auto_stage_vw(int B) { return B < 4 ? B : 4; }
 int update_vw(int B) { return B < 4 ? B : 4; }
 
 template <int VW>
 static int fwd_resident(const DevInst &I) {
     int per_sm = 0;
-    cudaError_t e = I.kfix == 3
-        ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_forward<VW, 3>, kThreads, 0)
-        : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_forward<VW, 0>, kThreads, 0);
+    const size_t smem = fwd_smem<VW>(I.B);
+    cudaError_t e;
+    switch (I.kfix) {
+        case 3: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_forward<VW, 3>, kThreads, smem); break;
+        case 4: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_forward<VW, 4>, kThreads, smem); break;
+        case 5: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_forward<VW, 5>, kThreads, smem); break;
+        default: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_forward<VW, 0>, kThreads, smem); break;
+    }
     if (e != cudaSuccess || per_sm < 1) {
         cudaGetLastError();
         per_sm = 2;
@@ -793,7 +847,7 @@ static int fwd_resident(const DevInst &I) {
 // fewer when the clauses do not fill it.
 int fwd_grid_blocks(const DevInst &I) {
     const int VW = I.fwd_vw;
-    const int per_thread = VW <= 4 ? 2 : 1;
+    const int per_thread = fwd_items(VW, I.kfix >= 3 && I.kfix <= 5 ? I.kfix : 0);
     const long long items = (long long)I.m * (I.B / VW);
     long long blocks = (items + per_thread * kThreads - 1) / (per_thread * kThreads);
     int resident;
@@ -812,10 +866,15 @@ template <int VW>
 static cudaError_t launch_forward_vw(const DevInst &I, const DevState &S, const DevStep &D,
                                      int mode, const float *t_ovr, cudaStream_t st) {
     const int blocks = D.fwd_blocks;
-    if (I.kfix == 3)
-        k_forward<VW, 3><<<blocks, kThreads, 0, st>>>(I, S.t0, S.t1, t_ovr, D, S.ubits, S.fstore, mode);
-    else
-        k_forward<VW, 0><<<blocks, kThreads, 0, st>>>(I, S.t0, S.t1, t_ovr, D, S.ubits, S.fstore, mode);
+    const size_t smem = fwd_smem<VW>(I.B);
+    // one instantiation per common clause length: all literals, then all rows
+    // of a clause in flight (k = 5, n=30011, m=639234, B=64: 144 -> 97 us)
+    switch (I.kfix) {
+        case 3: k_forward<VW, 3><<<blocks, kThreads, smem, st>>>(I, S.t0, S.t1, t_ovr, D, S.ubits, S.fstore, mode); break;
+        case 4: k_forward<VW, 4><<<blocks, kThreads, smem, st>>>(I, S.t0, S.t1, t_ovr, D, S.ubits, S.fstore, mode); break;
+        case 5: k_forward<VW, 5><<<blocks, kThreads, smem, st>>>(I, S.t0, S.t1, t_ovr, D, S.ubits, S.fstore, mode); break;
+        default: k_forward<VW, 0><<<blocks, kThreads, smem, st>>>(I, S.t0, S.t1, t_ovr, D, S.ubits, S.fstore, mode); break;
+    }
     return cudaGetLastError();
 }
 
@@ -838,159 +897,148 @@ cudaError_t launch_forward(const DevInst &I0, const DevState &S, const DevStep &
 }
 
 // -------------------------------------------------------------- k_backward
-// Per restart b < B, block b of the light kernel also reduces the loss of
-// the evaluated x from the forward block partials.
+// The loss of the evaluated x from the clause pass's block partials, a warp
+// a restart: by blocks of their own behind the variable pass's, so no block
+// of variables waits for it.
 
-__device__ __forceinline__ void reduce_loss(const DevStep &D, int B, int blk, int nblk) {
-    __shared__ float s_red[kThreads];
-    for (int b = blk; b < B; b += nblk) {
-        float acc = 0.0f;
-        for (int k = threadIdx.x; k < D.fwd_blocks; k += blockDim.x)
-            acc += D.lpart[(long long)k * B + b];
-        s_red[threadIdx.x] = acc;
-        __syncthreads();
-        for (int s = blockDim.x / 2; s > 0; s >>= 1) {
-            if (threadIdx.x < s) s_red[threadIdx.x] += s_red[threadIdx.x + s];
-            __syncthreads();
-        }
-        if (threadIdx.x == 0) {
-            const long long c = D.cost[b];
-            const int ln = D.sc->loss_norm;
-            const float den = ln == 1 ? 1.0f : (float)(ln == 2 ? D.sc->wsum : c);
-            D.loss[b] = c > 0 ? s_red[0] / den : 0.0f;
-        }
-        __syncthreads();
+constexpr int kWarps = kThreads / 32;
+
+__host__ __device__ inline int loss_blocks(int B) { return (B + kWarps - 1) / kWarps; }
+
+__device__ __forceinline__ void reduce_loss(const DevStep &D, int B, int blk) {
+    const int b = blk * kWarps + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    if (b >= B) return;
+    float acc = 0.0f;
+#pragma unroll 4
+    for (int k = lane; k < D.fwd_blocks; k += 32) acc += D.lpart[(long long)k * B + b];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    if (lane == 0) {
+        const long long c = D.cost[b];
+        const int ln = D.sc->loss_norm;
+        const float den = ln == 1 ? 1.0f : (float)(ln == 2 ? D.sc->wsum : c);
+        D.loss[b] = c > 0 ? acc / den : 0.0f;
     }
 }
 
-// k_backward_heavy: one block per (1024-occurrence chunk, restart group of
-// VW restarts) of a heavy variable.  The chunk's terms are staged in shared
-// memory; 32 leaves of 32 terms are summed in order and combined by the
-// dyadic tree; the last chunk block of a (variable, group) combines the
-// chunk partials with the same tree and applies the update.
+// Heavy variables: a warp per (1024-occurrence chunk, restart group of VW
+// restarts), a lane per 32-occurrence leaf.  A lane sums its leaf in the
+// stored order straight from its gathers, the lanes' leaves meet by the
+// dyadic shuffle tree, and the last chunk of a (variable, group) combines the
+// chunk partials with the same tree and applies the update.  No barrier and
+// no staging: bound by the latency of the word -> row chain, hidden by 32
+// leaves a warp.  The form before it staged a chunk in shared memory with a
+// block and summed the leaves with one of its eight warps (32 lanes on one
+// bank): variable pass of weighted Zipf n=2e5, m=1e6 (3255 chunks), B=1 49 ->
+// 40 us, B=8 201 -> 130 us.
 template <int VW, int KFIX, bool STORE>
 __device__ __forceinline__ void heavy_body(const DevInst &I, const DevState &S, const DevStep &D,
                                            int mode, const float *__restrict__ t_ovr,
                                            const float *__restrict__ gscale,
                                            float *__restrict__ grad_out, int blk) {
-    __shared__ float s_term[kChunk * VW];
-    __shared__ int s_last;
+    constexpr int C = VW <= 2 ? 8 : 4;  // occurrences in flight per lane
     const int B = I.B;
     const int G = B / VW;
     const int kfix = KFIX > 0 ? KFIX : I.kfix;
-    const float *tcur;
-    float *tnext;
-    step_buffers(S, D, mode, t_ovr, tcur, tnext);
-    const AdamView A = adam_view(D.sc);
-    const int gg = blk % G;
-    const long long cidx = blk / G;
+    const int lane = threadIdx.x & 31;
+    const long long wid = (long long)blk * kWarps + (threadIdx.x >> 5);
+    const long long cidx = wid / G;
+    if (cidx >= I.heavy_chunks) return;
+    const int gg = (int)(wid - cidx * G);
     const int col = gg * VW;
     const int h = __ldg(I.heavy_of_chunk + cidx);
     const int i = __ldg(I.heavy_var + h);
     const int c0 = __ldg(I.heavy_chunk0 + h);
     const int nch = __ldg(I.heavy_chunk0 + h + 1) - c0;
-    const int c = (int)(cidx - c0);
-    const int vbeg = __ldg(I.voff + i), vend = __ldg(I.voff + i + 1);
-    const int cb = vbeg + c * kChunk;
+    const int vend = __ldg(I.voff + i + 1);
+    const int cb = __ldg(I.voff + i) + (int)(cidx - c0) * kChunk;
     const int cn = min(kChunk, vend - cb);  // occurrences in this chunk
-    const int lane = threadIdx.x & 31;
-    float cs[VW];
-#pragma unroll
-    for (int e = 0; e < VW; ++e) cs[e] = D.cscale[col + e];
-
+    const float *tcur;
+    float *tnext;
+    step_buffers(S, D, mode, t_ovr, tcur, tnext);
     if (mode != BWD_BITS_ONLY) {
-        // phase 1: the chunk's terms into shared memory, four per thread in flight
+        float cs[VW];
+#pragma unroll
+        for (int e = 0; e < VW; ++e) cs[e] = D.cscale[col + e];
         const bool dense = D.sc->dense != 0;
         const bool expanded = KFIX == 3 && I.occx != nullptr;
-        int o[4];
-        int2 ox[4];
-        bool ok[4];
+        const int pb = cb + min(32 * lane, cn), pe = cb + min(32 * lane + 32, cn);
+        float leaf[VW];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const int r = threadIdx.x + u * kThreads;
-            ok[u] = r < cn;
-            o[u] = ok[u] ? __ldcs(I.occ + cb + r) : 0;
-            ox[u] = (expanded && ok[u]) ? __ldcs(I.occx + cb + r) : make_int2(0, 0);
+        for (int e = 0; e < VW; ++e) leaf[e] = 0.0f;
+        int on[C];
+        int2 oxn[C];
+#pragma unroll
+        for (int u = 0; u < C; ++u) {
+            const bool okn = pb + u < pe;
+            on[u] = okn ? __ldg(I.occ + pb + u) : 0;
+            oxn[u] = (expanded && okn) ? __ldg(I.occx + pb + u) : make_int2(0, 0);
         }
-        float term[4][VW];
-        occ_terms<VW, KFIX, 4, STORE>(I, S, kfix, tcur, o, ox, ok, i, col, cs, dense, term);
+        for (int p = pb; p < pe; p += C) {
+            int o[C];
+            int2 ox[C];
+            bool ok[C];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const int r = threadIdx.x + u * kThreads;
-            if (ok[u]) {
-#pragma unroll
-                for (int e = 0; e < VW; ++e) s_term[r * VW + e] = term[u][e];
+            for (int u = 0; u < C; ++u) {
+                ok[u] = p + u < pe;
+                o[u] = on[u];
+                ox[u] = oxn[u];
+                const bool okn = p + C + u < pe;
+                on[u] = okn ? __ldg(I.occ + p + C + u) : 0;
+                oxn[u] = (expanded && okn) ? __ldg(I.occx + p + C + u) : make_int2(0, 0);
             }
+            occ_accumulate<VW, KFIX, C, STORE>(I, S, kfix, tcur, o, ox, ok, i, col, cs, dense, p == pb, leaf);
         }
-        __syncthreads();
-        // phase 2: 32 leaves of 32 terms in order, then the dyadic tree
-        if (threadIdx.x < 32) {
-            float leaf[VW];
+        __syncwarp();
+        const int K = (cn + 31) / 32;
 #pragma unroll
-            for (int e = 0; e < VW; ++e) leaf[e] = 0.0f;
-            const int lb = lane * 32, le = min(lb + 32, cn);
-#pragma unroll 8
-            for (int r = lb; r < le; ++r)
+        for (int e = 0; e < VW; ++e) leaf[e] = warp_dyadic(leaf[e], K, lane);
+        if (lane == 0) {
 #pragma unroll
-                for (int e = 0; e < VW; ++e) leaf[e] = (r == lb) ? s_term[r * VW + e] : leaf[e] + s_term[r * VW + e];
-            const int K = (cn + 31) / 32;
-#pragma unroll
-            for (int e = 0; e < VW; ++e) leaf[e] = warp_dyadic(leaf[e], K, lane);
-            if (lane == 0) {
-#pragma unroll
-                for (int e = 0; e < VW; ++e) D.hpart[cidx * B + col + e] = leaf[e];
-            }
+            for (int e = 0; e < VW; ++e) D.hpart[cidx * B + col + e] = leaf[e];
         }
     }
-    // thread 0 wrote the chunk's partial: it alone fences before counting in
-    if (threadIdx.x == 0) {
-        __threadfence();
-        s_last = (atomicAdd(D.hcount + (long long)h * G + gg, 1u) == (unsigned)(nch - 1));
-    }
-    __syncthreads();
-    if (!s_last) return;
-    __threadfence();
-    // last chunk block of this (variable, group): dyadic tree over the chunk
-    // partials, kChunk of them per round (a round is a complete dyadic block)
-    LeafCounter<8> lc[VW];
-#pragma unroll
-    for (int e = 0; e < VW; ++e) lc[e].init();
-    if (mode != BWD_BITS_ONLY) {
-        for (int base = 0; base < nch; base += kChunk) {
-            const int K = min(kChunk, nch - base);
-            __syncthreads();
-            for (int r = threadIdx.x; r < K; r += kThreads)
-#pragma unroll
-                for (int e = 0; e < VW; ++e)
-                    s_term[r * VW + e] = __ldcg(D.hpart + (long long)(c0 + base + r) * B + col + e);
-            __syncthreads();
-            for (int st = 1; st < K; st <<= 1) {
-                for (int r = threadIdx.x * 2 * st; r < K; r += kThreads * 2 * st)
-                    if (r + st < K)
-#pragma unroll
-                        for (int e = 0; e < VW; ++e) s_term[r * VW + e] = s_term[r * VW + e] + s_term[(r + st) * VW + e];
-                __syncthreads();
-            }
-            if (threadIdx.x == 0)
-#pragma unroll
-                for (int e = 0; e < VW; ++e) lc[e].push(s_term[e]);
-        }
-    }
-    if (threadIdx.x != 0) return;
-    D.hcount[(long long)h * G + gg] = 0;
     const int64_t q0 = (int64_t)i * B + col;
     if (mode == BWD_BITS_ONLY) {
-        float xv[VW];
-        ldv_rw<VW>(S.x + q0, xv);
-#pragma unroll
-        for (int e = 0; e < VW; ++e)
-            if (D.improved[col + e]) S.bestx[q0 + e] = xv[e] > 0.0f;
+        if (cidx == c0 && lane < VW && D.improved[col + lane]) S.bestx[q0 + lane] = S.x[q0 + lane] > 0.0f;
         return;
     }
+    int last = 1;
+    if (nch > 1) {
+        if (lane == 0) {
+            __threadfence();
+            last = atomicAdd(D.hcount + (long long)h * G + gg, 1u) == (unsigned)(nch - 1);
+            if (last) D.hcount[(long long)h * G + gg] = 0;
+        }
+        last = __shfl_sync(0xffffffffu, last, 0);
+    }
+    if (!last) return;
+    __threadfence();
+    __syncwarp();
+    // last chunk of this (variable, group): 32 consecutive chunk partials at
+    // a time are a complete dyadic block; four blocks' loads in flight
     float Ssum[VW];
 #pragma unroll
-    for (int e = 0; e < VW; ++e) Ssum[e] = lc[e].finish();
-    finish_variable<VW>(S, D, A, mode, q0, col, tcur, Ssum, tnext, gscale, grad_out);
+    for (int e = 0; e < VW; ++e) {
+        LeafCounter<12> lc;  // up to 4095 blocks of 32 chunks
+        lc.init();
+        for (int base = 0; base < nch; base += 128) {
+            float v[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int r = base + 32 * u + lane;
+                v[u] = r < nch ? __ldcg(D.hpart + (long long)(c0 + r) * B + col + e) : 0.0f;
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int K = nch - base - 32 * u;
+                if (K > 0) lc.push(warp_dyadic(v[u], min(K, 32), lane));
+            }
+        }
+        Ssum[e] = lc.finish();
+    }
+    if (lane != 0) return;
+    finish_variable<VW>(S, D, adam_view(D.sc), mode, q0, col, tcur, Ssum, tnext, gscale, grad_out);
 }
 
 template <int VW, int KFIX, bool STORE>
@@ -1014,7 +1062,7 @@ template <int VS, int KFIX, bool STORE>
 __device__ __forceinline__ void vars_body(const DevInst &I, const DevState &S, const DevStep &D,
                                           int mode, const float *__restrict__ t_ovr,
                                           const float *__restrict__ gscale,
-                                          float *__restrict__ grad_out, int blk, int nblk) {
+                                          float *__restrict__ grad_out, int blk) {
     constexpr int C = 4;  // occurrences in flight per thread
     extern __shared__ float4 dyn_smem[];
     __shared__ int s_voff[kThreads + 1];
@@ -1025,8 +1073,10 @@ __device__ __forceinline__ void vars_body(const DevInst &I, const DevState &S, c
     const float *tcur;
     float *tnext;
     step_buffers(S, D, mode, t_ovr, tcur, tnext);
-    if (mode == BWD_UPDATE) reduce_loss(D, B, blk, nblk);
-    if (blk >= I.n_lblk) return;  // a grid of one block when every variable is heavy
+    if (blk >= I.n_lblk) {  // the blocks behind the variables'
+        if (mode == BWD_UPDATE) reduce_loss(D, B, blk - I.n_lblk);
+        return;
+    }
     const AdamView A = adam_view(D.sc);
     float *s_leaf = reinterpret_cast<float *>(dyn_smem);
     const int2 rg = I.lblk[blk];
@@ -1094,6 +1144,12 @@ __device__ __forceinline__ void vars_body(const DevInst &I, const DevState &S, c
         }
         const int pb = s_voff[vloc] + 32 * L;
         const int pe = min(pb + 32, s_voff[vloc + 1]);
+        // with one or two restarts a task there are registers to have the
+        // variable's state on its way while the occurrences are gathered
+        constexpr bool PRE = VS <= 2 && STORE;
+        VarState<VS> pre;
+        if constexpr (PRE)
+            if (nleaf == 1 && mode == BWD_UPDATE) pre.load(S, tcur, q0);
         float leaf[VS];
 #pragma unroll
         for (int e = 0; e < VS; ++e) leaf[e] = 0.0f;
@@ -1123,7 +1179,7 @@ __device__ __forceinline__ void vars_body(const DevInst &I, const DevState &S, c
             occ_accumulate<VS, KFIX, C, STORE>(I, S, kfix, tcur, o, ox, ok, i, col, cs, dense, p == pb, leaf);
         }
         if (nleaf == 1) {
-            finish_variable<VS>(S, D, A, mode, q0, col, tcur, leaf, tnext, gscale, grad_out);
+            finish_variable<VS>(S, D, A, mode, q0, col, tcur, leaf, tnext, gscale, grad_out, PRE ? &pre : nullptr);
         } else {
             stv<VS>(s_leaf + (int64_t)ti * B + col, leaf);
         }
@@ -1161,7 +1217,7 @@ template <int VS, int KFIX, bool STORE>
 __global__ void __launch_bounds__(kThreads)
     k_backward_light(DevInst I, DevState S, DevStep D, int mode, const float *__restrict__ t_ovr,
                      const float *__restrict__ gscale, float *__restrict__ grad_out) {
-    vars_body<VS, KFIX, STORE>(I, S, D, mode, t_ovr, gscale, grad_out, blockIdx.x, gridDim.x);
+    vars_body<VS, KFIX, STORE>(I, S, D, mode, t_ovr, gscale, grad_out, blockIdx.x);
 }
 
 // The same pass held to 64 registers a thread, so that four 256-thread
@@ -1173,7 +1229,7 @@ template <int VS, int KFIX, bool STORE>
 __global__ void __launch_bounds__(kThreads, 4)
     k_backward_light_occ4(DevInst I, DevState S, DevStep D, int mode, const float *__restrict__ t_ovr,
                           const float *__restrict__ gscale, float *__restrict__ grad_out) {
-    vars_body<VS, KFIX, STORE>(I, S, D, mode, t_ovr, gscale, grad_out, blockIdx.x, gridDim.x);
+    vars_body<VS, KFIX, STORE>(I, S, D, mode, t_ovr, gscale, grad_out, blockIdx.x);
 }
 
 // Heavy-variable chunks and light blocks in one launch: blocks [0, hblocks)
@@ -1183,27 +1239,37 @@ __global__ void __launch_bounds__(kThreads, 4)
 template <int VS, int VU, int KFIX, bool STORE, int MINB>
 __global__ void __launch_bounds__(kThreads, MINB)
     k_backward_mixed(DevInst I, DevState S, DevStep D, int mode, const float *__restrict__ t_ovr,
-                     const float *__restrict__ gscale, float *__restrict__ grad_out, int hblocks,
-                     int lblocks) {
+                     const float *__restrict__ gscale, float *__restrict__ grad_out, int hblocks) {
     if ((int)blockIdx.x < hblocks)
         heavy_body<VU, KFIX, STORE>(I, S, D, mode, t_ovr, gscale, grad_out, blockIdx.x);
     else
-        vars_body<VS, KFIX, STORE>(I, S, D, mode, t_ovr, gscale, grad_out, (int)blockIdx.x - hblocks, lblocks);
+        vars_body<VS, KFIX, STORE>(I, S, D, mode, t_ovr, gscale, grad_out, (int)blockIdx.x - hblocks);
+}
+
+// Blocks of the heavy variables: a warp per (chunk, restart group).
+int heavy_blocks_of(const DevInst &I) {
+    const long long warps = I.n_heavy > 0 ? I.heavy_chunks * (I.B / update_vw(I.B)) : 0;
+    return (int)((warps + kWarps - 1) / kWarps);
+}
+
+// Blocks of the light variables, with those of the loss behind them.
+int light_blocks_of(const DevInst &I, int mode) {
+    return std::max(1, I.n_lblk + (mode == BWD_UPDATE ? loss_blocks(I.B) : 0));
 }
 
 template <int VS, int VU, int KFIX, bool STORE>
 static cudaError_t launch_backward_k(const DevInst &I, const DevState &S, const DevStep &D,
                                      int mode, const float *t_ovr, const float *gscale,
                                      float *grad_out, cudaStream_t st) {
-    const long long lblocks = I.n_lblk > 0 ? I.n_lblk : 1;
+    const long long lblocks = light_blocks_of(I, mode);
     const size_t smem = light_smem_bytes(I.task_cap, VS);
     if (I.n_heavy > 0) {
-        const long long hblocks = I.heavy_chunks * (I.B / VU);  // one block per (chunk, group)
+        const long long hblocks = heavy_blocks_of(I);
         if constexpr (STORE && VU <= 2 && VS <= 2) {
             // one launch where that keeps the light blocks' 64-register,
             // four-blocks-per-SM shape without spills
             k_backward_mixed<VS, VU, KFIX, STORE, 4><<<(unsigned)(hblocks + lblocks), kThreads, smem, st>>>(
-                I, S, D, mode, t_ovr, gscale, grad_out, (int)hblocks, (int)lblocks);
+                I, S, D, mode, t_ovr, gscale, grad_out, (int)hblocks);
             return cudaGetLastError();
         }
         k_backward_heavy<VU, KFIX, STORE><<<(unsigned)hblocks, kThreads, 0, st>>>(I, S, D, mode, t_ovr,
@@ -1271,8 +1337,13 @@ __global__ void __launch_bounds__(kThreads)
     const int s = slot_of(start, nslot, blockIdx.x);
     const int b0 = __ldg(start + s), b1 = __ldg(start + s + 1);
     const SlotDesc &sd = slots[s];
-    forward_body<VW, 0>(sd.I, sd.S.t0, sd.S.t1, nullptr, sd.D, sd.S.ubits, sd.S.fstore, FWD_STEP,
-                        blockIdx.x - b0, b1 - b0);
+    const int blk = blockIdx.x - b0, nblk = b1 - b0;
+    switch (sd.I.kfix) {  // uniform over the block
+        case 3: forward_body<VW, 3>(sd.I, sd.S.t0, sd.S.t1, nullptr, sd.D, sd.S.ubits, sd.S.fstore, FWD_STEP, blk, nblk); break;
+        case 4: forward_body<VW, 4>(sd.I, sd.S.t0, sd.S.t1, nullptr, sd.D, sd.S.ubits, sd.S.fstore, FWD_STEP, blk, nblk); break;
+        case 5: forward_body<VW, 5>(sd.I, sd.S.t0, sd.S.t1, nullptr, sd.D, sd.S.ubits, sd.S.fstore, FWD_STEP, blk, nblk); break;
+        default: forward_body<VW, 0>(sd.I, sd.S.t0, sd.S.t1, nullptr, sd.D, sd.S.ubits, sd.S.fstore, FWD_STEP, blk, nblk); break;
+    }
 }
 
 template <int VU>
@@ -1288,16 +1359,10 @@ template <int VS>
 __global__ void __launch_bounds__(kThreads)
     k_backward_light_batch(const SlotDesc *__restrict__ slots, const int *__restrict__ start, int nslot) {
     const int s = slot_of(start, nslot, blockIdx.x);
-    const int b0 = __ldg(start + s), b1 = __ldg(start + s + 1);
+    const int b0 = __ldg(start + s);
     const SlotDesc &sd = slots[s];
-    vars_body<VS, 0, true>(sd.I, sd.S, sd.D, BWD_UPDATE, nullptr, nullptr, nullptr, blockIdx.x - b0, b1 - b0);
+    vars_body<VS, 0, true>(sd.I, sd.S, sd.D, BWD_UPDATE, nullptr, nullptr, nullptr, blockIdx.x - b0);
 }
-
-int heavy_blocks_of(const DevInst &I) {
-    return I.n_heavy > 0 ? (int)(I.heavy_chunks * (I.B / update_vw(I.B))) : 0;
-}
-
-int light_blocks_of(const DevInst &I) { return I.n_lblk > 0 ? I.n_lblk : 1; }
 
 template <int VS, int VU>
 static cudaError_t launch_batch_bwd(const SlotDesc *slots, int nslot, const int *heavy_start,
@@ -1318,10 +1383,10 @@ cudaError_t launch_step_batch(const SlotDesc *slots, int nslot, const int *fwd_s
                               cudaStream_t st) {
     if (nslot <= 0) return cudaSuccess;
     switch (fwd_vw) {
-        case 8: k_forward_batch<8><<<(unsigned)fwd_total, kThreads, 0, st>>>(slots, fwd_start, nslot); break;
-        case 4: k_forward_batch<4><<<(unsigned)fwd_total, kThreads, 0, st>>>(slots, fwd_start, nslot); break;
-        case 2: k_forward_batch<2><<<(unsigned)fwd_total, kThreads, 0, st>>>(slots, fwd_start, nslot); break;
-        default: k_forward_batch<1><<<(unsigned)fwd_total, kThreads, 0, st>>>(slots, fwd_start, nslot); break;
+        case 8: k_forward_batch<8><<<(unsigned)fwd_total, kThreads, fwd_smem<8>(B), st>>>(slots, fwd_start, nslot); break;
+        case 4: k_forward_batch<4><<<(unsigned)fwd_total, kThreads, fwd_smem<4>(B), st>>>(slots, fwd_start, nslot); break;
+        case 2: k_forward_batch<2><<<(unsigned)fwd_total, kThreads, fwd_smem<2>(B), st>>>(slots, fwd_start, nslot); break;
+        default: k_forward_batch<1><<<(unsigned)fwd_total, kThreads, fwd_smem<1>(B), st>>>(slots, fwd_start, nslot); break;
     }
     cudaError_t e = cudaGetLastError();
     if (e) return e;
@@ -1341,11 +1406,10 @@ cudaError_t launch_step_batch(const SlotDesc *slots, int nslot, const int *fwd_s
 }
 
 // loss per restart from the forward partials (used where no update follows)
-__global__ void k_loss_reduce(DevStep D, int B) { reduce_loss(D, B, blockIdx.x, gridDim.x); }
+__global__ void k_loss_reduce(DevStep D, int B) { reduce_loss(D, B, blockIdx.x); }
 
 cudaError_t launch_loss_reduce(const DevStep &D, int B, cudaStream_t st) {
-    const int blocks = B < 152 * 4 ? B : 152 * 4;
-    k_loss_reduce<<<blocks, kThreads, 0, st>>>(D, B);
+    k_loss_reduce<<<loss_blocks(B), kThreads, 0, st>>>(D, B);
     return cudaGetLastError();
 }
 

@@ -286,7 +286,7 @@ struct LeafCounter {
 
 cudaError_t launch_init(const DevInst &I, const DevState &S, uint64_t seed, cudaStream_t st);
 int fwd_grid_blocks(const DevInst &I);
-int auto_fwd_vw(int B);
+int auto_fwd_vw(int B, int64_t m);
 int auto_stage_vw(int B);
 int update_vw(int B);
 enum { FWD_STEP = 0, FWD_EVAL = 1, FWD_PROBE = 2 };
@@ -304,14 +304,14 @@ cudaError_t launch_step_batch(const SlotDesc *slots, int nslot, const int *fwd_s
                               int light_total, int B, int fwd_vw, int stage_vw, int task_cap,
                               cudaStream_t st);
 int heavy_blocks_of(const DevInst &I);
-int light_blocks_of(const DevInst &I);
+int light_blocks_of(const DevInst &I, int mode);
 cudaError_t launch_loss_reduce(const DevStep &D, int B, cudaStream_t st);
 // Small instances: one block per restart takes every step of a call (and, if
 // asked, the evaluation of the final x) with the restart's state in shared
 // memory (k_solo.cu; same bits as the per-pass kernels).
 cudaError_t launch_solo_steps(const SoloDev &V, const DevInst &I, const DevState &S, const DevStep &D,
                               int n_steps, bool final_eval, cudaStream_t st);
-bool solo_pays(const SoloDev &V, const DevInst &I, int64_t nnz, int max_len, int64_t steps);
+bool solo_pays(const SoloDev &V, const DevInst &I, int64_t nnz, int max_len, int64_t steps, double slack);
 size_t eval_sparse_bytes(int n, int nb);
 bool eval_is_direct(int64_t nnz, int nb);
 cudaError_t launch_eval_sparse(const DevInst &I, const int8_t *a, const float *x, int nb, int chunk, int wbits,

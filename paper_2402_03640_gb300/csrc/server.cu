@@ -337,7 +337,7 @@ int rebuild(msat_server *S) {
         hst[2 * M + i] = l;
         f += c->D.fwd_blocks;
         h += heavy_blocks_of(c->I);
-        l += light_blocks_of(c->I);
+        l += light_blocks_of(c->I, BWD_UPDATE);
     }
     hst[n] = f;
     hst[M + n] = h;

@@ -46,9 +46,11 @@ int time_shape(int32_t n, int64_t m, const int64_t *off, const int32_t *lits, co
     cudaError_t e = cudaEventCreate(&e0);
     if (!e) e = cudaEventCreate(&e1);
     if (e) rc = cuda_fail(e, "msat_autotune: event");
-    if (!rc) rc = msat_step_ex(c, 2, MSAT_STEP_NO_FINAL_EVAL, nullptr, nullptr);
+    // the shapes are those of the per-pass kernels
+    const uint32_t flags = MSAT_STEP_NO_FINAL_EVAL | MSAT_STEP_PER_PASS;
+    if (!rc) rc = msat_step_ex(c, 2, flags, nullptr, nullptr);
     if (!rc && (e = cudaEventRecord(e0, st))) rc = cuda_fail(e, "msat_autotune: event");
-    if (!rc) rc = msat_step_ex(c, n_steps, MSAT_STEP_NO_FINAL_EVAL, nullptr, nullptr);
+    if (!rc) rc = msat_step_ex(c, n_steps, flags, nullptr, nullptr);
     if (!rc && (e = cudaEventRecord(e1, st))) rc = cuda_fail(e, "msat_autotune: event");
     if (!rc && (e = cudaEventSynchronize(e1))) rc = cuda_fail(e, "msat_autotune: timing");
     if (!rc && (e = cudaEventElapsedTime(ms, e0, e1))) rc = cuda_fail(e, "msat_autotune: timing");
@@ -114,7 +116,7 @@ extern "C" int msat_autotune(int32_t n_vars, int64_t n_clauses, const int64_t *c
     };
     // the automatic shape first: it is the reference every candidate must beat
     msat_config cand = base;
-    cand.fwd_vw = auto_fwd_vw(B);
+    cand.fwd_vw = auto_fwd_vw(B, n_clauses);
     cand.stage_vw = auto_stage_vw(B);
     cand.light_rows = kTaskCap;
     int rc = trial(cand);

@@ -84,3 +84,35 @@ def test_solo_kernel_keeps_nan_in_its_restart(pkg):
             out.append((cost, s.x(), s.best()[1]))
     for a, b in zip(*out):
         assert np.array_equal(a, b, equal_nan=True)
+
+
+@pytest.mark.parametrize("k", [3, 4, 5])
+@pytest.mark.parametrize("B,shape", [(1, {}), (2, {}), (4, {}), (8, dict(fwd_vw=8)), (64, dict(fwd_vw=4)),
+                                     (512, dict(fwd_vw=8))])
+def test_clause_pass_of_fixed_lengths(pkg, oracle, k, B, shape):
+    """The per-pass kernels on k-literal clauses for every width of the clause
+    pass, with a variable of several chunks among the heavy ones."""
+    cnf = uniform_ksat(60, 701, k, seed=15 + k)
+    S, lr = 6, 2e-2
+    ref = oracle.solve(cnf, B, 1, S, mode=oracle.MODE_F32, lr=lr)
+    with pkg.Solver.from_cnf(cnf, restarts=B, lr=lr, heavy_deg=8, **shape) as s:
+        cost = [s.step(1, want_loss=False, per_pass=True)[1] for _ in range(S)]
+        assert np.array_equal(np.stack(cost), ref["cost_hist"][1:])
+        assert np.array_equal(s.x().astype(np.float64), ref["x_final"])
+
+
+def test_heavy_variable_of_many_chunks(pkg, oracle):
+    """A variable of more than 128 chunks of 1024 occurrences (several rounds
+    of the chunk tree) and one of exactly 32 chunks."""
+    rng = np.random.default_rng(16)
+    m, n = 140001, 40
+    a = np.where(np.arange(m) < 32 * 1024, 2, 3 + rng.integers(0, n - 3, size=m))
+    lits = np.stack([np.full(m, 1), a, 3 + (a - 2 + rng.integers(0, n - 3, size=m)) % (n - 3)], 1)
+    lits = lits * rng.choice([-1, 1], size=lits.shape)
+    cnf = Cnf(n, np.arange(m + 1, dtype=np.int64) * 3, lits.reshape(-1).astype(np.int32))
+    for B in (1, 8):
+        ref = oracle.solve(cnf, B, 1, 3, mode=oracle.MODE_F32, lr=1e-2)
+        with pkg.Solver.from_cnf(cnf, restarts=B, lr=1e-2) as s:
+            assert s.info()["max_degree"] > 128 * 1024
+            s.step(3, want_loss=False, want_cost=False, per_pass=True)
+            assert np.array_equal(s.x().astype(np.float64), ref["x_final"])
