@@ -273,9 +273,11 @@ int msat::ctx_create(msat_ctx **out, int32_t n_vars, int64_t n_clauses, const in
         shape.n = n_vars;
         shape.B = B;
         shape.kfix = kfix;
+        shape.n_heavy = (int32_t)hvar.size();
         // for a long call, with room for what the estimate does not know; each
-        // call then takes the faster route (the serving engine has only one)
-        use_solo = solo_pays(solo.dev, shape, nnz, max_len, 1 << 30, pool_alloc ? 1.0 : 1.5);
+        // call then takes the faster route (the serving engine has only one,
+        // and its batch does not start a step for this instance alone)
+        use_solo = solo_pays(solo.dev, shape, nnz, max_len, 1 << 30, pool_alloc ? 1.5 : 2.0);
     }
     // the serving engine runs such an instance on that kernel alone: its
     // context holds none of the per-pass kernels' lists and buffers

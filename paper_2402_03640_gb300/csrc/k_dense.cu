@@ -58,6 +58,7 @@
 #include <string>
 
 #include "bits.cuh"
+#include "pdl.cuh"
 #include "msat_internal.cuh"
 
 namespace msat {
@@ -149,13 +150,6 @@ __device__ __forceinline__ bool mbar_wait_abort(unsigned long long *bar, uint32_
 __device__ __forceinline__ void mbar_arrive(unsigned long long *bar) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
-
-// Programmatic dependent launch: the evaluator is launched to overlap the
-// kernel that packs its assignment operand; it waits for that kernel (and
-// the visibility of its writes) before its first read of the packed batch
-// or write of the costs.  The packing kernels let it start at once.
-__device__ __forceinline__ void grid_dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void grid_dep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 // Named barrier of the eight epilogue warps (256 threads).
 __device__ __forceinline__ void epi_sync() { asm volatile("bar.sync 1, 256;" ::: "memory"); }
@@ -749,21 +743,21 @@ __device__ __forceinline__ void pack_transpose(const T *__restrict__ src, int n,
     }
 }
 
-// From the caller's int8 [n][nb] batch (> 0 is true).
-__global__ void k_dense_convert(const int8_t *__restrict__ a, int n, int nb, uint8_t *__restrict__ Xt,
-                                int n_pad, int rows) {
+// From the caller's int8 [n][nb] batch (> 0 is true), or straight from the
+// relaxed x (float [n][nb]): x > 0 reads as +1, otherwise -1 -- the rounding
+// of Sec. 4 -- without an int8 copy.  The evaluator is launched to overlap
+// this kernel: it waits for it (and the visibility of its writes) before its
+// first read of the packed batch or write of the costs, which are cleared
+// here (a clear of its own between the two kept them apart: n=5000, 256
+// assignments a call after the other 27.5 -> 20.1 us).
+template <typename T>
+__global__ void k_dense_convert(const T *__restrict__ a, int n, int nb, uint8_t *__restrict__ Xt,
+                                int n_pad, int rows, long long *__restrict__ cost) {
     grid_dep_launch();
-    pack_transpose<int8_t>(a, n, nb, Xt, n_pad, rows);
-}
-
-// The same operand straight from the relaxed x (float [n][nb]): x > 0 reads
-// as +1, otherwise -1 -- the rounding of Sec. 4 -- without the int8 copy.
-__global__ void k_dense_convert_x(const float *__restrict__ x, int n, int nb, uint8_t *__restrict__ Xt,
-                                  int n_pad, int rows, long long *__restrict__ cost) {
-    grid_dep_launch();
+    grid_dep_wait();
     if (blockIdx.x == 0 && blockIdx.y == 0)  // the GEMM that follows in stream order adds into cost
         for (int b = threadIdx.y * 32 + threadIdx.x; b < nb; b += 32 * blockDim.y) cost[b] = 0;
-    pack_transpose<float>(x, n, nb, Xt, n_pad, rows);
+    pack_transpose<T>(a, n, nb, Xt, n_pad, rows);
 }
 
 PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
@@ -833,20 +827,20 @@ cudaError_t launch_dense_fill(const DevInst &I, uint8_t *Wt, int n_pad, cudaStre
     return cudaGetLastError();
 }
 
+template <typename T>
+static cudaError_t launch_convert(const DenseDev &d, const T *a, int n, int nb, long long *cost, cudaStream_t st) {
+    dim3 cb(32, 8), cg((unsigned)(d.n_pad / 64), (unsigned)((d.tmB_rows + 31) / 32));
+    return launch_pdl(k_dense_convert<T>, cg, cb, 0, st, a, n, nb, d.Xt, d.n_pad, d.tmB_rows, cost);
+}
+
 cudaError_t launch_dense_convert(const DenseDev &d, const int8_t *a, int n, int nb, long long *cost,
                                  cudaStream_t st) {
-    dim3 cb(32, 8), cg((unsigned)(d.n_pad / 64), (unsigned)((d.tmB_rows + 31) / 32));
-    k_dense_convert<<<cg, cb, 0, st>>>(a, n, nb, d.Xt, d.n_pad, d.tmB_rows);
-    cudaError_t e = cudaGetLastError();
-    if (e) return e;
-    return cudaMemsetAsync(cost, 0, sizeof(long long) * (size_t)nb, st);
+    return launch_convert(d, a, n, nb, cost, st);
 }
 
 cudaError_t launch_dense_convert_x(const DenseDev &d, const float *x, int n, int nb, long long *cost,
                                    cudaStream_t st) {
-    dim3 cb(32, 8), cg((unsigned)(d.n_pad / 64), (unsigned)((d.tmB_rows + 31) / 32));
-    k_dense_convert_x<<<cg, cb, 0, st>>>(x, n, nb, d.Xt, d.n_pad, d.tmB_rows, cost);
-    return cudaGetLastError();
+    return launch_convert(d, x, n, nb, cost, st);
 }
 
 // Whole tiles one per CTA when they fit one wave of one CTA per SM.  With
@@ -897,19 +891,9 @@ cudaError_t launch_dense_gemm(const DenseDev &d, int nb, long long *cost, cudaSt
         return cudaErrorInvalidValue;
     // launched to overlap the packing kernel before it in the stream (it
     // waits for that kernel's writes where it needs them)
-    cudaLaunchConfig_t lc = {};
-    lc.gridDim = dim3((unsigned)grid);
-    lc.blockDim = dim3(kDenseThreads);
-    lc.dynamicSmemBytes = smem;
-    lc.stream = st;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
-    lc.attrs = at;
-    lc.numAttrs = 1;
-    return cudaLaunchKernelEx(&lc, k_dense_eval, d.tmA, d.tmB, d.target, d.wgt, d.unit_w ? 1 : 0, p, tmem_cols, nb,
-                              reinterpret_cast<unsigned long long *>(cost), d.ptgt, d.pmask, d.part_cnt,
-                              d.errflag);
+    return launch_pdl(k_dense_eval, dim3((unsigned)grid), dim3(kDenseThreads), smem, st, d.tmA, d.tmB, d.target, d.wgt,
+                      d.unit_w ? 1 : 0, p, tmem_cols, nb, reinterpret_cast<unsigned long long *>(cost), d.ptgt, d.pmask,
+                      d.part_cnt, d.errflag);
 }
 
 size_t smem_max_dense() { return dense_smem_bytes(256); }

@@ -682,6 +682,7 @@ bool build_solo(int32_t n, int64_t m, int32_t kfix, int32_t max_len, int32_t max
     V.n_multi = sh.n_multi;
     V.n_wide = sh.n_wide;
     V.n_mtask = sh.n_mtask;
+    V.rows = (int)(sh.lit_rows + sh.occ_rows);
     return true;
 }
 
@@ -755,23 +756,24 @@ cudaError_t launch_solo_steps(const SoloDev &V, const DevInst &I, const DevState
 
 // Whether `steps` steps are taken faster by this kernel than by the per-pass
 // kernels, from what both measured on one GB300 (microseconds a step).  A
-// block takes 1 + 0.24 per thousand literals of 3-literal clauses (n=301
-// 1.9, n=5000 14.5), 0.33 where lengths differ (weighted Zipf n=3000 20.6)
-// and 0.43 with clauses of more than 32 literals (PHP(40) 30), one wave of
-// SMs at a time (n=5000, B=256: 29), and gathers and scatters its column of
-// the state once a call (7e-5 per variable and restart: n=5000, B=256 90).
-// The two passes take 16 (launches and dependent latency), 1.4 per million
-// literal evaluations (n=5000, B=256: 43) and, for clauses that are not all
-// of three literals, 0.2 per literal of the longest (PHP(40), B=1: 25) or,
-// with four or more restarts, 4 + 0.35 (the ordering principle on 31
-// elements, B=8: 31 against 19 here).  slack: factor allowed to this kernel.
+// block takes 1 + 0.0115 per list row (n=301 1.9, n=5000 14.5, ordering
+// principle on 31 elements 18.9), 1.4 times that with variables a warp
+// combines (weighted Zipf n=3000 20.6) and 1.6 with clauses of more than 32
+// literals (PHP(40) 30), one wave of SMs at a time (n=5000, B=256: 29), and
+// once a call loads its lists and gathers and scatters its column of the
+// state (8 + 7e-5 per variable and restart: n=5000, B=256 90).  The two passes take 10 (dependent latency;
+// n=5000, B=1: 10.7), 1.5 per million literal evaluations (n=5000, B=256:
+// 36), for clauses that are not all of three literals 2 + 0.15 per literal of
+// the longest, or 0.3 with four or more restarts (ordering principle, B=8:
+// 20.5), and then 12 for a launch of heavy variables (Zipf n=3000, B=4: 37).
+// slack: factor allowed to this kernel.
 bool solo_pays(const SoloDev &V, const DevInst &I, int64_t nnz, int max_len, int64_t steps, double slack) {
     const double waves = (I.B + V.sms - 1) / V.sms;
-    const double per_lit = V.kind == 0 ? 0.24e-3 : V.kind == 1 ? 0.33e-3 : 0.43e-3;
-    const double solo = 1.0 + per_lit * (double)nnz * waves;
-    const double passes = 16.0 + 1.4e-6 * (double)nnz * I.B +
-                          (I.kfix == 3 ? 0.0 : I.B < 4 ? 0.2 * max_len : 4.0 + 0.35 * max_len);
-    return (double)steps * solo + 7e-5 * (double)I.n * I.B <= slack * (double)std::max<int64_t>(steps, 1) * passes;
+    const double solo = 1.0 + 0.0115 * V.rows * waves * (V.n_wide > 0 ? 1.4 : 1.0) * (V.kind == 2 ? 1.6 : 1.0);
+    const double passes = 10.0 + 1.5e-6 * (double)nnz * I.B +
+                          (I.kfix == 3 ? 0.0 : 2.0 + (I.B < 4 ? 0.15 : 0.3) * max_len) +
+                          (I.n_heavy > 0 && I.B >= 4 ? 12.0 : 0.0);
+    return (double)steps * solo + 8.0 + 7e-5 * (double)I.n * I.B <= slack * (double)std::max<int64_t>(steps, 1) * passes;
 }
 
 }  // namespace msat

@@ -24,6 +24,7 @@
 #include <algorithm>
 
 #include "msat_internal.cuh"
+#include "pdl.cuh"
 #include "step_math.cuh"
 
 namespace msat {
@@ -38,40 +39,63 @@ __device__ __forceinline__ uint64_t splitmix64_at(uint64_t seed, uint64_t c) {
 }
 
 // --------------------------------------------------------- vector access
-// VW floats at p (16-byte aligned for VW >= 4): read-only (nc) loads,
-// coherent loads, streaming (evict-first) loads and stores.  Streaming is
-// used for data touched once per pass, so the gathered rows of t, the unsat
-// bits and the f store keep their L2 lines.
+// VW floats at p (16-byte aligned for VW >= 4): plain and streaming
+// (evict-first) loads and stores.  Streaming is used for data touched once
+// per pass, so the gathered rows of t, the unsat bits and the f store keep
+// their L2 lines.  Everything loaded here is written by the kernel before in
+// the stream, which may still run when this one starts (pdl.cuh): the loads
+// are volatile so that none moves above the wait, and not read-only-cache
+// loads, which a write during the kernel's life would break.
 
-template <int VW>
-__device__ __forceinline__ void ldv(const float *__restrict__ p, float (&o)[VW]) {
-    if constexpr (VW >= 4) {
-#pragma unroll
-        for (int k = 0; k < VW / 4; ++k) {
-            const float4 v = __ldg(reinterpret_cast<const float4 *>(p) + k);
-            o[4 * k] = v.x; o[4 * k + 1] = v.y; o[4 * k + 2] = v.z; o[4 * k + 3] = v.w;
-        }
-    } else if constexpr (VW == 2) {
-        const float2 v = __ldg(reinterpret_cast<const float2 *>(p));
-        o[0] = v.x; o[1] = v.y;
-    } else {
-        o[0] = __ldg(p);
-    }
+__device__ __forceinline__ float4 ld4(const float4 *p) {
+    float4 v;
+    asm volatile("ld.global.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ float4 ld4_stream(const float4 *p) {
+    float4 v;
+    asm volatile("ld.global.cs.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ float2 ld2(const float2 *p) {
+    float2 v;
+    asm volatile("ld.global.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ float2 ld2_stream(const float2 *p) {
+    float2 v;
+    asm volatile("ld.global.cs.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ float ld1(const float *p) {
+    float v;
+    asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ float ld1_stream(const float *p) {
+    float v;
+    asm volatile("ld.global.cs.f32 %0, [%1];" : "=f"(v) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ uint32_t ld1(const uint32_t *p) {
+    uint32_t v;
+    asm volatile("ld.global.u32 %0, [%1];" : "=r"(v) : "l"(p));
+    return v;
 }
 
 template <int VW>
-__device__ __forceinline__ void ldv_rw(const float *p, float (&o)[VW]) {
+__device__ __forceinline__ void ldv(const float *p, float (&o)[VW]) {
     if constexpr (VW >= 4) {
 #pragma unroll
         for (int k = 0; k < VW / 4; ++k) {
-            const float4 v = reinterpret_cast<const float4 *>(p)[k];
+            const float4 v = ld4(reinterpret_cast<const float4 *>(p) + k);
             o[4 * k] = v.x; o[4 * k + 1] = v.y; o[4 * k + 2] = v.z; o[4 * k + 3] = v.w;
         }
     } else if constexpr (VW == 2) {
-        const float2 v = *reinterpret_cast<const float2 *>(p);
+        const float2 v = ld2(reinterpret_cast<const float2 *>(p));
         o[0] = v.x; o[1] = v.y;
     } else {
-        o[0] = *p;
+        o[0] = ld1(p);
     }
 }
 
@@ -80,14 +104,14 @@ __device__ __forceinline__ void ldv_stream(const float *p, float (&o)[VW]) {
     if constexpr (VW >= 4) {
 #pragma unroll
         for (int k = 0; k < VW / 4; ++k) {
-            const float4 v = __ldcs(reinterpret_cast<const float4 *>(p) + k);
+            const float4 v = ld4_stream(reinterpret_cast<const float4 *>(p) + k);
             o[4 * k] = v.x; o[4 * k + 1] = v.y; o[4 * k + 2] = v.z; o[4 * k + 3] = v.w;
         }
     } else if constexpr (VW == 2) {
-        const float2 v = __ldcs(reinterpret_cast<const float2 *>(p));
+        const float2 v = ld2_stream(reinterpret_cast<const float2 *>(p));
         o[0] = v.x; o[1] = v.y;
     } else {
-        o[0] = __ldcs(p);
+        o[0] = ld1_stream(p);
     }
 }
 
@@ -375,7 +399,7 @@ __device__ __forceinline__ void occ_accumulate(const DevInst &I, const DevState 
         uint32_t wd[C];
 #pragma unroll
         for (int u = 0; u < C; ++u) {
-            wd[u] = ok[u] ? __ldg(ubits_word(I, S.ubits, o[u], col)) : 0u;
+            wd[u] = ok[u] ? ld1(ubits_word(I, S.ubits, o[u], col)) : 0u;
             if (dense && ok[u]) fetch_f<VW, KFIX>(I, kfix, tcur, o[u], ox[u], own_var, col, v[u]);
         }
 #pragma unroll
@@ -556,6 +580,7 @@ __device__ __forceinline__ void forward_body(const DevInst &I, const float *__re
     extern __shared__ float4 dyn_smem[];
     __shared__ int s_last;
 
+    grid_dep_wait();
     const int B = I.B;
     const int G = B / VW;
     const long long steps = D.sc->steps_done;
@@ -725,6 +750,11 @@ __device__ __forceinline__ void forward_body(const DevInst &I, const float *__re
     if (threadIdx.x == 0) s_last = (atomicAdd(&D.sc->counter, 1u) == nblk - 1);
     __syncthreads();
     if (!s_last) return;
+    // the variable pass's blocks may start: every other block is done, so
+    // they spread over empty SMs (started before the blocks' sums they crowd
+    // onto the SMs that were free first: weighted Zipf n=20000, B=1 21 -> 36
+    // us a step)
+    grid_dep_launch();
     __threadfence();
     // the last block's finish: every block's additions are complete (fence
     // before the counter).  The last thread makes the step's Adam scalars
@@ -870,12 +900,11 @@ static cudaError_t launch_forward_vw(const DevInst &I, const DevState &S, const 
     // one instantiation per common clause length: all literals, then all rows
     // of a clause in flight (k = 5, n=30011, m=639234, B=64: 144 -> 97 us)
     switch (I.kfix) {
-        case 3: k_forward<VW, 3><<<blocks, kThreads, smem, st>>>(I, S.t0, S.t1, t_ovr, D, S.ubits, S.fstore, mode); break;
-        case 4: k_forward<VW, 4><<<blocks, kThreads, smem, st>>>(I, S.t0, S.t1, t_ovr, D, S.ubits, S.fstore, mode); break;
-        case 5: k_forward<VW, 5><<<blocks, kThreads, smem, st>>>(I, S.t0, S.t1, t_ovr, D, S.ubits, S.fstore, mode); break;
-        default: k_forward<VW, 0><<<blocks, kThreads, smem, st>>>(I, S.t0, S.t1, t_ovr, D, S.ubits, S.fstore, mode); break;
+        case 3: return launch_pdl(k_forward<VW, 3>, blocks, kThreads, smem, st, I, S.t0, S.t1, t_ovr, D, S.ubits, S.fstore, mode);
+        case 4: return launch_pdl(k_forward<VW, 4>, blocks, kThreads, smem, st, I, S.t0, S.t1, t_ovr, D, S.ubits, S.fstore, mode);
+        case 5: return launch_pdl(k_forward<VW, 5>, blocks, kThreads, smem, st, I, S.t0, S.t1, t_ovr, D, S.ubits, S.fstore, mode);
+        default: return launch_pdl(k_forward<VW, 0>, blocks, kThreads, smem, st, I, S.t0, S.t1, t_ovr, D, S.ubits, S.fstore, mode);
     }
-    return cudaGetLastError();
 }
 
 cudaError_t launch_forward(const DevInst &I0, const DevState &S, const DevStep &D, int mode,
@@ -953,6 +982,7 @@ __device__ __forceinline__ void heavy_body(const DevInst &I, const DevState &S, 
     const int vend = __ldg(I.voff + i + 1);
     const int cb = __ldg(I.voff + i) + (int)(cidx - c0) * kChunk;
     const int cn = min(kChunk, vend - cb);  // occurrences in this chunk
+    grid_dep_wait();  // the list loads above need nothing of the clause pass
     const float *tcur;
     float *tnext;
     step_buffers(S, D, mode, t_ovr, tcur, tnext);
@@ -1003,6 +1033,7 @@ __device__ __forceinline__ void heavy_body(const DevInst &I, const DevState &S, 
         if (cidx == c0 && lane < VW && D.improved[col + lane]) S.bestx[q0 + lane] = S.x[q0 + lane] > 0.0f;
         return;
     }
+    grid_dep_launch();
     int last = 1;
     if (nch > 1) {
         if (lane == 0) {
@@ -1070,14 +1101,11 @@ __device__ __forceinline__ void vars_body(const DevInst &I, const DevState &S, c
     __shared__ int s_wtot[kThreads / 32];
     const int B = I.B;
     const int kfix = KFIX > 0 ? KFIX : I.kfix;
-    const float *tcur;
-    float *tnext;
-    step_buffers(S, D, mode, t_ovr, tcur, tnext);
     if (blk >= I.n_lblk) {  // the blocks behind the variables'
+        grid_dep_wait();
         if (mode == BWD_UPDATE) reduce_loss(D, B, blk - I.n_lblk);
         return;
     }
-    const AdamView A = adam_view(D.sc);
     float *s_leaf = reinterpret_cast<float *>(dyn_smem);
     const int2 rg = I.lblk[blk];
     const int v0 = rg.x, nv = rg.y - rg.x;  // nv <= kThreads
@@ -1107,6 +1135,11 @@ __device__ __forceinline__ void vars_body(const DevInst &I, const DevState &S, c
     if (threadIdx.x < nv) s_lpre[threadIdx.x] = before + inc - nl;
     if (threadIdx.x == nv - 1) s_lpre[nv] = before + inc;
     __syncthreads();
+    grid_dep_wait();  // the offsets above need nothing of the clause pass
+    const float *tcur;
+    float *tnext;
+    step_buffers(S, D, mode, t_ovr, tcur, tnext);
+    const AdamView A = adam_view(D.sc);
 
     const int GS = B / VS;
     const int gshift = __ffs(GS) - 1;  // GS is a power of two <= kThreads
@@ -1136,7 +1169,7 @@ __device__ __forceinline__ void vars_body(const DevInst &I, const DevState &S, c
         const int64_t q0 = (int64_t)i * B + col;
         if (mode == BWD_BITS_ONLY) {
             float xv[VS];
-            ldv_rw<VS>(S.x + q0, xv);
+            ldv<VS>(S.x + q0, xv);
 #pragma unroll
             for (int e = 0; e < VS; ++e)
                 if (D.improved[col + e]) S.bestx[q0 + e] = xv[e] > 0.0f;
@@ -1184,6 +1217,7 @@ __device__ __forceinline__ void vars_body(const DevInst &I, const DevState &S, c
             stv<VS>(s_leaf + (int64_t)ti * B + col, leaf);
         }
     }
+    grid_dep_launch();
     if (mode == BWD_BITS_ONLY || nleaves == nv) return;  // uniform: no variable has two leaves
     __syncthreads();
     for (int t = threadIdx.x; t < ntasks; t += kThreads) {
@@ -1201,7 +1235,8 @@ __device__ __forceinline__ void vars_body(const DevInst &I, const DevState &S, c
         for (int e = 0; e < VS; ++e) lc[e].init();
         for (int l = 0; l < nleaf; ++l) {
             float v[VS];
-            ldv_rw<VS>(s_leaf + (int64_t)(ti + l) * B + col, v);
+#pragma unroll
+            for (int e = 0; e < VS; ++e) v[e] = s_leaf[(ti + l) * B + col + e];
 #pragma unroll
             for (int e = 0; e < VS; ++e) lc[e].push(v[e]);
         }
@@ -1268,22 +1303,19 @@ static cudaError_t launch_backward_k(const DevInst &I, const DevState &S, const 
         if constexpr (STORE && VU <= 2 && VS <= 2) {
             // one launch where that keeps the light blocks' 64-register,
             // four-blocks-per-SM shape without spills
-            k_backward_mixed<VS, VU, KFIX, STORE, 4><<<(unsigned)(hblocks + lblocks), kThreads, smem, st>>>(
-                I, S, D, mode, t_ovr, gscale, grad_out, (int)hblocks);
-            return cudaGetLastError();
+            return launch_pdl(k_backward_mixed<VS, VU, KFIX, STORE, 4>, (unsigned)(hblocks + lblocks), kThreads, smem, st,
+                              I, S, D, mode, t_ovr, gscale, grad_out, (int)hblocks);
         }
-        k_backward_heavy<VU, KFIX, STORE><<<(unsigned)hblocks, kThreads, 0, st>>>(I, S, D, mode, t_ovr,
-                                                                                   gscale, grad_out);
-        const cudaError_t e = cudaGetLastError();
+        const cudaError_t e = launch_pdl(k_backward_heavy<VU, KFIX, STORE>, (unsigned)hblocks, kThreads, 0, st, I, S, D, mode,
+                                         t_ovr, gscale, grad_out);
         if (e) return e;
     }
     if constexpr ((STORE && VS <= 4) || VS <= 2)
-        k_backward_light_occ4<VS, KFIX, STORE><<<(unsigned)lblocks, kThreads, smem, st>>>(I, S, D, mode, t_ovr,
-                                                                                      gscale, grad_out);
+        return launch_pdl(k_backward_light_occ4<VS, KFIX, STORE>, (unsigned)lblocks, kThreads, smem, st, I, S, D, mode, t_ovr,
+                          gscale, grad_out);
     else
-        k_backward_light<VS, KFIX, STORE><<<(unsigned)lblocks, kThreads, smem, st>>>(I, S, D, mode, t_ovr,
-                                                                                     gscale, grad_out);
-    return cudaGetLastError();
+        return launch_pdl(k_backward_light<VS, KFIX, STORE>, (unsigned)lblocks, kThreads, smem, st, I, S, D, mode, t_ovr,
+                          gscale, grad_out);
 }
 
 template <int VS, int VU>
@@ -1369,12 +1401,11 @@ static cudaError_t launch_batch_bwd(const SlotDesc *slots, int nslot, const int 
                                     int heavy_total, const int *light_start, int light_total,
                                     size_t smem, cudaStream_t st) {
     if (heavy_total > 0) {
-        k_backward_heavy_batch<VU><<<(unsigned)heavy_total, kThreads, 0, st>>>(slots, heavy_start, nslot);
-        const cudaError_t e = cudaGetLastError();
+        const cudaError_t e =
+            launch_pdl(k_backward_heavy_batch<VU>, (unsigned)heavy_total, kThreads, 0, st, slots, heavy_start, nslot);
         if (e) return e;
     }
-    k_backward_light_batch<VS><<<(unsigned)light_total, kThreads, smem, st>>>(slots, light_start, nslot);
-    return cudaGetLastError();
+    return launch_pdl(k_backward_light_batch<VS>, (unsigned)light_total, kThreads, smem, st, slots, light_start, nslot);
 }
 
 cudaError_t launch_step_batch(const SlotDesc *slots, int nslot, const int *fwd_start, int fwd_total,
@@ -1382,13 +1413,13 @@ cudaError_t launch_step_batch(const SlotDesc *slots, int nslot, const int *fwd_s
                               int light_total, int B, int fwd_vw, int stage_vw, int task_cap,
                               cudaStream_t st) {
     if (nslot <= 0) return cudaSuccess;
+    cudaError_t e;
     switch (fwd_vw) {
-        case 8: k_forward_batch<8><<<(unsigned)fwd_total, kThreads, fwd_smem<8>(B), st>>>(slots, fwd_start, nslot); break;
-        case 4: k_forward_batch<4><<<(unsigned)fwd_total, kThreads, fwd_smem<4>(B), st>>>(slots, fwd_start, nslot); break;
-        case 2: k_forward_batch<2><<<(unsigned)fwd_total, kThreads, fwd_smem<2>(B), st>>>(slots, fwd_start, nslot); break;
-        default: k_forward_batch<1><<<(unsigned)fwd_total, kThreads, fwd_smem<1>(B), st>>>(slots, fwd_start, nslot); break;
+        case 8: e = launch_pdl(k_forward_batch<8>, (unsigned)fwd_total, kThreads, fwd_smem<8>(B), st, slots, fwd_start, nslot); break;
+        case 4: e = launch_pdl(k_forward_batch<4>, (unsigned)fwd_total, kThreads, fwd_smem<4>(B), st, slots, fwd_start, nslot); break;
+        case 2: e = launch_pdl(k_forward_batch<2>, (unsigned)fwd_total, kThreads, fwd_smem<2>(B), st, slots, fwd_start, nslot); break;
+        default: e = launch_pdl(k_forward_batch<1>, (unsigned)fwd_total, kThreads, fwd_smem<1>(B), st, slots, fwd_start, nslot); break;
     }
-    cudaError_t e = cudaGetLastError();
     if (e) return e;
     const size_t smem = light_smem_bytes(task_cap, stage_vw);
     const int vu = update_vw(B);

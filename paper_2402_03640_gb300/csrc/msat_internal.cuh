@@ -117,6 +117,7 @@ struct SoloDev {
     int n_multi = 0;   // variables of several leaves
     int n_wide = 0;    // of these, the ones a warp combines (first)
     int n_mtask = 0;   // leaf tasks of the variables of several leaves
+    int rows = 0;      // rows of both lists
     int kind = 0;      // 0: every clause has 3 literals, 1: at most 32, 2: any length
     bool pairs = false;          // w*f held as {q, -q}
     int sms = 1;                 // multiprocessors of the device
