@@ -35,6 +35,7 @@ int cuda_fail(cudaError_t e, const char *what) {
 using namespace msat;
 
 #include "ctx.cuh"
+#include "dev_cnf.cuh"
 #include "host_cnf.cuh"
 
 #include <nvtx3/nvToolsExt.h>
@@ -163,10 +164,16 @@ int msat::ctx_create(msat_ctx **out, int32_t n_vars, int64_t n_clauses, const in
         !(cfg.eps >= 0))
         return fail(MSAT_EINVAL, "msat_create: Adam settings out of range");
     const int64_t m = n_clauses;
-    // checks, canonical clauses and the transposed CSR (host_cnf.cu, on the
-    // host's cores)
+    // checks, canonical clauses and the transposed CSR: on the device for
+    // large clean instances (dev_cnf.cu), else on the host's cores
+    // (host_cnf.cu); the same arrays
+    const bool auto_store = (double)m * cfg.restarts * sizeof(float) <= 8.0 * (1 << 30) || cfg.restarts <= 2;
+    const bool use_fstore = cfg.f_mode == MSAT_F_STORE || (cfg.f_mode == MSAT_F_AUTO && auto_store);
     HostCnf hc;
-    {
+    DevCnf dv;
+    bool on_dev = !pool_alloc && use_fstore && m > 0 && dev_cnf_worth(n_vars, m, clause_off[m]) &&
+                  dv.check(n_vars, m, clause_off, lits, weights, stream, hc);
+    if (!on_dev) {
         const int hrc = build_host_cnf(n_vars, m, clause_off, lits, weights, hc);
         if (hrc) return hrc;
     }
@@ -240,8 +247,7 @@ int msat::ctx_create(msat_ctx **out, int32_t n_vars, int64_t n_clauses, const in
     // the stored w*f costs one [m][B] write and one row gather per
     // occurrence; recomputing gathers the unsat bits and every literal's row
     // of t, which measured slower even when the store does not fit in L2
-    const bool auto_store = (double)m * B * sizeof(float) <= 8.0 * (1 << 30) || B <= 2;
-    const bool use_fstore = cfg.f_mode == MSAT_F_STORE || (cfg.f_mode == MSAT_F_AUTO && auto_store);
+    // (auto_store above)
     // recomputing f of 3-literal clauses reads the other two literals from an
     // expanded occurrence record streamed with the occurrence list
     const bool expand = cfg.f_mode == MSAT_F_EXPANDED ||
@@ -255,13 +261,20 @@ int msat::ctx_create(msat_ctx **out, int32_t n_vars, int64_t n_clauses, const in
                             (cfg.row_order == 2 ||
                              (cfg.row_order == 0 && (double)m * B * sizeof(float) > 32.0 * (1 << 20)));
     RowOrder ro;
-    if (block_rows) {
+    if (on_dev && ((block_rows && !dv.rows(lblk)) || !dv.occurrences())) {
+        // a row group past the device sort, or no memory: the host path after
+        // all (every number above is the same there)
+        on_dev = false;
+        const int hrc = build_host_cnf(n_vars, m, clause_off, lits, weights, hc);
+        if (hrc) return hrc;
+    }
+    if (block_rows && !on_dev) {
         const int rrc = build_block_rows(n_vars, m, kfix, coff, lit, weights, lblk, ro);
         if (rrc) return rrc;
     }
     // a forced row order is a request for the per-pass kernels
     SoloHost solo;
-    bool use_solo = cfg.row_order != 2 && build_solo(n_vars, m, kfix, max_len, max_deg, hc, solo);
+    bool use_solo = cfg.row_order != 2 && !on_dev && build_solo(n_vars, m, kfix, max_len, max_deg, hc, solo);
     if (use_solo) {
         int dev = 0;
         cudaGetDevice(&dev);
@@ -282,7 +295,7 @@ int msat::ctx_create(msat_ctx **out, int32_t n_vars, int64_t n_clauses, const in
     // the serving engine runs such an instance on that kernel alone: its
     // context holds none of the per-pass kernels' lists and buffers
     const bool solo_only = use_solo && pool_alloc;
-    if (!solo_only) scatter_occurrences(n_vars, m, hc, block_rows ? &ro.row : nullptr);
+    if (!solo_only && !on_dev) scatter_occurrences(n_vars, m, hc, block_rows ? &ro.row : nullptr);
     std::vector<int64_t> solo_w;
     if (use_solo && weights && !solo.slot.empty()) {
         solo_w.resize((size_t)m);
@@ -338,19 +351,33 @@ int msat::ctx_create(msat_ctx **out, int32_t n_vars, int64_t n_clauses, const in
         rc = dalloc_t(c, &(ptr), (size_t)(count));     \
         if (rc) { free_all(c); delete c; return rc; }  \
     } while (0)
-    if (!solo_only) {
+    if (on_dev) {
+        auto take = [&](auto *&dst, auto *&src, int64_t count) {
+            dst = DevCnf::release(src);
+            c->allocs.push_back(dst);
+            c->device_bytes += std::max<int64_t>(16, count * (int64_t)sizeof(*dst));
+        };
+        take(d_coff, dv.coff, m + 1);
+        take(d_lit, dv.lit, nnz);
+        take(d_voff, dv.voff, (int64_t)n_vars + 1);
+        take(d_occ, dv.occ, nnz);
+        if (weights) take(d_w, dv.w, m);
+        if (block_rows) take(d_plit, dv.plit, nnz);
+        if (dv.pcoff) take(d_pcoff, dv.pcoff, m + 1);
+        if (dv.pw) take(d_pw, dv.pw, m);
+    } else if (!solo_only) {
         TRY_ALLOC(d_coff, m + 1);
         TRY_ALLOC(d_lit, nnz);
         TRY_ALLOC(d_voff, (int64_t)n_vars + 1);
         TRY_ALLOC(d_occ, nnz);
     }
-    if (weights) TRY_ALLOC(d_w, m);
+    if (weights && !on_dev) TRY_ALLOC(d_w, m);
     TRY_ALLOC(d_hvar, (int64_t)hvar.size());
     TRY_ALLOC(d_hch, (int64_t)hchunk0.size());
     TRY_ALLOC(d_hofc, std::max<int64_t>(1, hchunk0.back()));
     TRY_ALLOC(d_lblk, (int64_t)lblk.size());
     if (expand) TRY_ALLOC(d_occx, nnz);
-    if (block_rows) {
+    if (block_rows && !on_dev) {
         TRY_ALLOC(d_plit, nnz);
         if (kfix == 0) TRY_ALLOC(d_pcoff, m + 1);
         if (weights) TRY_ALLOC(d_pw, m);
@@ -442,11 +469,12 @@ int msat::ctx_create(msat_ctx **out, int32_t n_vars, int64_t n_clauses, const in
     sc.loss_norm = cfg.loss_norm;
     std::vector<long long> best((size_t)B, (long long)wsum);
     cudaError_t e = cudaSuccess;
-    if (!e && !solo_only) e = up(d_coff, coff.data(), sizeof(int32_t) * coff.size());
-    if (!e && !solo_only) e = up(d_lit, lit.data(), sizeof(int32_t) * lit.size());
-    if (!e && weights) e = up(d_w, weights, sizeof(int64_t) * (size_t)m);
-    if (!e && !solo_only) e = up(d_voff, voff.data(), sizeof(int32_t) * voff.size());
-    if (!e && !solo_only) e = up(d_occ, occ.data(), sizeof(int32_t) * occ.size());
+    const bool lists = !solo_only && !on_dev;
+    if (!e && lists) e = up(d_coff, coff.data(), sizeof(int32_t) * coff.size());
+    if (!e && lists) e = up(d_lit, lit.data(), sizeof(int32_t) * lit.size());
+    if (!e && weights && !on_dev) e = up(d_w, weights, sizeof(int64_t) * (size_t)m);
+    if (!e && lists) e = up(d_voff, voff.data(), sizeof(int32_t) * voff.size());
+    if (!e && lists) e = up(d_occ, occ.data(), sizeof(int32_t) * occ.size());
     if (!e) e = up(d_hvar, hvar.data(), sizeof(int32_t) * hvar.size());
     if (!e) e = up(d_hch, hchunk0.data(), sizeof(int32_t) * hchunk0.size());
     // the heavy variable of every chunk (one load per chunk block)
@@ -456,9 +484,9 @@ int msat::ctx_create(msat_ctx **out, int32_t n_vars, int64_t n_clauses, const in
     if (!e) e = up(d_hofc, hofc.data(), sizeof(int32_t) * hofc.size());
     if (!e) e = up(d_lblk, lblk.data(), sizeof(int2) * lblk.size());
     if (!e && expand) e = up(d_occx, occx.data(), sizeof(int2) * occx.size());
-    if (!e && block_rows) e = up(d_plit, ro.plit.data(), sizeof(int32_t) * ro.plit.size());
-    if (!e && d_pcoff) e = up(d_pcoff, ro.pcoff.data(), sizeof(int32_t) * ro.pcoff.size());
-    if (!e && d_pw) e = up(d_pw, ro.pw.data(), sizeof(int64_t) * ro.pw.size());
+    if (!e && block_rows && !on_dev) e = up(d_plit, ro.plit.data(), sizeof(int32_t) * ro.plit.size());
+    if (!e && d_pcoff && !on_dev) e = up(d_pcoff, ro.pcoff.data(), sizeof(int32_t) * ro.pcoff.size());
+    if (!e && d_pw && !on_dev) e = up(d_pw, ro.pw.data(), sizeof(int64_t) * ro.pw.size());
     if (!e && use_solo) e = up(d_slists, solo.lists.data(), solo.lists.size());
     if (!e && use_solo) e = up(d_sperm, solo.perm.data(), sizeof(int32_t) * solo.perm.size());
     if (!e && d_sw) e = up(d_sw, solo_w.data(), sizeof(int64_t) * solo_w.size());
@@ -709,6 +737,16 @@ static int dense_setup(msat_ctx *c) {
     if ((rc = dalloc_t(c, &d.target, (size_t)d.m_pad))) return rc;
     if ((rc = dalloc_t(c, &d.wgt, (size_t)d.m_pad))) return rc;
     if ((rc = dalloc_t(c, &d.errflag, 1))) return rc;
+    // clause lengths of an instance prepared on the device (no clause of it
+    // holds x and not x)
+    if (c->clen.empty() && c->m > 0) {
+        std::vector<int32_t> off((size_t)c->m + 1);
+        MSAT_CUDA_TRY(cudaMemcpyAsync(off.data(), c->I.coff, sizeof(int32_t) * off.size(), cudaMemcpyDeviceToHost, c->stream));
+        MSAT_CUDA_TRY(cudaStreamSynchronize(c->stream));
+        c->clen.resize((size_t)c->m);
+        for (int64_t j = 0; j < c->m; ++j) c->clen[(size_t)j] = off[(size_t)j + 1] - off[(size_t)j];
+        c->taut.assign((size_t)c->m, 0);
+    }
     std::vector<float> tgt((size_t)d.m_pad, std::nanf(""));
     std::vector<uint32_t> w32((size_t)d.m_pad, 0u);
     d.unit_w = true;
@@ -929,9 +967,24 @@ extern "C" int msat_best(msat_ctx *c, uint8_t *assign01, int64_t *best_cost) {
     if (best_cost)
         MSAT_CUDA_TRY(cudaMemcpyAsync(best_cost, c->D.best, sizeof(int64_t) * (size_t)c->B,
                                       cudaMemcpyDeviceToHost, c->stream));
+    const size_t nB = (size_t)c->n * c->B;
+    if (assign01 && c->B > 1 && nB >= (1 << 16)) {
+        // transposed on the device into the tanh buffer that the next step
+        // writes; from n=5000, B=256 (0.86 ms -> @BEST@) on, the host loop's
+        // strided bytes cost more than the kernel and the copy
+        StepScalars sc;
+        MSAT_CUDA_TRY(cudaMemcpyAsync(&sc, c->D.sc, sizeof(sc), cudaMemcpyDeviceToHost, c->stream));
+        MSAT_CUDA_TRY(cudaStreamSynchronize(c->stream));
+        uint8_t *tr = reinterpret_cast<uint8_t *>((sc.steps_done & 1) ? c->S.t0 : c->S.t1);
+        const cudaError_t e = launch_transpose_u8(c->S.bestx, tr, c->n, c->B, c->stream);
+        if (e) return cuda_fail(e, "msat_best: transposition");
+        MSAT_CUDA_TRY(cudaMemcpyAsync(assign01, tr, nB, cudaMemcpyDeviceToHost, c->stream));
+        MSAT_CUDA_TRY(cudaStreamSynchronize(c->stream));
+        return MSAT_OK;
+    }
     std::vector<uint8_t> tmp;
     if (assign01) {
-        tmp.resize((size_t)c->n * c->B);
+        tmp.resize(nB);
         MSAT_CUDA_TRY(cudaMemcpyAsync(tmp.data(), c->S.bestx, tmp.size(), cudaMemcpyDeviceToHost,
                                       c->stream));
     }

@@ -1,0 +1,59 @@
+// Device-side CNF preparation of msat_create (dev_cnf.cu).
+#pragma once
+
+#include <cuda_runtime.h>
+#include <stdint.h>
+
+#include <vector>
+
+#include "host_cnf.cuh"
+
+namespace msat {
+
+// The arrays of a checked CNF on the device, built there from the caller's
+// host arrays.  Owns them until release(); temporaries are freed in order on
+// the stream.
+struct DevCnf {
+    int32_t n = 0;
+    int64_t m = 0, nnz = 0;
+    int32_t kfix = 0;
+    cudaStream_t st = nullptr;
+    int32_t *coff = nullptr, *lit = nullptr, *voff = nullptr, *occ = nullptr;
+    int64_t *w = nullptr;
+    int32_t *row = nullptr;  // temporary: clause -> row of the store
+    int32_t *plit = nullptr, *pcoff = nullptr;
+    int64_t *pw = nullptr;
+
+    DevCnf() = default;
+    DevCnf(const DevCnf &) = delete;
+    DevCnf &operator=(const DevCnf &) = delete;
+    ~DevCnf();
+
+    // Checks and packs the clauses and makes the occurrence offsets; fills
+    // the sizes, kfix, max_len, max_deg, wsum, wor and voff of `out`.  False:
+    // the instance is for the host path (a violation, whose message that path
+    // gives; a repeated variable in a clause; a clause of more than 32
+    // literals; a variable of more than 1024 occurrences; no memory).
+    bool check(int32_t n_vars, int64_t n_clauses, const int64_t *off, const int32_t *lits, const int64_t *weights,
+               cudaStream_t stream, HostCnf &out);
+    // Rows of the store grouped by light block (RowOrder): row, plit, pcoff, pw.
+    bool rows(const std::vector<int2> &lblk);
+    // The occurrence list in (clause, position) order, with rows if rows() ran.
+    bool occurrences();
+    // Hands an array over to the caller.
+    template <typename T>
+    static T *release(T *&p) {
+        T *q = p;
+        p = nullptr;
+        return q;
+    }
+};
+
+// Instances worth the device path: below this many literals the host's cores
+// are as fast (3-SAT n=2e4: 2.2 ms either way), and small instances need the
+// host's clause list for the one-block-per-restart kernel.
+inline bool dev_cnf_worth(int32_t n, int64_t m, int64_t raw) {
+    return raw >= (1 << 19) && (m > 65534 || n > 32766);
+}
+
+}  // namespace msat

@@ -561,6 +561,31 @@ __device__ __forceinline__ int cost_replicas(int B) {
 // values a literal) leave the registers for it.
 __host__ __device__ constexpr int fwd_items(int VW, int KFIX) { return VW <= 4 && VW * KFIX <= 12 ? 2 : 1; }
 
+// out[cols][rows] = in[rows][cols] of bytes, 32 columns by 128 rows a block
+// through shared memory.
+__global__ void __launch_bounds__(kThreads)
+    k_transpose_u8(const uint8_t *__restrict__ in, uint8_t *__restrict__ out, int rows, int cols) {
+    __shared__ uint8_t s[128][33];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int c0 = blockIdx.y * 32;
+    for (int64_t r0 = (int64_t)blockIdx.x * 128; r0 < rows; r0 += (int64_t)gridDim.x * 128) {
+        for (int r = warp; r < 128; r += kThreads / 32)
+            if (r0 + r < rows && c0 + lane < cols) s[r][lane] = in[(r0 + r) * cols + c0 + lane];
+        __syncthreads();
+        for (int k = threadIdx.x; k < 128 * 32; k += kThreads) {
+            const int c = k >> 7, r = k & 127;
+            if (r0 + r < rows && c0 + c < cols) out[(int64_t)(c0 + c) * rows + r0 + r] = s[r][c];
+        }
+        __syncthreads();
+    }
+}
+
+cudaError_t launch_transpose_u8(const uint8_t *in, uint8_t *out, int rows, int cols, cudaStream_t st) {
+    const dim3 grid((unsigned)std::min(((int64_t)rows + 127) / 128, (int64_t)152 * 16), (unsigned)((cols + 31) / 32));
+    k_transpose_u8<<<grid, kThreads, 0, st>>>(in, out, rows, cols);
+    return cudaGetLastError();
+}
+
 // --------------------------------------------------------------- k_forward
 // One item = (clause j, restart group g of VW restarts).  For VW <= 4 the
 // grid-stride loop is unrolled by two (items base + lane and base + stride +

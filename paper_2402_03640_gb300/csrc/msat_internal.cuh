@@ -297,6 +297,7 @@ cudaError_t launch_backward(const DevInst &I, const DevState &S, const DevStep &
                             const float *t_override, const float *gscale, float *grad_out,
                             cudaStream_t st);
 cudaError_t launch_tanh(const float *x, float *t, int64_t count, cudaStream_t st);
+cudaError_t launch_transpose_u8(const uint8_t *in, uint8_t *out, int rows, int cols, cudaStream_t st);
 // Batched step over nslot instances (all with the same B and launch shape,
 // f stored by the clause pass; variable-length clause path): fwd_start / heavy_start / light_start are device int[nslot+1]
 // block prefixes; totals are the grid sizes.
