@@ -170,8 +170,8 @@ int msat::ctx_create(msat_ctx **out, int32_t n_vars, int64_t n_clauses, const in
     const bool auto_store = (double)m * cfg.restarts * sizeof(float) <= 8.0 * (1 << 30) || cfg.restarts <= 2;
     const bool use_fstore = cfg.f_mode == MSAT_F_STORE || (cfg.f_mode == MSAT_F_AUTO && auto_store);
     HostCnf hc;
-    DevCnf dv;
-    bool on_dev = !pool_alloc && use_fstore && m > 0 && dev_cnf_worth(n_vars, m, clause_off[m]) &&
+    DevCnf dv(pool_alloc);
+    bool on_dev = use_fstore && m > 0 && dev_cnf_worth(n_vars, m, clause_off[m]) &&
                   dv.check(n_vars, m, clause_off, lits, weights, stream, hc);
     if (!on_dev) {
         const int hrc = build_host_cnf(n_vars, m, clause_off, lits, weights, hc);
@@ -970,7 +970,7 @@ extern "C" int msat_best(msat_ctx *c, uint8_t *assign01, int64_t *best_cost) {
     const size_t nB = (size_t)c->n * c->B;
     if (assign01 && c->B > 1 && nB >= (1 << 16)) {
         // transposed on the device into the tanh buffer that the next step
-        // writes; from n=5000, B=256 (0.86 ms -> @BEST@) on, the host loop's
+        // writes; from n=5000, B=256 (0.86 ms -> 0.05) on, the host loop's
         // strided bytes cost more than the kernel and the copy
         StepScalars sc;
         MSAT_CUDA_TRY(cudaMemcpyAsync(&sc, c->D.sc, sizeof(sc), cudaMemcpyDeviceToHost, c->stream));

@@ -343,9 +343,12 @@ struct Temps {
     }
 };
 
+// An array that outlives the preparation.
 template <typename T>
-cudaError_t own(T **out, size_t count) {
-    const cudaError_t e = cudaMalloc(reinterpret_cast<void **>(out), std::max<size_t>(16, count * sizeof(T)));
+cudaError_t own(const DevCnf &d, T **out, size_t count) {
+    const size_t bytes = std::max<size_t>(16, count * sizeof(T));
+    const cudaError_t e = d.pool ? cudaMallocAsync(reinterpret_cast<void **>(out), bytes, d.st)
+                                 : cudaMalloc(reinterpret_cast<void **>(out), bytes);
     if (e != cudaSuccess) *out = nullptr;
     return e;
 }
@@ -355,7 +358,10 @@ cudaError_t own(T **out, size_t count) {
 DevCnf::~DevCnf() {
     // pending kernels may still use them: cudaFree waits for the device
     for (void *p : {(void *)coff, (void *)lit, (void *)voff, (void *)occ, (void *)w, (void *)plit, (void *)pcoff, (void *)pw})
-        if (p) cudaFree(p);
+        if (p) {
+            if (pool) cudaFreeAsync(p, st);
+            else cudaFree(p);
+        }
     if (row) cudaFreeAsync(row, st);
 }
 
@@ -370,10 +376,10 @@ bool DevCnf::check(int32_t n_vars, int64_t n_clauses, const int64_t *off, const 
     int64_t *d_off = nullptr;
     int32_t *d_raw = nullptr, *deg = nullptr, *part = nullptr;
     CnfStat *stat = nullptr;
-    cudaError_t e = own(&coff, (size_t)m + 1);
-    if (!e) e = own(&lit, (size_t)raw);
-    if (!e) e = own(&voff, (size_t)n + 1);
-    if (!e && weights) e = own(&w, (size_t)m);
+    cudaError_t e = own(*this, &coff, (size_t)m + 1);
+    if (!e) e = own(*this, &lit, (size_t)raw);
+    if (!e) e = own(*this, &voff, (size_t)n + 1);
+    if (!e && weights) e = own(*this, &w, (size_t)m);
     if (!e) e = T.get(&d_off, (size_t)m + 1);
     if (!e) e = T.get(&d_raw, (size_t)raw);
     if (!e) e = T.get(&deg, (size_t)n);
@@ -418,9 +424,9 @@ bool DevCnf::rows(const std::vector<int2> &lblk) {
     int32_t *vblk = nullptr, *group = nullptr, *count = nullptr, *start = nullptr, *cur = nullptr, *list = nullptr;
     int32_t *part = nullptr, *rlen = nullptr;
     CnfStat *stat = nullptr;
-    cudaError_t e = own(&plit, (size_t)nnz);
-    if (!e && kfix == 0) e = own(&pcoff, (size_t)m + 1);
-    if (!e && w) e = own(&pw, (size_t)m);
+    cudaError_t e = own(*this, &plit, (size_t)nnz);
+    if (!e && kfix == 0) e = own(*this, &pcoff, (size_t)m + 1);
+    if (!e && w) e = own(*this, &pw, (size_t)m);
     if (!e) e = cudaMallocAsync(reinterpret_cast<void **>(&row), sizeof(int32_t) * (size_t)m, st);
     if (!e) e = T.get(&d_lblk, (size_t)nb);
     if (!e) e = T.get(&vblk, (size_t)n);
@@ -466,7 +472,7 @@ bool DevCnf::rows(const std::vector<int2> &lblk) {
 bool DevCnf::occurrences() {
     Temps T(st);
     int32_t *cur = nullptr;
-    cudaError_t e = own(&occ, (size_t)nnz);
+    cudaError_t e = own(*this, &occ, (size_t)nnz);
     if (!e) e = T.get(&cur, (size_t)n);
     if (!e) e = cudaMemcpyAsync(cur, voff, sizeof(int32_t) * (size_t)n, cudaMemcpyDeviceToDevice, st);
     if (!e) {

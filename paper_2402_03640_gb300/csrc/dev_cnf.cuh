@@ -18,13 +18,14 @@ struct DevCnf {
     int64_t m = 0, nnz = 0;
     int32_t kfix = 0;
     cudaStream_t st = nullptr;
+    bool pool = false;  // arrays from the stream-ordered pool (contexts of the server)
     int32_t *coff = nullptr, *lit = nullptr, *voff = nullptr, *occ = nullptr;
     int64_t *w = nullptr;
     int32_t *row = nullptr;  // temporary: clause -> row of the store
     int32_t *plit = nullptr, *pcoff = nullptr;
     int64_t *pw = nullptr;
 
-    DevCnf() = default;
+    explicit DevCnf(bool pool_alloc) : pool(pool_alloc) {}
     DevCnf(const DevCnf &) = delete;
     DevCnf &operator=(const DevCnf &) = delete;
     ~DevCnf();
@@ -50,10 +51,11 @@ struct DevCnf {
 };
 
 // Instances worth the device path: below this many literals the host's cores
-// are as fast (3-SAT n=2e4: 2.2 ms either way), and small instances need the
-// host's clause list for the one-block-per-restart kernel.
+// are as fast, and an instance that may fit the one-block-per-restart kernel
+// (its 21 bytes a variable and 4 a clause within an SM's shared memory) needs
+// the host's clause list for that kernel's lists.
 inline bool dev_cnf_worth(int32_t n, int64_t m, int64_t raw) {
-    return raw >= (1 << 19) && (m > 65534 || n > 32766);
+    return raw >= (1 << 17) && 21LL * n + 4LL * m > 227 * 1024;
 }
 
 }  // namespace msat

@@ -680,17 +680,22 @@ extern "C" int msat_submit(msat_server *S, const msat_request *req, uint64_t *ti
     if (req->n_vars < 1 || m < 0 || req->steps < 0 || !req->clause_off)
         return fail(MSAT_EINVAL, "msat_submit: need n_vars >= 1, n_clauses >= 0, steps >= 0, clause_off");
     if (req->clause_off[0] != 0) return fail(MSAT_EINVAL, "msat_submit: clause_off[0] must be 0");
-    for (int64_t j = 0; j < m; ++j)
-        if (req->clause_off[j + 1] < req->clause_off[j])
-            return fail(MSAT_EINVAL, "msat_submit: clause_off is not non-decreasing");
+    // the checks as whole-array reductions without early exits (the compiler
+    // vectorises them)
+    int32_t bad = 0;
+    for (int64_t j = 0; j < m; ++j) bad |= req->clause_off[j + 1] < req->clause_off[j];
+    if (bad) return fail(MSAT_EINVAL, "msat_submit: clause_off is not non-decreasing");
     const int64_t nnz = req->clause_off[m];
     if (nnz > 0 && !req->lits) return fail(MSAT_EINVAL, "msat_submit: lits is NULL");
-    for (int64_t q = 0; q < nnz; ++q)
-        if (req->lits[q] == 0 || req->lits[q] > req->n_vars || req->lits[q] < -req->n_vars)
-            return fail(MSAT_EINVAL, "msat_submit: literal names no variable");
+    const int32_t n_vars = req->n_vars;
+    for (int64_t q = 0; q < nnz; ++q) {
+        const int32_t l = req->lits[q];
+        bad |= (l == 0) | (l > n_vars) | (l < -n_vars);
+    }
+    if (bad) return fail(MSAT_EINVAL, "msat_submit: literal names no variable");
     if (req->weights)
-        for (int64_t j = 0; j < m; ++j)
-            if (req->weights[j] < 1) return fail(MSAT_EINVAL, "msat_submit: weight below 1");
+        for (int64_t j = 0; j < m; ++j) bad |= req->weights[j] < 1;
+    if (bad) return fail(MSAT_EINVAL, "msat_submit: weight below 1");
     SrvRequest r;
     r.n = req->n_vars;
     r.m = m;

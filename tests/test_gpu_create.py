@@ -49,13 +49,13 @@ def _doubled(cnf):
     return Cnf(cnf.n, off, lits.astype(np.int32), cnf.weights)
 
 
-@pytest.mark.parametrize("maker,B", [("k3", 1), ("k3", 64), ("mixed", 2), ("mixed", 128)])
+@pytest.mark.parametrize("maker,B", [("k3_small", 1), ("k3", 1), ("k3", 64), ("mixed", 2), ("mixed", 128)])
 def test_device_and_host_preparation_agree(pkg, oracle, maker, B):
     """B=64 and 128 have the store's rows grouped by block."""
     import torch
-    cnf = uniform_ksat(60000, 258000, 3, seed=3) if maker == "k3" else _mixed(4)
+    cnf = _mixed(4) if maker == "mixed" else uniform_ksat(*((60000, 258000) if maker == "k3" else (12000, 51600)), 3, seed=3)
     deg = np.bincount(np.abs(cnf.lits) - 1, minlength=cnf.n)
-    assert maker == "k3" or 33 < deg.max() <= 1024
+    assert maker != "mixed" or 33 < deg.max() <= 1024
     a = torch.randint(0, 2, (cnf.n, 5), device="cuda", dtype=torch.int8) * 2 - 1
     got = []
     for c in (cnf, _doubled(cnf)):
