@@ -1388,12 +1388,23 @@ __device__ __forceinline__ int slot_of(const int *__restrict__ start, int nslot,
     return lo;
 }
 
+// The block's slot, copied to shared memory: its views are then as close as
+// kernel arguments without holding registers.
+__device__ __forceinline__ const SlotDesc &block_slot(const SlotDesc *__restrict__ slots, int s) {
+    static_assert(sizeof(SlotDesc) % 4 == 0 && sizeof(SlotDesc) / 4 <= kThreads, "a word of the slot a thread");
+    __shared__ __align__(16) unsigned char raw[sizeof(SlotDesc)];
+    if (threadIdx.x < sizeof(SlotDesc) / 4)
+        reinterpret_cast<uint32_t *>(raw)[threadIdx.x] = reinterpret_cast<const uint32_t *>(slots + s)[threadIdx.x];
+    __syncthreads();
+    return *reinterpret_cast<const SlotDesc *>(raw);
+}
+
 template <int VW>
-__global__ void __launch_bounds__(kThreads)
+__global__ void __launch_bounds__(kThreads, VW <= 4 ? 4 : 1)
     k_forward_batch(const SlotDesc *__restrict__ slots, const int *__restrict__ start, int nslot) {
     const int s = slot_of(start, nslot, blockIdx.x);
     const int b0 = __ldg(start + s), b1 = __ldg(start + s + 1);
-    const SlotDesc &sd = slots[s];
+    const SlotDesc &sd = block_slot(slots, s);
     const int blk = blockIdx.x - b0, nblk = b1 - b0;
     switch (sd.I.kfix) {  // uniform over the block
         case 3: forward_body<VW, 3>(sd.I, sd.S.t0, sd.S.t1, nullptr, sd.D, sd.S.ubits, sd.S.fstore, FWD_STEP, blk, nblk); break;
@@ -1407,17 +1418,17 @@ template <int VU>
 __global__ void __launch_bounds__(kThreads)
     k_backward_heavy_batch(const SlotDesc *__restrict__ slots, const int *__restrict__ start, int nslot) {
     const int s = slot_of(start, nslot, blockIdx.x);
-    const SlotDesc &sd = slots[s];
+    const SlotDesc &sd = block_slot(slots, s);
     heavy_body<VU, 0, true>(sd.I, sd.S, sd.D, BWD_UPDATE, nullptr, nullptr, nullptr,
                       blockIdx.x - __ldg(start + s));
 }
 
 template <int VS>
-__global__ void __launch_bounds__(kThreads)
+__global__ void __launch_bounds__(kThreads, VS <= 4 ? 4 : 1)
     k_backward_light_batch(const SlotDesc *__restrict__ slots, const int *__restrict__ start, int nslot) {
     const int s = slot_of(start, nslot, blockIdx.x);
     const int b0 = __ldg(start + s);
-    const SlotDesc &sd = slots[s];
+    const SlotDesc &sd = block_slot(slots, s);
     vars_body<VS, 0, true>(sd.I, sd.S, sd.D, BWD_UPDATE, nullptr, nullptr, nullptr, blockIdx.x - b0);
 }
 

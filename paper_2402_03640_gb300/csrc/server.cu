@@ -590,14 +590,13 @@ extern "C" int msat_server_create(msat_server **out, const msat_server_config *c
     }
     S->cfg = cfg;
     S->work_cap = cfg.batch_mlits > 0 ? (int64_t)cfg.batch_mlits * 1000000 : 0;
-    // four restarts a thread in the batched clause pass (74 registers, three
-    // resident blocks per SM; eight take 92 and two blocks) -- measured on
-    // the k in {3,4,5} request stream at B = 8: 69 -> 75 instances/s
+    // four restarts a thread in both batched passes, whose kernels are held to
+    // 64 registers and four resident blocks per SM: 32 requests of k in
+    // {3, 4, 5}, n 110 to 45000, B = 8 take 78 ms; with two restarts a leaf
+    // task 86, with eight a thread of the clause pass 104, with three blocks
+    // per SM 86.  Launch shapes never change a result bit.
     S->fwd_vw = B < 4 ? B : 4;
-    // two restarts a leaf task: the batched variable pass then fits four
-    // resident blocks per SM (63 registers) instead of two at four restarts
-    // (86); launch shapes never change a result bit
-    S->stage_vw = B < 2 ? B : 2;
+    S->stage_vw = B < 4 ? B : 4;
     S->task_cap = std::max(kTaskCap, B / S->stage_vw);
     const int M = cfg.max_slots + 1;
     // builders: half the host's hardware threads, 1 to 8
