@@ -362,10 +362,15 @@ __device__ __forceinline__ void term_from_f(const DevInst &I, int o, uint32_t ni
 // valid where ok) of variable own_var for VW restarts at col to the sum of
 // their leaf, in order, all their loads in flight together (first: they open
 // the leaf, so the first term starts the sum instead of being added to +0).
-// With the clause pass's store, q = (float)w_j * f_j (NaN where satisfied)
-// gives the term +-(q * 2/W_U) or +0; otherwise the unsat bits select the
+// With the clause pass's store, q = (float)w_j * f_j (+0 where satisfied)
+// gives the term +-(q * 2/W_U); otherwise the unsat bits select the
 // restarts whose f is recomputed (fetched together with the bits when unsat
 // clauses are dense).
+// Bound by the gathers of q and, at one restart a thread, by the issue of the
+// ordered sum; +0 in place of a marker takes the test out of it: weighted
+// Zipf n=2e5, B=1 61.5 -> 59.0 us a step, n=1e6, B=16 462 -> 459, 5-SAT
+// n=30011, B=64 281 -> 275.  Without predicates (and with packed products) at
+// VW >= 2 fewer loads are in flight: n=1e6, B=16 494, n=30011 291.
 template <int VW, int KFIX, int C, bool STORE>
 __device__ __forceinline__ void occ_accumulate(const DevInst &I, const DevState &S, int kfix,
                                                const float *__restrict__ tcur, const int (&o)[C],
@@ -384,15 +389,24 @@ __device__ __forceinline__ void occ_accumulate(const DevInst &I, const DevState 
                 for (int e = 0; e < VW; ++e) v[u][e] = 0.0f;
             }
         }
+        // Satisfied occurrences add +-0, which can only change the sign of a
+        // zero sum (brought to +0 where it is used).  One restart a thread:
+        // the sign goes into the scale, +-(q * c) = q * (+-c), and missing
+        // occurrences add 0 too (no predicate in the chain)
 #pragma unroll
         for (int u = 0; u < C; ++u) {
-            if (!ok[u]) continue;
-            const bool neg = o[u] & 1;
+            if constexpr (VW == 1) {
+                const uint32_t sgn = (uint32_t)o[u] << 31;
+                leaf[0] = leaf[0] + v[u][0] * __uint_as_float(__float_as_uint(cs[0]) ^ sgn);
+            } else {
+                if (!ok[u]) continue;
+                const bool neg = o[u] & 1;
 #pragma unroll
-            for (int e = 0; e < VW; ++e) {
-                const float g = v[u][e] * cs[e];
-                const float term = (v[u][e] != v[u][e]) ? 0.0f : (neg ? -g : g);
-                leaf[e] = (first && u == 0) ? term : leaf[e] + term;
+                for (int e = 0; e < VW; ++e) {
+                    const float g = v[u][e] * cs[e];
+                    const float term = neg ? -g : g;
+                    leaf[e] = (first && u == 0) ? term : leaf[e] + term;
+                }
             }
         }
     } else {
@@ -461,7 +475,7 @@ __device__ __forceinline__ void finish_variable(const DevState &S, const DevStep
         ldv<VW>(tcur + q0, tv);
 #pragma unroll
         for (int e = 0; e < VW; ++e) {
-            gr[e] = Ssum[e] * fmaf(-tv[e], tv[e], 1.0f);
+            gr[e] = (Ssum[e] + 0.0f) * fmaf(-tv[e], tv[e], 1.0f);
             gr[e] = gscale ? gr[e] * gscale[col + e] : gr[e];
         }
         stv<VW>(grad_out + q0, gr);
@@ -473,7 +487,7 @@ __device__ __forceinline__ void finish_variable(const DevState &S, const DevStep
     float tn[VW];
 #pragma unroll
     for (int e = 0; e < VW; ++e) {
-        const float gr = Ssum[e] * fmaf(-w.t[e], w.t[e], 1.0f);
+        const float gr = (Ssum[e] + 0.0f) * fmaf(-w.t[e], w.t[e], 1.0f);
         if (D.improved[col + e]) S.bestx[q0 + e] = w.x[e] > 0.0f;
         if (D.cost[col + e] != 0) {
             w.x[e] = adam_update(A, w.x[e], w.m[e], w.v[e], gr);
@@ -682,12 +696,15 @@ __device__ __forceinline__ void forward_body(const DevInst &I, const float *__re
                 float q[VW];
 #pragma unroll
                 for (int e = 0; e < VW; ++e) {
-                    q[e] = __int_as_float(0x7fc00000);  // satisfied: NaN marker
+                    q[e] = 0.0f;  // satisfied
                     if (!sat[h][e]) {
                         nib |= 1u << e;
                         wacc[e] += (unsigned long long)wj;
                         q[e] = wf * f[h][e];
                         lacc[e] += q[e] * f[h][e];
+                        // f of an unsat clause is a sum of values <= 0; the
+                        // minimum keeps it and makes a NaN add nothing
+                        q[e] = fminf(q[e], 0.0f);
                     }
                 }
                 if (fstore) stv<VW>(fstore + (int64_t)jj[h] * B + col, q);

@@ -98,7 +98,7 @@ struct DevState {
     uint32_t *ubits;       // unsat bits, flat index row*B + b (row = j unless grouped)
     uint8_t *bestx;        // [n][B] best assignment (0/1)
     float *fstore;         // [m][B] of the last clause pass: (float)w_j * f_j where clause
-                           // j is unsat for restart b, NaN where it is satisfied; or
+                           // j is unsat for restart b, +0 where it is satisfied; or
                            // nullptr: the variable pass recomputes f from the unsat bits
 };
 

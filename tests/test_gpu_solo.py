@@ -116,3 +116,16 @@ def test_heavy_variable_of_many_chunks(pkg, oracle):
             assert s.info()["max_degree"] > 128 * 1024
             s.step(3, want_loss=False, want_cost=False, per_pass=True)
             assert np.array_equal(s.x().astype(np.float64), ref["x_final"])
+
+
+@pytest.mark.parametrize("B", [1, 2, 8])
+def test_nan_in_x_adds_nothing_on_the_per_pass_kernels(pkg, B):
+    """A NaN in x: with stored w*f the clauses that hold it contribute nothing
+    to the gradient of their other variables, which stay finite."""
+    cnf = uniform_ksat(60, 240, 3, seed=14)
+    with pkg.Solver.from_cnf(cnf, restarts=B, lr=1e-2, f_mode="store") as s:
+        st = s.get_state()
+        st["x"][7, 0] = np.nan
+        s.set_state(st)
+        s.step(1, want_loss=False, per_pass=True)
+        assert np.isfinite(np.delete(s.x(), 7, axis=0)).all()
