@@ -411,7 +411,7 @@ int msat::ctx_create(msat_ctx **out, int32_t n_vars, int64_t n_clauses, const in
         TRY_ALLOC(d_sperm, n_vars);
         if (!solo_w.empty()) TRY_ALLOC(d_sw, m);
     }
-    if (use_fstore && !solo_only) TRY_ALLOC(c->S.fstore, m * B);
+    if (use_fstore && !solo_only) TRY_ALLOC(c->S.fstore, (m + 1) * B);
     TRY_ALLOC(c->S.x, nB);
     TRY_ALLOC(c->S.mom, nB);
     TRY_ALLOC(c->S.vel, nB);
@@ -523,6 +523,7 @@ int msat::ctx_create(msat_ctx **out, int32_t n_vars, int64_t n_clauses, const in
     if (!e) e = cudaMemsetAsync(D.loss, 0, sizeof(float) * (size_t)B, st);
     if (!e) e = cudaMemsetAsync(D.hcount, 0, sizeof(unsigned) * std::max<size_t>(1, hvar.size() * (size_t)G), st);
     if (!e && !solo_only) e = cudaMemsetAsync(c->S.ubits, 0, sizeof(uint32_t) * (size_t)((m * B + 31) / 32 + 1), st);
+    if (!e && c->S.fstore) e = cudaMemsetAsync(c->S.fstore + m * B, 0, sizeof(float) * (size_t)B, st);
     if (!e) e = launch_init(I, c->S, cfg.seed_x, st);
     if (!e) e = cudaStreamSynchronize(st);  // host vectors above are freed on return
     if (e) {
@@ -1122,7 +1123,7 @@ static int ensure_probe(msat_ctx *c) {
     if ((rc = dalloc_t(c, &c->PS.ubits, (c->m * B + 31) / 32 + 1))) return rc;
     if ((rc = dalloc_t(c, &c->PD.sc, 1))) return rc;
     if ((rc = dalloc_t(c, &c->PD.wu_acc, (int64_t)kRep * B))) return rc;
-    if (c->S.fstore && (rc = dalloc_t(c, &c->PS.fstore, c->m * B))) return rc;
+    if (c->S.fstore && (rc = dalloc_t(c, &c->PS.fstore, (c->m + 1) * B))) return rc;
     if ((rc = dalloc_t(c, &c->PD.cost, B))) return rc;
     if ((rc = dalloc_t(c, &c->PD.cscale, B))) return rc;
     if ((rc = dalloc_t(c, &c->PD.lpart, (int64_t)c->PD.fwd_blocks * B))) return rc;
@@ -1135,6 +1136,8 @@ static int ensure_probe(msat_ctx *c) {
     sc.counter = 0;
     sc.steps_done = 0;
     MSAT_CUDA_TRY(cudaMemcpyAsync(c->PD.sc, &sc, sizeof(sc), cudaMemcpyHostToDevice, c->stream));
+    if (c->PS.fstore)
+        MSAT_CUDA_TRY(cudaMemsetAsync(c->PS.fstore + c->m * B, 0, sizeof(float) * (size_t)B, c->stream));
     MSAT_CUDA_TRY(cudaMemsetAsync(c->PD.wu_acc, 0, sizeof(unsigned long long) * (size_t)kRep * B, c->stream));
     MSAT_CUDA_TRY(cudaStreamSynchronize(c->stream));
     c->probe_ready = true;

@@ -361,17 +361,25 @@ __device__ __forceinline__ void term_from_f(const DevInst &I, int o, uint32_t ni
 // Adds the terms of C consecutive occurrences (words o, expanded records ox,
 // valid where ok) of variable own_var for VW restarts at col to the sum of
 // their leaf, in order, all their loads in flight together (first: they open
-// the leaf, so the first term starts the sum instead of being added to +0).
+// the leaf, so recomputed terms start the sum instead of being added to +0).
 // With the clause pass's store, q = (float)w_j * f_j (+0 where satisfied)
 // gives the term +-(q * 2/W_U); otherwise the unsat bits select the
 // restarts whose f is recomputed (fetched together with the bits when unsat
 // clauses are dense).
-// Bound by the gathers of q and, at one restart a thread, by the issue of the
-// ordered sum; +0 in place of a marker takes the test out of it: weighted
-// Zipf n=2e5, B=1 61.5 -> 59.0 us a step, n=1e6, B=16 462 -> 459, 5-SAT
-// n=30011, B=64 281 -> 275.  Without predicates (and with packed products) at
-// VW >= 2 fewer loads are in flight: n=1e6, B=16 494, n=30011 291.
-template <int VW, int KFIX, int C, bool STORE>
+// The store path is bound by its gathers (n=1e6, B=16: 1.4 GB read at 5.2
+// TB/s) with the issue slots half taken, so it is held to few instructions:
+// the sign is an exact factor of +-1 of the addition, or at one restart a
+// thread goes into the scale; satisfied occurrences add +-0 (a marker's test
+// and select are gone), which can only change the sign of a zero sum, brought
+// to +0 where it is used; missing occurrences read the store's zero row
+// instead of being predicated (at one restart a thread the predicate is
+// cheaper).  Us a step, marker and selects / without / packed pairs and the
+// zero row: weighted Zipf n=2e5, B=1 61.5 / 59.0 / -, B=8 190 / 186 / 182,
+// n=1e6, B=16 462 / 459 / 444, 5-SAT n=30011, B=64 281 / 274 / 261, 3-SAT
+// n=5000, B=256 36.0 / 35.5 / 33.9.  PACKED: two restarts a product and a
+// sum, in the light pass (a chunk's warp measured slower with it: Zipf
+// n=20000, B=16 49.3 against 46.5).
+template <int VW, int KFIX, int C, bool STORE, bool PACKED>
 __device__ __forceinline__ void occ_accumulate(const DevInst &I, const DevState &S, int kfix,
                                                const float *__restrict__ tcur, const int (&o)[C],
                                                const int2 (&ox)[C], const bool (&ok)[C],
@@ -382,31 +390,27 @@ __device__ __forceinline__ void occ_accumulate(const DevInst &I, const DevState 
     if constexpr (STORE) {
 #pragma unroll
         for (int u = 0; u < C; ++u) {
-            if (ok[u]) {
-                ldv<VW>(S.fstore + (int64_t)(o[u] >> I.occ_shift) * B + col, v[u]);
-            } else {
-#pragma unroll
-                for (int e = 0; e < VW; ++e) v[u][e] = 0.0f;
-            }
+            if (VW > 1 || ok[u]) ldv<VW>(S.fstore + (int64_t)(o[u] >> I.occ_shift) * B + col, v[u]);
+            else v[u][0] = 0.0f;
         }
-        // Satisfied occurrences add +-0, which can only change the sign of a
-        // zero sum (brought to +0 where it is used).  One restart a thread:
-        // the sign goes into the scale, +-(q * c) = q * (+-c), and missing
-        // occurrences add 0 too (no predicate in the chain)
 #pragma unroll
         for (int u = 0; u < C; ++u) {
-            if constexpr (VW == 1) {
+            if constexpr (PACKED) {
+                const float sg = (o[u] & 1) ? -1.0f : 1.0f;
+#pragma unroll
+                for (int e = 0; e < VW; e += 2) {
+                    const float2 l = fma2(mul2(make_float2(v[u][e], v[u][e + 1]), make_float2(cs[e], cs[e + 1])),
+                                          make_float2(sg, sg), make_float2(leaf[e], leaf[e + 1]));
+                    leaf[e] = l.x;
+                    leaf[e + 1] = l.y;
+                }
+            } else if constexpr (VW == 1) {
                 const uint32_t sgn = (uint32_t)o[u] << 31;
                 leaf[0] = leaf[0] + v[u][0] * __uint_as_float(__float_as_uint(cs[0]) ^ sgn);
             } else {
-                if (!ok[u]) continue;
-                const bool neg = o[u] & 1;
+                const float sg = (o[u] & 1) ? -1.0f : 1.0f;
 #pragma unroll
-                for (int e = 0; e < VW; ++e) {
-                    const float g = v[u][e] * cs[e];
-                    const float term = neg ? -g : g;
-                    leaf[e] = (first && u == 0) ? term : leaf[e] + term;
-                }
+                for (int e = 0; e < VW; ++e) leaf[e] = fmaf(v[u][e] * cs[e], sg, leaf[e]);
             }
         }
     } else {
@@ -1038,12 +1042,13 @@ __device__ __forceinline__ void heavy_body(const DevInst &I, const DevState &S, 
         float leaf[VW];
 #pragma unroll
         for (int e = 0; e < VW; ++e) leaf[e] = 0.0f;
+        const int none = STORE && VW > 1 ? I.m << I.occ_shift : 0;  // the store's zero row
         int on[C];
         int2 oxn[C];
 #pragma unroll
         for (int u = 0; u < C; ++u) {
             const bool okn = pb + u < pe;
-            on[u] = okn ? __ldg(I.occ + pb + u) : 0;
+            on[u] = okn ? __ldg(I.occ + pb + u) : none;
             oxn[u] = (expanded && okn) ? __ldg(I.occx + pb + u) : make_int2(0, 0);
         }
         for (int p = pb; p < pe; p += C) {
@@ -1056,10 +1061,10 @@ __device__ __forceinline__ void heavy_body(const DevInst &I, const DevState &S, 
                 o[u] = on[u];
                 ox[u] = oxn[u];
                 const bool okn = p + C + u < pe;
-                on[u] = okn ? __ldg(I.occ + p + C + u) : 0;
+                on[u] = okn ? __ldg(I.occ + p + C + u) : none;
                 oxn[u] = (expanded && okn) ? __ldg(I.occx + p + C + u) : make_int2(0, 0);
             }
-            occ_accumulate<VW, KFIX, C, STORE>(I, S, kfix, tcur, o, ox, ok, i, col, cs, dense, p == pb, leaf);
+            occ_accumulate<VW, KFIX, C, STORE, false>(I, S, kfix, tcur, o, ox, ok, i, col, cs, dense, p == pb, leaf);
         }
         __syncwarp();
         const int K = (cn + 31) / 32;
@@ -1230,12 +1235,13 @@ __device__ __forceinline__ void vars_body(const DevInst &I, const DevState &S, c
         for (int e = 0; e < VS; ++e) leaf[e] = 0.0f;
         // occurrence words one batch ahead: the next batch's words are in
         // flight while this batch's f values are gathered
+        const int none = STORE && VS > 1 ? I.m << I.occ_shift : 0;  // the store's zero row
         int on[C];
         int2 oxn[C];
 #pragma unroll
         for (int u = 0; u < C; ++u) {
             const bool okn = pb + u < pe;
-            on[u] = okn ? __ldg(I.occ + pb + u) : 0;
+            on[u] = okn ? __ldg(I.occ + pb + u) : none;
             oxn[u] = (expanded && okn) ? __ldg(I.occx + pb + u) : make_int2(0, 0);
         }
         for (int p = pb; p < pe; p += C) {
@@ -1248,10 +1254,10 @@ __device__ __forceinline__ void vars_body(const DevInst &I, const DevState &S, c
                 o[u] = on[u];
                 ox[u] = oxn[u];
                 const bool okn = p + C + u < pe;
-                on[u] = okn ? __ldg(I.occ + p + C + u) : 0;
+                on[u] = okn ? __ldg(I.occ + p + C + u) : none;
                 oxn[u] = (expanded && okn) ? __ldg(I.occx + p + C + u) : make_int2(0, 0);
             }
-            occ_accumulate<VS, KFIX, C, STORE>(I, S, kfix, tcur, o, ox, ok, i, col, cs, dense, p == pb, leaf);
+            occ_accumulate<VS, KFIX, C, STORE, (VS >= 2)>(I, S, kfix, tcur, o, ox, ok, i, col, cs, dense, p == pb, leaf);
         }
         if (nleaf == 1) {
             finish_variable<VS>(S, D, A, mode, q0, col, tcur, leaf, tnext, gscale, grad_out, PRE ? &pre : nullptr);

@@ -97,9 +97,10 @@ struct DevState {
     float *t0, *t1;        // double-buffered tanh(x), [n][B]
     uint32_t *ubits;       // unsat bits, flat index row*B + b (row = j unless grouped)
     uint8_t *bestx;        // [n][B] best assignment (0/1)
-    float *fstore;         // [m][B] of the last clause pass: (float)w_j * f_j where clause
-                           // j is unsat for restart b, +0 where it is satisfied; or
-                           // nullptr: the variable pass recomputes f from the unsat bits
+    float *fstore;         // [m+1][B] of the last clause pass: (float)w_j * f_j where clause
+                           // j is unsat for restart b, +0 where it is satisfied, the last
+                           // row +0; or nullptr: the variable pass recomputes f from the
+                           // unsat bits
 };
 
 // Lists of the one-block-per-restart step kernel (k_solo.cu): 16-bit literal

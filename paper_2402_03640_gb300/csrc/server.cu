@@ -161,7 +161,7 @@ size_t estimate_bytes(int64_t n, int64_t m, int64_t nnz, bool weighted, int B) {
     b += 4 * (size_t)(n + 1) + 4 * (size_t)nnz;                                   // transposed CSR
     b += 8 * (size_t)n + 8 * (size_t)(n + 1);                                     // heavy and light tables
     b += 21 * (size_t)n * B;                                                      // x, m, v, t0, t1, best
-    b += 4 * ((size_t)m * B / 32 + 2) + 4 * (size_t)m * B;                        // unsat bits, f store
+    b += 4 * ((size_t)m * B / 32 + 2) + 4 * (size_t)(m + 1) * B;                  // unsat bits, f store
     b += 8 * (size_t)kRep * B + 64 * (size_t)B + 4 * 1216 * (size_t)B;           // step state, partials
     b += 4 * ((size_t)nnz / kChunk + (size_t)n / 512 + 1) * B + 8 * (size_t)n;   // heavy partials
     b += 40 * 256 + (1 << 16);                                                    // rounding slack
