@@ -11,6 +11,7 @@
 #include <chrono>
 #include <cmath>
 #include <string>
+#include <system_error>
 #include <thread>
 #include <vector>
 
@@ -55,18 +56,28 @@ struct NvtxRange {
 // fresh heap 14 ms, after one write a page 0.7 (64 MB, eight cores: 2.9 ->
 // 1.8).
 static cudaError_t copy_out(void *dst, const void *src, size_t bytes, cudaStream_t st) {
-    if (bytes >= (1 << 20)) {
+    cudaPointerAttributes at{};
+    const bool plain = bytes >= (1 << 20) && cudaPointerGetAttributes(&at, dst) == cudaSuccess &&
+                       at.type == cudaMemoryTypeUnregistered;
+    cudaGetLastError();
+    if (plain) {  // pinned, managed or device memory has its pages
         const size_t page = (size_t)sysconf(_SC_PAGESIZE);
         volatile char *d = static_cast<volatile char *>(dst);
-        const int T = (int)std::max<size_t>(1, std::min<size_t>(8, bytes >> 23));
-        std::vector<std::thread> th;
         auto touch = [=](size_t b, size_t e) {
             for (size_t q = b; q < e; q += page) d[q] = 0;
         };
-        for (int t = 1; t < T; ++t) th.emplace_back(touch, bytes * t / T, bytes * (t + 1) / T);
+        const int T = (int)std::max<size_t>(1, std::min<size_t>(8, bytes >> 23));
+        std::thread th[8];
+        int t = 1;
+        try {
+            for (; t < T; ++t) th[t] = std::thread(touch, bytes * t / T, bytes * (t + 1) / T);
+        } catch (const std::system_error &) {  // no more threads: the rest here
+            touch(bytes * t / T, bytes);
+        }
         touch(0, bytes / T);
         d[bytes - 1] = 0;
-        for (std::thread &x : th) x.join();
+        for (std::thread &x : th)
+            if (x.joinable()) x.join();
     }
     return cudaMemcpyAsync(dst, src, bytes, cudaMemcpyDeviceToHost, st);
 }
@@ -198,6 +209,7 @@ int msat::ctx_create(msat_ctx **out, int32_t n_vars, int64_t n_clauses, const in
     bool on_dev = use_fstore && m > 0 && dev_cnf_worth(n_vars, m, clause_off[m]) &&
                   dv.check(n_vars, m, clause_off, lits, weights, stream, hc);
     if (!on_dev) {
+        dv.clear();  // what the device path took is the host path's to use
         const int hrc = build_host_cnf(n_vars, m, clause_off, lits, weights, hc);
         if (hrc) return hrc;
     }
@@ -289,6 +301,7 @@ int msat::ctx_create(msat_ctx **out, int32_t n_vars, int64_t n_clauses, const in
         // a row group past the device sort, or no memory: the host path after
         // all (every number above is the same there)
         on_dev = false;
+        dv.clear();
         const int hrc = build_host_cnf(n_vars, m, clause_off, lits, weights, hc);
         if (hrc) return hrc;
     }

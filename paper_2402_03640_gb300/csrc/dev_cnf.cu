@@ -355,14 +355,25 @@ cudaError_t own(const DevCnf &d, T **out, size_t count) {
 
 }  // namespace
 
-DevCnf::~DevCnf() {
+void DevCnf::clear() {
     // pending kernels may still use them: cudaFree waits for the device
-    for (void *p : {(void *)coff, (void *)lit, (void *)voff, (void *)occ, (void *)w, (void *)plit, (void *)pcoff, (void *)pw})
+    auto drop = [&](auto *&p) {
         if (p) {
             if (pool) cudaFreeAsync(p, st);
             else cudaFree(p);
         }
+        p = nullptr;
+    };
+    drop(coff);
+    drop(lit);
+    drop(voff);
+    drop(occ);
+    drop(w);
+    drop(plit);
+    drop(pcoff);
+    drop(pw);
     if (row) cudaFreeAsync(row, st);
+    row = nullptr;
 }
 
 bool DevCnf::check(int32_t n_vars, int64_t n_clauses, const int64_t *off, const int32_t *lits, const int64_t *weights,

@@ -28,7 +28,10 @@ struct DevCnf {
     explicit DevCnf(bool pool_alloc) : pool(pool_alloc) {}
     DevCnf(const DevCnf &) = delete;
     DevCnf &operator=(const DevCnf &) = delete;
-    ~DevCnf();
+    ~DevCnf() { clear(); }
+
+    // Frees every array still held here.
+    void clear();
 
     // Checks and packs the clauses and makes the occurrence offsets; fills
     // the sizes, kfix, max_len, max_deg, wsum, wor and voff of `out`.  False:
