@@ -1164,13 +1164,11 @@ extern "C" int msat_forward(msat_ctx *c, const float *x, float *loss, int64_t *c
     cudaStream_t st = c->stream;
     const int64_t nB = (int64_t)c->n * c->B;
     cudaError_t e = launch_tanh(x, c->PS.t0, nB, st);
-    if (!e) e = launch_forward(c->I, c->PS, c->PD, FWD_PROBE, c->PS.t0, st);
     DevStep d = c->PD;
     d.loss = loss;
-    if (!e) e = launch_loss_reduce(d, c->B, st);
-    if (!e && cost)
-        e = cudaMemcpyAsync(cost, c->PD.cost, sizeof(int64_t) * (size_t)c->B,
-                            cudaMemcpyDeviceToDevice, st);
+    if (cost) d.cost = reinterpret_cast<long long *>(cost);  // nothing later reads the context's own
+    if (!e) e = launch_forward(c->I, c->PS, d, FWD_PROBE, c->PS.t0, st);
+    if (!e && !probe_takes_loss(c->I)) e = launch_loss_reduce(d, c->B, st);
     if (e) return cuda_fail(e, "msat_forward");
     return MSAT_OK;
 }

@@ -207,7 +207,8 @@ __global__ void __launch_bounds__(kSoloMaxThreads, 1)
     const int nslice = (m + 31) >> 5;
     const int n_task = V.n_mtask + V.n_single;
     const int ntslice = (n_task + 31) >> 5;
-    float lpart = 0.0f, lden = 0.0f;  // of the loss of the last updated x
+    float lpart = 0.0f;  // of the loss of the last updated x, and its normaliser
+    double lden = 0.0;
     int imp = 0;
     float cs = 0.0f;
     long long cost = 0;
@@ -337,7 +338,8 @@ __global__ void __launch_bounds__(kSoloMaxThreads, 1)
         }
         const float den = fixed_den > 0.0f ? fixed_den : costf;
         cs = cost > 0 ? 2.0f / den : 0.0f;
-        if (step == n_steps - 1) lden = cost > 0 ? den : 0.0f;
+        if (step == n_steps - 1 && cost > 0)
+            lden = sc->loss_norm == 1 ? 1.0 : (double)(sc->loss_norm == 2 ? sc->wsum : cost);
     };
     auto update = [&](int i, float sum, float a_t, float r_t) {
         AdamView A = A0;
@@ -433,16 +435,17 @@ __global__ void __launch_bounds__(kSoloMaxThreads, 1)
     }
     // the loss of the last updated x (the terms of the last step's clause pass)
     if (n_steps > 0) {
-        float lsum = lpart;
+        double lsum = lpart;
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) lsum += __shfl_xor_sync(0xffffffffu, lsum, o);
         __syncthreads();
-        if (worker && lane == 0) s_part[warp] = (unsigned long long)__float_as_uint(lsum);
+        if (worker && lane == 0) s_part[warp] = (unsigned long long)__double_as_longlong(lsum);
         __syncthreads();
-        if (tid == 0) {
-            float sum = 0.0f;
-            for (int k = 0; k < nwarps; ++k) sum += __uint_as_float((unsigned)s_part[k]);
-            D.loss[b] = lden > 0.0f ? sum / lden : 0.0f;
+        if (warp == 0) {
+            lsum = lane < nwarps ? __longlong_as_double((long long)s_part[lane]) : 0.0;
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) lsum += __shfl_xor_sync(0xffffffffu, lsum, o);
+            if (lane == 0) D.loss[b] = lden > 0.0 ? (float)(lsum / lden) : 0.0f;
         }
     }
     if (capture)

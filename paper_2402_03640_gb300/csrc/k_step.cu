@@ -604,6 +604,60 @@ cudaError_t launch_transpose_u8(const uint8_t *in, uint8_t *out, int rows, int c
     return cudaGetLastError();
 }
 
+// The loss of the evaluated x from the clause pass's block partials, a warp
+// a restart: by blocks of their own behind the variable pass's, so no block
+// of variables waits for it, or, in a probe of few restarts, by the clause
+// pass's last block.  The partials' rounding errors average out over their
+// many blocks; what the reported value's error would come from is this chain
+// and its division, so both carry a second word (3-SAT n=1e6, B=16, 20
+// steps, against 64 bits: 5.6e-8 with one word, 2.2e-8 with two).
+
+constexpr int kWarps = kThreads / 32;
+
+__host__ __device__ inline int loss_blocks(int B) { return (B + kWarps - 1) / kWarps; }
+
+// s + lo += v, the rounding error of the addition collected in lo.
+__device__ __forceinline__ void add_two(float &s, float &lo, float v) {
+    const float t = s + v, z = t - s;
+    lo += (s - (t - z)) + (v - z);
+    s = t;
+}
+
+__device__ __forceinline__ void reduce_loss(const DevStep &D, int B, int blk) {
+    const int b = blk * kWarps + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    if (b >= B) return;
+    float s = 0.0f, lo = 0.0f;
+#pragma unroll 4
+    for (int k = lane; k < D.fwd_blocks; k += 32) add_two(s, lo, __ldcg(D.lpart + (long long)k * B + b));
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const float ol = __shfl_xor_sync(0xffffffffu, lo, o);
+        add_two(s, lo, __shfl_xor_sync(0xffffffffu, s, o));
+        lo += ol;
+    }
+    if (lane == 0) {
+        const long long c = D.cost[b];
+        const int ln = D.sc->loss_norm;
+        const long long d = ln == 1 ? 1 : ln == 2 ? D.sc->wsum : c;
+        const float den = (float)d, dlo = (float)(d - (long long)den);
+        const float q = s / den;
+        const float r = (fmaf(-q, den, s) + lo) - q * dlo;
+        D.loss[b] = c > 0 ? q + r / den : 0.0f;
+    }
+}
+
+// The same as a call, where inlined it would cost the kernel registers.
+static __device__ __noinline__ void call_reduce_loss(const DevStep &D, int B, int blk) { reduce_loss(D, B, blk); }
+
+// Probes of up to this many restarts (a warp of one block each) take their
+// loss in the clause pass's last block and save the reduction's launch (with
+// the cost written in place of a copy, 3-SAT n=1000, B=8: forward and backward
+// 281 -> 258 us, all of it the host's; 5-SAT n=30011, B=64 286 -> 266).  Eight
+// restarts a thread are left out: k = 5 would go from 80 registers to 87, two
+// resident blocks instead of three.
+__host__ __device__ constexpr bool takes_loss(int VW, int B) { return VW <= 4 && B <= kWarps; }
+bool probe_takes_loss(const DevInst &I) { return takes_loss(I.fwd_vw, I.B); }
+
 // --------------------------------------------------------------- k_forward
 // One item = (clause j, restart group g of VW restarts).  For VW <= 4 the
 // grid-stride loop is unrolled by two (items base + lane and base + stride +
@@ -859,6 +913,12 @@ __device__ __forceinline__ void forward_body(const DevInst &I, const float *__re
         }
     }
     if (threadIdx.x == 0) D.sc->counter = 0;
+    if constexpr (VW <= 4) {
+        if (mode == FWD_PROBE && takes_loss(VW, B)) {
+            __syncthreads();  // the costs
+            call_reduce_loss(D, B, 0);
+        }
+    }
     if (fstore) return;  // uniform: only a recomputing variable pass reads the density
     s_w = reinterpret_cast<unsigned long long *>(dyn_smem);
     __syncthreads();
@@ -972,30 +1032,6 @@ cudaError_t launch_forward(const DevInst &I0, const DevState &S, const DevStep &
 }
 
 // -------------------------------------------------------------- k_backward
-// The loss of the evaluated x from the clause pass's block partials, a warp
-// a restart: by blocks of their own behind the variable pass's, so no block
-// of variables waits for it.
-
-constexpr int kWarps = kThreads / 32;
-
-__host__ __device__ inline int loss_blocks(int B) { return (B + kWarps - 1) / kWarps; }
-
-__device__ __forceinline__ void reduce_loss(const DevStep &D, int B, int blk) {
-    const int b = blk * kWarps + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-    if (b >= B) return;
-    float acc = 0.0f;
-#pragma unroll 4
-    for (int k = lane; k < D.fwd_blocks; k += 32) acc += D.lpart[(long long)k * B + b];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    if (lane == 0) {
-        const long long c = D.cost[b];
-        const int ln = D.sc->loss_norm;
-        const float den = ln == 1 ? 1.0f : (float)(ln == 2 ? D.sc->wsum : c);
-        D.loss[b] = c > 0 ? acc / den : 0.0f;
-    }
-}
-
 // Heavy variables: a warp per (1024-occurrence chunk, restart group of VW
 // restarts), a lane per 32-occurrence leaf.  A lane sums its leaf in the
 // stored order straight from its gathers, the lanes' leaves meet by the
@@ -1150,7 +1186,10 @@ __device__ __forceinline__ void vars_body(const DevInst &I, const DevState &S, c
     const int kfix = KFIX > 0 ? KFIX : I.kfix;
     if (blk >= I.n_lblk) {  // the blocks behind the variables'
         grid_dep_wait();
-        if (mode == BWD_UPDATE) reduce_loss(D, B, blk - I.n_lblk);
+        if (mode == BWD_UPDATE) {
+            if constexpr (STORE) reduce_loss(D, B, blk - I.n_lblk);
+            else call_reduce_loss(D, B, blk - I.n_lblk);
+        }
         return;
     }
     float *s_leaf = reinterpret_cast<float *>(dyn_smem);

@@ -308,6 +308,7 @@ cudaError_t launch_step_batch(const SlotDesc *slots, int nslot, const int *fwd_s
                               cudaStream_t st);
 int heavy_blocks_of(const DevInst &I);
 int light_blocks_of(const DevInst &I, int mode);
+bool probe_takes_loss(const DevInst &I);
 cudaError_t launch_loss_reduce(const DevStep &D, int B, cudaStream_t st);
 // Small instances: one block per restart takes every step of a call (and, if
 // asked, the evaluation of the final x) with the restart's state in shared
