@@ -228,13 +228,16 @@ __global__ void __launch_bounds__(kThreads)
     }
 }
 
-// Up to this many literal evaluations the direct kernel: below it a call is
-// bound by its launches on the host, where a clear and one kernel (5.2 us)
-// beat two kernels (8.2 us); 3-SAT m=21500 with 64 assignments, 4.1 million,
-// takes 12.3 us directly and 11.7 packed.
-constexpr long long kDirectEvals = 1 << 20;
+// Up to this many literals read by a warp (each for 32 assignments, or for
+// fewer at the same cost) the direct kernel: below it a call is bound by its
+// launches on the host, where a clear and one kernel (5.2 us) beat two kernels
+// (8.2 us).  Whole calls, directly / packed: 80000 reads (weighted Zipf
+// n=2000, 33 assignments) 10.2 / 11.1 us, 129000 (3-SAT m=21500, 64) 12.3 /
+// 11.7, 213000 (5-SAT n=2000, 1) 12.4 / 10.7, 400000 (weighted Zipf n=20000,
+// 1) 23.0 / 10.9.
+constexpr long long kDirectReads = 96 << 10;
 
-bool eval_is_direct(int64_t nnz, int nb) { return nnz * nb <= kDirectEvals; }
+bool eval_is_direct(int64_t nnz, int nb) { return nnz * ((nb + 31) / 32) <= kDirectReads; }
 
 // Words a lane carries: rows of up to 128 assignments are one load.
 static int eval_vw(int nb) { return nb > 64 ? 4 : nb > 32 ? 2 : 1; }
