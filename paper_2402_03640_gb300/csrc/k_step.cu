@@ -627,7 +627,7 @@ __device__ __forceinline__ void reduce_loss(const DevStep &D, int B, int blk) {
     const int b = blk * kWarps + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     if (b >= B) return;
     float s = 0.0f, lo = 0.0f;
-#pragma unroll 4
+#pragma unroll 8
     for (int k = lane; k < D.fwd_blocks; k += 32) add_two(s, lo, __ldcg(D.lpart + (long long)k * B + b));
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
