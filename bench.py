@@ -396,7 +396,7 @@ def measure_workload(pkg, args, workload, ws, rank, with_cpu=True, with_e2e=True
     stream = torch.cuda.current_stream()
     dense = workload in DENSE_EVAL
     dense_cost = torch.empty(B, dtype=torch.int64, device="cuda")
-    # small instances run every step of a call in one single-CTA launch:
+    # small instances run every step of a call in one one-block-per-restart launch:
     # time one call of K steps (per-pass timing would force the per-pass
     # kernels)
     small = bool(solver.info()["small_kernel"]) and not dense
@@ -570,10 +570,10 @@ def measure_workload(pkg, args, workload, ws, rank, with_cpu=True, with_e2e=True
         "config": {"workload": workload, "description": desc, "n": cnf.n, "m": cnf.m,
                    "nnz": nnz, "restarts": B, "lr": LR,
                    "l2": ("flushed (256 MiB write) before the timed call, whose K steps run in one "
-                          "single-CTA launch with the state in shared memory" if small else
+                          "one-block-per-restart launch with the state in shared memory" if small else
                           "flushed (256 MiB write) before every timed step" if flush
                           else "working set larger than L2"),
-                   "route": "single-CTA kernel" if small else "per-pass kernels",
+                   "route": "one-block-per-restart kernel" if small else "per-pass kernels",
                    "launch": ("one launch of K steps" if small else
                               "each step replayed from a CUDA graph of its launches" if graph_err is None
                               else "plain launches (graph capture failed: %s)" % graph_err),
@@ -695,7 +695,7 @@ def other_configs(pkg, args, rank):
             ms = e0.elapsed_time(e1)
             _, cost = s.step(0, want_loss=False)
             _, best = s.best()
-            route = "single-CTA kernel" if s.info()["small_kernel"] else "per-pass kernels"
+            route = "one-block-per-restart kernel" if s.info()["small_kernel"] else "per-pass kernels"
         ent = {"description": desc, "n": cnf.n, "m": cnf.m, "nnz": cnf.nnz, "restarts": B, "steps": steps,
                "lr": LR, "route": route, "ms": ms, "us_per_step": 1e3 * ms / steps,
                "literal_evals_per_s": cnf.nnz * B * steps / (ms / 1e3),
@@ -998,10 +998,10 @@ def run_serving(args):
 
 # a kernel's sources and those of the data layout it reads (host_cnf.cu
 # builds the row order of the stored w f)
-KERNEL_SOURCES = {"forward": ("k_step.cu", "msat_internal.cuh", "host_cnf.cu"),
-                  "backward": ("k_step.cu", "msat_internal.cuh", "host_cnf.cu"),
+KERNEL_SOURCES = {"forward": ("k_step.cu", "step_math.cuh", "msat_internal.cuh", "host_cnf.cu"),
+                  "backward": ("k_step.cu", "step_math.cuh", "msat_internal.cuh", "host_cnf.cu"),
                   "dense_eval": ("k_dense.cu", "msat_internal.cuh"),
-                  "small_steps": ("k_step.cu", "msat_internal.cuh")}
+                  "small_steps": ("k_solo.cu", "step_math.cuh", "msat_internal.cuh")}
 
 
 def kernel_hash(kind="forward"):
