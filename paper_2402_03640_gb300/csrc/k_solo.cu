@@ -450,8 +450,10 @@ __global__ void __launch_bounds__(kSoloMaxThreads, 1)
     }
     if (capture)
         for (int i = tid; i < n; i += blockDim.x) sbest[i] = sx[i] > 0.0f;
-    __syncthreads();
+    // read before the barrier that every thread passes ahead of the block's
+    // count: the block that counts last writes the step scalars
     const long long steps_end = sc->steps_done + n_steps;
+    __syncthreads();
     const bool improved = s_improved != 0;
     float *t_out = (steps_end & 1) ? S.t1 : S.t0;
     for (int i = tid; i < n; i += blockDim.x) {
@@ -481,8 +483,9 @@ __global__ void __launch_bounds__(kSoloMaxThreads, 1)
         D.improved[b] = imp;
         D.cscale[b] = cs;
         __threadfence();
-        // the last block to finish (every block has read the scalars by then)
-        // leaves the step scalars of the call's end
+        // the last block to finish leaves the step scalars of the call's end;
+        // every thread of every block has read steps_done by then (its read
+        // lies before its block's last barrier, the count after it)
         s_last = atomicAdd(&sc->counter, 1u) == gridDim.x - 1;
     }
     __syncthreads();

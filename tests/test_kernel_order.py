@@ -1,0 +1,32 @@
+"""Orders inside kernels that no run can show to be missing: read from the
+sources, since a late access would have to be provoked on a GPU."""
+import os
+import re
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2402_03640_gb300", "csrc")
+
+
+def _body(name, kernel):
+    """The text of a kernel, without comments."""
+    text = open(os.path.join(CSRC, name)).read()
+    text = re.sub(r"//[^\n]*|/\*.*?\*/", "", text, flags=re.S)
+    at = text.index("{", re.search(r"\b%s\s*\(" % kernel, text).end())
+    depth = 0
+    for end in range(at, len(text)):
+        depth += {"{": 1, "}": -1}.get(text[end], 0)
+        if depth == 0:
+            return text[at:end]
+
+
+def test_step_scalars_are_read_before_the_block_is_counted():
+    """k_solo_steps: the block that counts last writes steps_done, so every
+    thread's read of it has to be ordered before its own block's count, that
+    is, to lie before the last barrier ahead of it (thread 0's own apart)."""
+    body = _body("k_solo.cu", "k_solo_steps")
+    count = body.index("atomicAdd(&sc->counter")
+    barrier = body.rindex("__syncthreads()", 0, count)
+    assert "steps_done" not in body[barrier:count]
+    assert "sc->p1" not in body[barrier:count] and "sc->p2" not in body[barrier:count]
+    # and the scalars are written behind the barrier that follows the count
+    write = body.index("sc->steps_done =")
+    assert "__syncthreads()" in body[count:write]
