@@ -134,9 +134,14 @@ static void free_all(msat_ctx *c) {
         if (c->pool_alloc) cudaFreeAsync(p, c->stream); else cudaFree(p);
     }
     c->allocs.clear();
-    if (c->ebits) cudaFree(c->ebits);
-    c->ebits = nullptr;
-    c->ebits_bytes = 0;
+    if (c->scratch.ev) {
+        cudaEventSynchronize(c->scratch.ev);  // the last use may be on another stream than the context's
+        cudaEventDestroy(c->scratch.ev);
+        c->scratch.ev = nullptr;
+    }
+    if (c->scratch.p) cudaFree(c->scratch.p);
+    c->scratch.p = nullptr;
+    c->scratch.bytes = 0;
     if (c->dense.Xt) cudaFree(c->dense.Xt);
     c->dense.Xt = nullptr;
     c->dense.xt_bytes = 0;
@@ -830,6 +835,48 @@ extern "C" int msat_check(msat_ctx *c) {
 
 static int dense_eval(msat_ctx *c, const int8_t *a, const float *x, int32_t nb, int64_t *cost_out);
 
+// The scratch buffer, at least `bytes` large, for launches on `st`; nullptr
+// where the memory cannot be had.  The caller holds the lock and ends its use
+// with scratch_done.
+static uint32_t *scratch_take(msat_ctx *c, size_t bytes, cudaStream_t st) {
+    EvalScratch &s = c->scratch;
+    unsigned long long id = 0;
+    cudaError_t e = cudaStreamGetId(st, &id);
+    if (!e && !s.ev) e = cudaEventCreateWithFlags(&s.ev, cudaEventDisableTiming);
+    else if (!e && id != s.stream_id) e = cudaStreamWaitEvent(st, s.ev, 0);
+    if (e) {
+        cudaGetLastError();
+        return nullptr;
+    }
+    s.stream_id = id;
+    if (bytes > s.bytes) {
+        if (s.p) {
+            cudaEventSynchronize(s.ev);
+            cudaFree(s.p);
+            s.p = nullptr;
+            s.bytes = 0;
+        }
+        e = cudaMalloc(&s.p, bytes);
+        if (e) {
+            cudaGetLastError();
+            s.p = nullptr;
+            return nullptr;
+        }
+        s.bytes = bytes;
+    }
+    return s.p;
+}
+
+// Ends a use of the scratch: what follows on another stream waits for it.
+static cudaError_t scratch_done(msat_ctx *c, cudaStream_t st) {
+    cudaError_t e = cudaEventRecord(c->scratch.ev, st);
+    if (e) {  // nothing to wait for later: wait here
+        cudaGetLastError();
+        e = cudaStreamSynchronize(st);
+    }
+    return e;
+}
+
 // Clause-list evaluation of a batch given as int8 +-1 (a) or as relaxed x
 // read through its rounding.  The packed batch lies in a buffer kept with the
 // context, at most 256 MiB (a larger batch goes through it in parts) or, where
@@ -837,50 +884,42 @@ static int dense_eval(msat_ctx *c, const int8_t *a, const float *x, int32_t nb, 
 // takes it from the stream-ordered pool instead, allocated and freed by the
 // graph: the graph may outlive the context's buffer.
 static int sparse_eval(msat_ctx *c, const int8_t *a, const float *x, int32_t nb, int64_t *cost_out) {
-    if (eval_is_direct(c->nnz, nb)) {
+    const cudaStream_t st = c->stream;
+    auto run = [&](int chunk, uint32_t *bits) {
         prof_begin(c, PROF_EVAL);
-        const cudaError_t e = launch_eval_sparse(c->I, a, x, nb, nb, c->wbits, nullptr, (long long *)cost_out, c->stream);
+        const cudaError_t e = launch_eval_sparse(c->I, a, x, nb, chunk, c->wbits, bits, (long long *)cost_out, st);
         prof_end(c);
+        return e;
+    };
+    if (eval_is_direct(c->nnz, nb)) {
+        const cudaError_t e = run(nb, nullptr);
         return e ? cuda_fail(e, "msat_evaluate: sparse kernel") : MSAT_OK;
     }
     constexpr int kGroup = 128;
     const int64_t groups = (256LL << 20) / (int64_t)eval_sparse_bytes(c->n, kGroup);
     int chunk = (int)std::min<int64_t>(nb, std::max<int64_t>(1, groups) * kGroup);
-    size_t need = eval_sparse_bytes(c->n, chunk);
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(c->stream, &cap) != cudaSuccess) cudaGetLastError();
-    const bool own = cap != cudaStreamCaptureStatusNone;
-    uint32_t *bits = c->ebits;
+    if (cudaStreamIsCapturing(st, &cap) != cudaSuccess) cudaGetLastError();
     cudaError_t e = cudaSuccess;
-    if (own) {
-        e = cudaMallocAsync(&bits, need, c->stream);
-    } else if (need > c->ebits_bytes) {
-        if (c->ebits) {
-            cudaStreamSynchronize(c->stream);
-            cudaFree(c->ebits);
-            c->ebits = nullptr;
-            c->ebits_bytes = 0;
-        }
-        e = cudaMalloc(&c->ebits, need);
-        if (e && chunk > kGroup) {
+    if (cap != cudaStreamCaptureStatusNone) {
+        uint32_t *bits = nullptr;
+        if (cudaMallocAsync(&bits, eval_sparse_bytes(c->n, chunk), st) != cudaSuccess) {
             cudaGetLastError();
-            chunk = kGroup;
-            need = eval_sparse_bytes(c->n, chunk);
-            e = cudaMalloc(&c->ebits, need);
+            return fail(MSAT_ENOMEM, "msat_evaluate: packed assignment buffer allocation failed");
         }
-        if (!e) c->ebits_bytes = need;
-        else c->ebits = nullptr;
-        bits = c->ebits;
-    }
-    if (e) {
-        cudaGetLastError();
-        return fail(MSAT_ENOMEM, "msat_evaluate: packed assignment buffer allocation failed");
-    }
-    prof_begin(c, PROF_EVAL);
-    e = launch_eval_sparse(c->I, a, x, nb, chunk, c->wbits, bits, (long long *)cost_out, c->stream);
-    prof_end(c);
-    if (own) {
-        const cudaError_t f = cudaFreeAsync(bits, c->stream);
+        e = run(chunk, bits);
+        const cudaError_t f = cudaFreeAsync(bits, st);
+        if (!e) e = f;
+    } else {
+        std::lock_guard<std::mutex> lk(c->scratch.mu);
+        uint32_t *bits = scratch_take(c, eval_sparse_bytes(c->n, chunk), st);
+        if (!bits && chunk > kGroup) {
+            chunk = kGroup;
+            bits = scratch_take(c, eval_sparse_bytes(c->n, chunk), st);
+        }
+        if (!bits) return fail(MSAT_ENOMEM, "msat_evaluate: packed assignment buffer allocation failed");
+        e = run(chunk, bits);
+        const cudaError_t f = scratch_done(c, st);
         if (!e) e = f;
     }
     if (e) return cuda_fail(e, "msat_evaluate: sparse kernel");

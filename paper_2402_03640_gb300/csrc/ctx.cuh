@@ -5,9 +5,24 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <mutex>
 #include <vector>
 
 #include "msat_internal.cuh"
+
+// Device scratch of a context for calls that write it and read it back in
+// kernels of their own.  A call holds `mu` from its first launch that touches
+// the buffer to the record of `ev` behind its last one, so that the launches
+// of two host threads' calls do not interleave; a call on another stream than
+// the last one's first waits for `ev` there.  stream_id: cudaStreamGetId of
+// the last use (a handle may name another stream by now).
+struct EvalScratch {
+    std::mutex mu;
+    uint32_t *p = nullptr;
+    size_t bytes = 0;
+    cudaEvent_t ev = nullptr;
+    unsigned long long stream_id = 0;
+};
 
 // Device memory of one context.  Every buffer is a separate allocation so
 // each starts on a 256-byte boundary (vector loads need 16 bytes).
@@ -42,8 +57,7 @@ struct msat_ctx {
     msat::DenseDev dense;
     // sparse evaluation: the packed batch (grown on use) and the bits of the
     // largest clause weight (0: all 1)
-    uint32_t *ebits = nullptr;
-    size_t ebits_bytes = 0;
+    EvalScratch scratch;
     int wbits = 0;
     long long *hgap = nullptr;    // [2][B] counts of msat_heuristic_gap, allocated on first use
 
