@@ -881,8 +881,9 @@ static cudaError_t scratch_done(msat_ctx *c, cudaStream_t st) {
 // read through its rounding.  The packed batch lies in a buffer kept with the
 // context, at most 256 MiB (a larger batch goes through it in parts) or, where
 // that cannot be had, 128 assignments' worth.  A call captured into a graph
-// takes it from the stream-ordered pool instead, allocated and freed by the
-// graph: the graph may outlive the context's buffer.
+// takes the kernel without scratch: the graph may outlive the context's
+// buffer and run beside another use of it, and scratch allocated by the graph
+// would leave it with one instance at a time and no use inside another graph.
 static int sparse_eval(msat_ctx *c, const int8_t *a, const float *x, int32_t nb, int64_t *cost_out) {
     const cudaStream_t st = c->stream;
     auto run = [&](int chunk, uint32_t *bits) {
@@ -891,26 +892,18 @@ static int sparse_eval(msat_ctx *c, const int8_t *a, const float *x, int32_t nb,
         prof_end(c);
         return e;
     };
-    if (eval_is_direct(c->nnz, nb)) {
-        const cudaError_t e = run(nb, nullptr);
-        return e ? cuda_fail(e, "msat_evaluate: sparse kernel") : MSAT_OK;
-    }
-    constexpr int kGroup = 128;
-    const int64_t groups = (256LL << 20) / (int64_t)eval_sparse_bytes(c->n, kGroup);
-    int chunk = (int)std::min<int64_t>(nb, std::max<int64_t>(1, groups) * kGroup);
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(st, &cap) != cudaSuccess) cudaGetLastError();
+    auto captured = [&] {
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        if (cudaStreamIsCapturing(st, &cap) != cudaSuccess) cudaGetLastError();
+        return cap != cudaStreamCaptureStatusNone;
+    };
     cudaError_t e = cudaSuccess;
-    if (cap != cudaStreamCaptureStatusNone) {
-        uint32_t *bits = nullptr;
-        if (cudaMallocAsync(&bits, eval_sparse_bytes(c->n, chunk), st) != cudaSuccess) {
-            cudaGetLastError();
-            return fail(MSAT_ENOMEM, "msat_evaluate: packed assignment buffer allocation failed");
-        }
-        e = run(chunk, bits);
-        const cudaError_t f = cudaFreeAsync(bits, st);
-        if (!e) e = f;
+    if (eval_is_direct(c->nnz, nb) || captured()) {
+        e = run(nb, nullptr);
     } else {
+        constexpr int kGroup = 128;
+        const int64_t groups = (256LL << 20) / (int64_t)eval_sparse_bytes(c->n, kGroup);
+        int chunk = (int)std::min<int64_t>(nb, std::max<int64_t>(1, groups) * kGroup);
         std::lock_guard<std::mutex> lk(c->scratch.mu);
         uint32_t *bits = scratch_take(c, eval_sparse_bytes(c->n, chunk), st);
         if (!bits && chunk > kGroup) {

@@ -195,12 +195,13 @@ __global__ void __launch_bounds__(kThreads)
     }
 }
 
-// Small batches of small instances, in one launch without scratch: a lane is
-// one assignment and a warp walks clauses, reading 32 entries of a variable's
-// row per literal.
+// Small batches of small instances, and calls that may not have scratch, in
+// one launch: a lane is one assignment and a warp walks clauses, reading 32
+// entries of a variable's row (of `row` entries, the first nb evaluated) per
+// literal.
 template <typename T>
 __global__ void __launch_bounds__(kThreads)
-    k_eval_direct(EvalInst I, const T *__restrict__ a, int nb, unsigned long long *__restrict__ cost) {
+    k_eval_direct(EvalInst I, const T *__restrict__ a, int row, int nb, unsigned long long *__restrict__ cost) {
     __shared__ unsigned long long s_acc[kEvalWarps][32];
     const int lane = threadIdx.x & 31;
     const int warp = threadIdx.x >> 5;
@@ -213,7 +214,7 @@ __global__ void __launch_bounds__(kThreads)
         bool sat = false;
         for (int p = beg; p < end; ++p) {
             const int L = __ldg(I.lit + p);
-            const T v = live ? __ldg(a + (long long)(L >> 1) * nb + b) : T(0);
+            const T v = live ? __ldg(a + (long long)(L >> 1) * row + b) : T(0);
             sat |= is_true(v) != (bool)(L & 1);
         }
         if (!sat) acc += I.w ? (unsigned long long)__ldg(I.w + j) : 1ull;
@@ -279,15 +280,20 @@ cudaError_t launch_eval_sparse(const DevInst &I, const int8_t *a, const float *x
     if (I.m == 0 || !bits) {
         e = cudaMemsetAsync(cost_out, 0, sizeof(long long) * (size_t)nb, st);
         if (e != cudaSuccess || I.m == 0) return e;
-        const int gy = (nb + 31) / 32;
         const long long need = ((long long)I.m + kEvalWarps - 1) / kEvalWarps;
-        const dim3 grid((unsigned)std::max<long long>(1, std::min<long long>(need, (152LL * 8 + gy - 1) / gy)),
-                        (unsigned)gy);
         const EvalInst E{I.m, I.kfix, I.coff, I.lit, I.w};
         unsigned long long *cost = reinterpret_cast<unsigned long long *>(cost_out);
-        if (a) k_eval_direct<int8_t><<<grid, kThreads, 0, st>>>(E, a, nb, cost);
-        else k_eval_direct<float><<<grid, kThreads, 0, st>>>(E, x, nb, cost);
-        return cudaGetLastError();
+        constexpr long long kGridY = 65535;  // a launch's limit, in words of 32 assignments
+        for (long long b0 = 0; b0 < nb && e == cudaSuccess; b0 += 32 * kGridY) {
+            const int k = (int)std::min<long long>(32 * kGridY, nb - b0);
+            const int gy = (k + 31) / 32;
+            const dim3 grid((unsigned)std::max<long long>(1, std::min<long long>(need, (152LL * 8 + gy - 1) / gy)),
+                            (unsigned)gy);
+            if (a) k_eval_direct<int8_t><<<grid, kThreads, 0, st>>>(E, a + b0, nb, k, cost + b0);
+            else k_eval_direct<float><<<grid, kThreads, 0, st>>>(E, x + b0, nb, k, cost + b0);
+            e = cudaGetLastError();
+        }
+        return e;
     }
     for (int b0 = 0; b0 < nb && e == cudaSuccess; b0 += chunk) {
         const int k = std::min(chunk, nb - b0);

@@ -81,3 +81,59 @@ def test_evaluations_from_two_threads(pkg, batches):
         for t in (0, 1):
             assert len(got[t]) == 100
             assert all(np.array_equal(g.cpu().numpy(), want[t]) for g in got[t])
+
+
+def test_captured_evaluation_holds_no_allocation(pkg, batches):
+    """A graph with a captured evaluation can have two instances at a time,
+    and both give the batch's costs."""
+    import ctypes
+
+    import torch
+    cnf, dev, want = batches
+    st = torch.cuda.Stream()
+    rt = ctypes.CDLL("libcudart.so.%s" % torch.version.cuda.split(".")[0])
+    raw = ctypes.c_void_p(st.cuda_stream)
+    with pkg.Solver.from_cnf(cnf, restarts=1, stream=st) as s:
+        out = torch.empty(dev[0].shape[1], dtype=torch.int64, device="cuda")
+        torch.cuda.synchronize()
+        graph, execs = ctypes.c_void_p(), [ctypes.c_void_p(), ctypes.c_void_p()]
+        assert rt.cudaStreamBeginCapture(raw, 1) == 0  # this thread's calls
+        rc = s._lib.msat_evaluate(s._ctx, ctypes.c_void_p(dev[0].data_ptr()), dev[0].shape[1],
+                                  ctypes.c_void_p(out.data_ptr()), 0)
+        assert rt.cudaStreamEndCapture(raw, ctypes.byref(graph)) == 0 and rc == 0
+        for e in execs:
+            assert rt.cudaGraphInstantiate(ctypes.byref(e), graph, ctypes.c_ulonglong(0)) == 0
+        for e in execs:
+            out.fill_(-1)
+            torch.cuda.synchronize()
+            assert rt.cudaGraphLaunch(e, raw) == 0
+            torch.cuda.synchronize()
+            assert np.array_equal(out.cpu().numpy(), want[0])
+        for e in execs:
+            rt.cudaGraphExecDestroy(e)
+        rt.cudaGraphDestroy(graph)
+
+
+def test_captured_evaluation_of_very_many_assignments(pkg):
+    """Past one launch's range of the kernel without scratch."""
+    import torch
+    from synth import Cnf
+    cnf = Cnf.from_clauses(3, [[1, 2], [-1, 3], [-2, -3]], weights=[5, 1 << 33, 7])
+    nb = 65535 * 32 + 33
+    rng = np.random.default_rng(8)
+    a = rng.choice(np.array([-1, 1], np.int8), size=(3, nb))
+    t = a > 0
+    want = 5 * ~(t[0] | t[1]) + (1 << 33) * ~(~t[0] | t[2]) + 7 * ~(~t[1] | ~t[2])
+    dev = torch.from_numpy(a).cuda()
+    st = torch.cuda.Stream()
+    with pkg.Solver.from_cnf(cnf, restarts=1, stream=st) as s:
+        g = torch.cuda.CUDAGraph()
+        torch.cuda.synchronize()
+        with torch.cuda.graph(g, stream=st):
+            out = s.evaluate(dev, "sparse")
+        g.replay()
+        torch.cuda.synchronize()
+        assert np.array_equal(out.cpu().numpy(), want)
+        out = s.evaluate(dev, "sparse")
+        torch.cuda.synchronize()
+        assert np.array_equal(out.cpu().numpy(), want)
