@@ -234,7 +234,10 @@ int msat_autotune(int32_t n_vars, int64_t n_clauses, const int64_t *clause_off,
  *   cost_out    device int64[nb]: sum of w_j over clauses with no true literal
  *   backend     MSAT_BACKEND_SPARSE or MSAT_BACKEND_DENSE
  * Asynchronous on the context stream; the result is exact for both
- * backends.  The dense backend multiplies the clause matrix W^T (e2m1,
+ * backends.  The clause-list backend packs large calls into device scratch
+ * that it keeps with the context (at most 256 MiB, or 16 bytes a variable);
+ * where that cannot be had, and in a call captured into a graph, it needs
+ * none and takes longer.  The dense backend multiplies the clause matrix W^T (e2m1,
  * m x n, packed two codes a byte, built on its first use: m_pad * n_pad / 2
  * bytes, rejected above 64 GiB) by the batch on the tensor cores; it needs
  * weights below 2^25.
@@ -271,6 +274,14 @@ int msat_check(msat_ctx *ctx);
  * device stays usable.  Synchronous; allocates and frees one 4-byte flag.
  */
 int msat_selftest_bounded_wait(int64_t spins);
+
+/*
+ * Self-test of the calls that keep device scratch with a context: from now on
+ * scratch above `bytes` counts as memory that cannot be had on this context
+ * (a negative value: no such limit).  The calls then take their routes with
+ * less scratch or none, which give the same results.
+ */
+int msat_selftest_scratch_limit(msat_ctx *ctx, int64_t bytes);
 
 /*
  * Measured peak of the dense backend's tensor-core instruction (no

@@ -840,6 +840,7 @@ static int dense_eval(msat_ctx *c, const int8_t *a, const float *x, int32_t nb, 
 // with scratch_done.
 static uint32_t *scratch_take(msat_ctx *c, size_t bytes, cudaStream_t st) {
     EvalScratch &s = c->scratch;
+    if (s.limit >= 0 && bytes > (size_t)s.limit) return nullptr;
     unsigned long long id = 0;
     cudaError_t e = cudaStreamGetId(st, &id);
     if (!e && !s.ev) e = cudaEventCreateWithFlags(&s.ev, cudaEventDisableTiming);
@@ -880,10 +881,11 @@ static cudaError_t scratch_done(msat_ctx *c, cudaStream_t st) {
 // Clause-list evaluation of a batch given as int8 +-1 (a) or as relaxed x
 // read through its rounding.  The packed batch lies in a buffer kept with the
 // context, at most 256 MiB (a larger batch goes through it in parts) or, where
-// that cannot be had, 128 assignments' worth.  A call captured into a graph
-// takes the kernel without scratch: the graph may outlive the context's
-// buffer and run beside another use of it, and scratch allocated by the graph
-// would leave it with one instance at a time and no use inside another graph.
+// that cannot be had, 128 assignments' worth, or else the kernel without
+// scratch runs.  A call captured into a graph takes that one: the graph may
+// outlive the context's buffer and run beside another use of it, and scratch
+// allocated by the graph would leave it with one instance at a time and no use
+// inside another graph.
 static int sparse_eval(msat_ctx *c, const int8_t *a, const float *x, int32_t nb, int64_t *cost_out) {
     const cudaStream_t st = c->stream;
     auto run = [&](int chunk, uint32_t *bits) {
@@ -898,9 +900,8 @@ static int sparse_eval(msat_ctx *c, const int8_t *a, const float *x, int32_t nb,
         return cap != cudaStreamCaptureStatusNone;
     };
     cudaError_t e = cudaSuccess;
-    if (eval_is_direct(c->nnz, nb) || captured()) {
-        e = run(nb, nullptr);
-    } else {
+    bool packed = false;
+    if (!eval_is_direct(c->nnz, nb) && !captured()) {
         constexpr int kGroup = 128;
         const int64_t groups = (256LL << 20) / (int64_t)eval_sparse_bytes(c->n, kGroup);
         int chunk = (int)std::min<int64_t>(nb, std::max<int64_t>(1, groups) * kGroup);
@@ -910,11 +911,14 @@ static int sparse_eval(msat_ctx *c, const int8_t *a, const float *x, int32_t nb,
             chunk = kGroup;
             bits = scratch_take(c, eval_sparse_bytes(c->n, chunk), st);
         }
-        if (!bits) return fail(MSAT_ENOMEM, "msat_evaluate: packed assignment buffer allocation failed");
-        e = run(chunk, bits);
-        const cudaError_t f = scratch_done(c, st);
-        if (!e) e = f;
+        if (bits) {
+            packed = true;
+            e = run(chunk, bits);
+            const cudaError_t f = scratch_done(c, st);
+            if (!e) e = f;
+        }
     }
+    if (!packed) e = run(nb, nullptr);
     if (e) return cuda_fail(e, "msat_evaluate: sparse kernel");
     return MSAT_OK;
 }
@@ -1231,6 +1235,13 @@ extern "C" int msat_selftest_bounded_wait(int64_t spins) {
         return fail(MSAT_ETIMEOUT, "msat_selftest_bounded_wait: the wait gave up after " +
                                        (spins ? std::to_string(spins) + " tries" : std::string("its time limit")) +
                                        " (flag " + std::to_string(h) + ")");
+    return MSAT_OK;
+}
+
+extern "C" int msat_selftest_scratch_limit(msat_ctx *c, int64_t bytes) {
+    if (!c) return fail(MSAT_EINVAL, "msat_selftest_scratch_limit: ctx is NULL");
+    std::lock_guard<std::mutex> lk(c->scratch.mu);
+    c->scratch.limit = bytes;
     return MSAT_OK;
 }
 

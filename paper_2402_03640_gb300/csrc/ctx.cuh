@@ -22,6 +22,7 @@ struct EvalScratch {
     size_t bytes = 0;
     cudaEvent_t ev = nullptr;
     unsigned long long stream_id = 0;
+    int64_t limit = -1;  // msat_selftest_scratch_limit
 };
 
 // Device memory of one context.  Every buffer is a separate allocation so

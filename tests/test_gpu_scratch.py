@@ -137,3 +137,19 @@ def test_captured_evaluation_of_very_many_assignments(pkg):
         out = s.evaluate(dev, "sparse")
         torch.cuda.synchronize()
         assert np.array_equal(out.cpu().numpy(), want)
+
+
+def test_evaluation_without_scratch(pkg, batches):
+    """Where the packed batch cannot be allocated, 128 assignments' worth of
+    it, and where that cannot be had the kernel without scratch, give the same
+    costs."""
+    cnf, dev, want = batches
+    group = 16 * cnf.n  # bytes of 128 packed assignments
+    with pkg.Solver.from_cnf(cnf, restarts=2) as s:
+        for limit in (0, group - 1, group, -1):
+            assert s._lib.msat_selftest_scratch_limit(s._ctx, limit) == 0
+            for a, w in zip(dev, want):
+                assert np.array_equal(s.evaluate(a, "sparse").cpu().numpy(), w), limit
+        s._lib.msat_selftest_scratch_limit(s._ctx, 0)
+        x = s.x()
+        assert np.array_equal(s.evaluate_x("sparse").cpu().numpy(), costs(cnf, np.where(x > 0, 1, -1)))
