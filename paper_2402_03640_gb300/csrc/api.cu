@@ -851,13 +851,11 @@ static uint32_t *scratch_take(msat_ctx *c, size_t bytes, cudaStream_t st) {
     }
     s.stream_id = id;
     if (bytes > s.bytes) {
-        if (s.p) {
-            cudaEventSynchronize(s.ev);
-            cudaFree(s.p);
-            s.p = nullptr;
-            s.bytes = 0;
-        }
-        e = cudaMalloc(&s.p, bytes);
+        // in stream order: the call stays asynchronous
+        if (s.p) cudaFreeAsync(s.p, st);
+        s.p = nullptr;
+        s.bytes = 0;
+        e = cudaMallocAsync(&s.p, bytes, st);
         if (e) {
             cudaGetLastError();
             s.p = nullptr;

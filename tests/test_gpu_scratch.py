@@ -153,3 +153,22 @@ def test_evaluation_without_scratch(pkg, batches):
         s._lib.msat_selftest_scratch_limit(s._ctx, 0)
         x = s.x()
         assert np.array_equal(s.evaluate_x("sparse").cpu().numpy(), costs(cnf, np.where(x > 0, 1, -1)))
+
+
+def test_growing_scratch_does_not_wait_for_the_stream(pkg, batches):
+    """The first evaluation of a context and one with a larger batch return
+    while earlier work of their stream still runs."""
+    import torch
+    cnf, dev, want = batches
+    st = torch.cuda.Stream()
+    for rep in range(2):  # the first round loads the kernels
+        with pkg.Solver.from_cnf(cnf, restarts=1, stream=st) as s, torch.cuda.stream(st):
+            torch.cuda.synchronize()
+            torch.cuda._sleep(400_000_000)  # about 0.2 s
+            busy = torch.cuda.Event()
+            busy.record(st)
+            got = [s.evaluate(a, "sparse") for a in dev]
+            waited = busy.query()
+            torch.cuda.synchronize()
+            assert all(np.array_equal(g.cpu().numpy(), w) for g, w in zip(got, want))
+    assert not waited
