@@ -1090,7 +1090,10 @@ extern "C" int msat_get_info(msat_ctx *c, msat_info *info) {
     info->m = c->m;
     info->nnz = c->nnz;
     info->steps_done = sc.steps_done;
-    info->device_bytes = c->device_bytes;
+    {
+        std::lock_guard<std::mutex> lk(c->scratch.mu);
+        info->device_bytes = c->device_bytes + (int64_t)c->scratch.bytes;
+    }
     info->max_clause_len = c->max_len;
     info->max_degree = c->max_deg;
     info->n_heavy = c->I.n_heavy;

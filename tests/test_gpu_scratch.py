@@ -172,3 +172,15 @@ def test_growing_scratch_does_not_wait_for_the_stream(pkg, batches):
             torch.cuda.synchronize()
             assert all(np.array_equal(g.cpu().numpy(), w) for g, w in zip(got, want))
     assert not waited
+
+
+def test_scratch_is_reported(pkg, batches):
+    """msat_info counts the packed batch among the device memory held."""
+    cnf, dev, _ = batches
+    with pkg.Solver.from_cnf(cnf, restarts=1) as s:
+        b0 = s.info()["device_bytes"]
+        for a in dev:
+            words = (a.shape[1] + 31) // 32
+            words = (words + 3) // 4 * 4 if a.shape[1] > 64 else words
+            s.evaluate(a, "sparse")
+            assert s.info()["device_bytes"] == b0 + 4 * words * cnf.n
