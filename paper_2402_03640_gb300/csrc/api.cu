@@ -1041,18 +1041,23 @@ extern "C" int msat_best(msat_ctx *c, uint8_t *assign01, int64_t *best_cost) {
                                       cudaMemcpyDeviceToHost, c->stream));
     const size_t nB = (size_t)c->n * c->B;
     if (assign01 && c->B > 1 && nB >= (1 << 16)) {
-        // transposed on the device into the tanh buffer that the next step
-        // writes; from n=5000, B=256 (0.86 ms -> 0.05) on, the host loop's
-        // strided bytes cost more than the kernel and the copy
-        StepScalars sc;
-        MSAT_CUDA_TRY(cudaMemcpyAsync(&sc, c->D.sc, sizeof(sc), cudaMemcpyDeviceToHost, c->stream));
-        MSAT_CUDA_TRY(cudaStreamSynchronize(c->stream));
-        uint8_t *tr = reinterpret_cast<uint8_t *>((sc.steps_done & 1) ? c->S.t0 : c->S.t1);
-        const cudaError_t e = launch_transpose_u8(c->S.bestx, tr, c->n, c->B, c->stream);
-        if (e) return cuda_fail(e, "msat_best: transposition");
-        MSAT_CUDA_TRY(copy_out(assign01, tr, nB, c->stream));
-        MSAT_CUDA_TRY(cudaStreamSynchronize(c->stream));
-        return MSAT_OK;
+        // transposed on the device in the context's scratch, which no step
+        // touches: steps of this context may be running on another stream or
+        // be issued by another thread meanwhile.  From n=5000, B=256 (0.86 ms
+        // -> 0.05) on, the host loop's strided bytes cost more than the kernel
+        // and the copy; it remains for where there is no memory for a copy.
+        const cudaStream_t st = c->stream;
+        MSAT_CUDA_TRY(cudaStreamSynchronize(st));  // not under the lock
+        std::lock_guard<std::mutex> lk(c->scratch.mu);
+        if (uint8_t *tr = reinterpret_cast<uint8_t *>(scratch_take(c, nB, st))) {
+            cudaError_t e = launch_transpose_u8(c->S.bestx, tr, c->n, c->B, st);
+            if (!e) e = copy_out(assign01, tr, nB, st);
+            const cudaError_t f = scratch_done(c, st);
+            if (!e) e = f;
+            if (!e) e = cudaStreamSynchronize(st);
+            if (e) return cuda_fail(e, "msat_best: transposition");
+            return MSAT_OK;
+        }
     }
     std::vector<uint8_t> tmp;
     if (assign01 && c->B == 1) {

@@ -5,7 +5,7 @@ import threading
 import numpy as np
 import pytest
 
-from synth import zipf_weighted
+from synth import uniform_ksat, zipf_weighted
 
 pytestmark = pytest.mark.gpu
 
@@ -184,3 +184,52 @@ def test_scratch_is_reported(pkg, batches):
             words = (words + 3) // 4 * 4 if a.shape[1] > 64 else words
             s.evaluate(a, "sparse")
             assert s.info()["device_bytes"] == b0 + 4 * words * cnf.n
+
+
+@pytest.mark.parametrize("how", ["stream", "thread"])
+def test_best_beside_running_steps(pkg, how):
+    """Reading the best assignments while steps of the context run on another
+    stream, or are issued by another thread, leaves the trajectory as it is."""
+    import torch
+    cnf = uniform_ksat(3001, 12907, 3, seed=11)
+    B, steps, lr = 64, 2001, 1e-2
+    with pkg.Solver.from_cnf(cnf, restarts=B, lr=lr) as s:
+        s.step(steps, want_loss=False, per_pass=True)
+        want = s.x()
+    with pkg.Solver.from_cnf(cnf, restarts=B, lr=lr) as s:
+        s.best()  # loads the kernel
+        calls = 0
+        if how == "stream":
+            a, b = torch.cuda.Stream(), torch.cuda.Stream()
+            s.set_stream(a)
+            s.step_async(steps, per_pass=True)
+            s.set_stream(b)
+            while not a.query():
+                s.best()
+                calls += 1
+            s.set_stream(a)
+        else:
+            def work():
+                for _ in range(steps):
+                    s.step_async(1, final_eval=False, per_pass=True)
+                s.step_async(0, per_pass=True)
+            t = threading.Thread(target=work)
+            t.start()
+            while t.is_alive():
+                s.best()
+                calls += 1
+            t.join()
+        torch.cuda.synchronize()
+        assert calls > 3
+        assert np.array_equal(s.x(), want)
+
+
+def test_best_without_scratch(pkg):
+    """Where the transposed copy cannot be allocated the host transposes."""
+    cnf = uniform_ksat(1501, 6000, 3, seed=6)
+    with pkg.Solver.from_cnf(cnf, restarts=64, lr=1e-2) as s:
+        s.step(3, per_pass=True)
+        want = s.get_state()["best_assign"].T
+        for limit in (0, cnf.n * 64 - 1, -1):
+            s._lib.msat_selftest_scratch_limit(s._ctx, limit)
+            assert np.array_equal(s.best()[0], want), limit
