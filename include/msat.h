@@ -284,6 +284,15 @@ int msat_selftest_bounded_wait(int64_t spins);
 int msat_selftest_scratch_limit(msat_ctx *ctx, int64_t bytes);
 
 /*
+ * Self-test of msat_create's two preparations, which give the same arrays:
+ * which one made this context's.
+ */
+#define MSAT_PREP_HOST 0
+#define MSAT_PREP_DEVICE 1
+#define MSAT_PREP_HOST_AFTER_DEVICE 2 /* the device path gave up after reading the literals */
+int msat_selftest_preparation(msat_ctx *ctx, int32_t *route);
+
+/*
  * Measured peak of the dense backend's tensor-core instruction (no
  * counterpart in the paper; a benchmark helper): every SM issues `iters`
  * stages of four block-scaled kind::mxf4 MMAs (M = 128 clauses, N =

@@ -363,6 +363,7 @@ int msat::ctx_create(msat_ctx **out, int32_t n_vars, int64_t n_clauses, const in
     c->cfg = cfg;
     c->stream = stream;
     c->pool_alloc = pool_alloc;
+    c->prep_route = on_dev ? MSAT_PREP_DEVICE : dv.read_lits ? MSAT_PREP_HOST_AFTER_DEVICE : MSAT_PREP_HOST;
     cudaGetDevice(&c->device);
     c->n = n_vars;
     c->B = cfg.restarts;
@@ -1248,6 +1249,12 @@ extern "C" int msat_selftest_scratch_limit(msat_ctx *c, int64_t bytes) {
     if (!c) return fail(MSAT_EINVAL, "msat_selftest_scratch_limit: ctx is NULL");
     std::lock_guard<std::mutex> lk(c->scratch.mu);
     c->scratch.limit = bytes;
+    return MSAT_OK;
+}
+
+extern "C" int msat_selftest_preparation(msat_ctx *c, int32_t *route) {
+    if (!c || !route) return fail(MSAT_EINVAL, "msat_selftest_preparation: NULL argument");
+    *route = c->prep_route;
     return MSAT_OK;
 }
 

@@ -37,6 +37,7 @@ struct msat_ctx {
     int32_t kfix = 0, max_len = 0, max_deg = 0;
     int64_t wsum = 0;
     int64_t steps_done_host = 0;
+    int32_t prep_route = 0;       // msat_selftest_preparation
     std::vector<void *> allocs;
     int64_t device_bytes = 0;
 

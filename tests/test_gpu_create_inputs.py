@@ -52,3 +52,49 @@ def test_no_literal_is_read_before_the_offsets_are_checked(pkg):
         pkg.Solver(cnf.n, off, lits, None, restarts=1)
     assert "non-decreasing at clause 100" in str(e.value)
     assert _resident(buf, head, total) == 0
+
+
+def _route(s):
+    r = ctypes.c_int32(-1)
+    assert s._lib.msat_selftest_preparation(s._ctx, ctypes.byref(r)) == 0
+    return {0: "host", 1: "device", 2: "host after device"}[r.value]
+
+
+@pytest.mark.parametrize("what,want", [("clean", "device"), ("small", "host"), ("long", "host"), ("hot", "host"),
+                                       ("doubled", "host"), ("one_doubled", "host after device"),
+                                       ("just_past_a_warp", "host after device")])
+def test_instances_for_the_host_are_seen_early(pkg, what, want):
+    """A clause too long, variables in very many clauses and repeats in most
+    clauses keep an instance off the device path before its literals are
+    uploaded; a single repeat and a variable of 1025 occurrences are found
+    there."""
+    from synth import Cnf, zipf_weighted
+    rng = np.random.default_rng(2)
+    cnf = uniform_ksat(*((60000, 258000) if what != "small" else (300, 1290)), 3, seed=3)
+    lits, off, w = cnf.lits.copy(), cnf.off, cnf.weights
+    if what == "long":
+        lits, off = np.concatenate([lits, np.arange(1, 34, dtype=np.int32)]), np.append(off, off[-1] + 33)
+    elif what == "hot":
+        z = zipf_weighted(20000, 60000, seed=4)
+        assert np.bincount(np.abs(z.lits)).max() > 4096
+        lits, off, w = z.lits, z.off, z.weights
+    elif what == "doubled":
+        lits[1::3] = lits[0::3]
+    elif what == "one_doubled":
+        lits[off[-2] + 1] = lits[off[-2]]
+    elif what == "just_past_a_warp":
+        cl = lits.reshape(-1, 3)
+        have = (np.abs(cl) == 1).any(axis=1)
+        add = rng.choice(np.flatnonzero(~have), size=1025 - have.sum(), replace=False)
+        cl[add, 0] = 1
+        assert (np.abs(lits) == 1).sum() == 1025
+    n = z.n if what == "hot" else cnf.n
+    with pkg.Solver(n, off, lits, w, restarts=1, lr=1e-2) as s:
+        assert _route(s) == want
+        a = rng.choice(np.array([-1, 1], np.int8), size=(n, 3))
+        import torch
+        got = s.evaluate(torch.from_numpy(a).cuda(), "sparse").cpu().numpy()
+    clause = np.repeat(np.arange(off.size - 1), np.diff(off))
+    for b in range(3):
+        sat = np.bincount(clause[(a[np.abs(lits) - 1, b] > 0) == (lits > 0)], minlength=off.size - 1)
+        assert got[b] == (np.ones(off.size - 1, np.int64) if w is None else w)[sat == 0].sum()
