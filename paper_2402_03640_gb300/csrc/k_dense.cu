@@ -723,16 +723,18 @@ __global__ void k_dense_fill(DevInst I, uint8_t *__restrict__ Wt, int n_pad) {
 // X^T in packed e2m1 (rows = assignments, n_pad / 2 bytes each, zero
 // padding) from a batch stored [n][nb]: a block transposes 64 variables x
 // 32 assignments through shared memory, reading along the batch and
-// writing 32 bytes (64 codes) of each assignment's row.
+// writing 32 bytes (64 codes) of each assignment's row.  The step before may
+// still be writing x when this kernel starts: the batch is read by loads that
+// stay behind the wait.
 template <typename T>
-__device__ __forceinline__ void pack_transpose(const T *__restrict__ src, int n, int nb, uint8_t *__restrict__ Xt,
+__device__ __forceinline__ void pack_transpose(const T *src, int n, int nb, uint8_t *__restrict__ Xt,
                                                int n_pad, int rows) {
     __shared__ uint8_t tile[64][33];
     const int v0 = blockIdx.x * 64, b0 = blockIdx.y * 32;
     for (int r = threadIdx.y; r < 64; r += blockDim.y) {
         const int v = v0 + r, b = b0 + threadIdx.x;
         uint8_t e = 0;
-        if (v < n && b < nb) e = src[(long long)v * nb + b] > (T)0 ? kE2M1One : kE2M1MinusOne;
+        if (v < n && b < nb) e = ld_ordered(src + (long long)v * nb + b) > (T)0 ? kE2M1One : kE2M1MinusOne;
         tile[r][threadIdx.x] = e;
     }
     __syncthreads();
@@ -751,7 +753,7 @@ __device__ __forceinline__ void pack_transpose(const T *__restrict__ src, int n,
 // here (a clear of its own between the two kept them apart: n=5000, 256
 // assignments a call after the other 27.5 -> 20.1 us).
 template <typename T>
-__global__ void k_dense_convert(const T *__restrict__ a, int n, int nb, uint8_t *__restrict__ Xt,
+__global__ void k_dense_convert(const T *a, int n, int nb, uint8_t *__restrict__ Xt,
                                 int n_pad, int rows, long long *__restrict__ cost) {
     grid_dep_launch();
     grid_dep_wait();

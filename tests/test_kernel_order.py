@@ -30,3 +30,14 @@ def test_step_scalars_are_read_before_the_block_is_counted():
     # and the scalars are written behind the barrier that follows the count
     write = body.index("sc->steps_done =")
     assert "__syncthreads()" in body[count:write]
+
+
+def test_dense_batch_is_read_behind_the_wait():
+    """k_dense_convert may start while the kernel that writes its batch still
+    runs: it waits, and then reads the batch by ordered loads only, never
+    through the read-only cache."""
+    body = _body("k_dense.cu", "k_dense_convert")
+    wait = body.index("grid_dep_wait()")
+    assert "cost[" not in body[:wait] and "pack_transpose" not in body[:wait]
+    pack = _body("k_dense.cu", "pack_transpose")
+    assert pack.count("src") == 1 and "ld_ordered(src" in pack
