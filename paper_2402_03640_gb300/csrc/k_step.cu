@@ -480,7 +480,7 @@ __device__ __forceinline__ void finish_variable(const DevState &S, const DevStep
 #pragma unroll
         for (int e = 0; e < VW; ++e) {
             gr[e] = (Ssum[e] + 0.0f) * fmaf(-tv[e], tv[e], 1.0f);
-            gr[e] = gscale ? gr[e] * gscale[col + e] : gr[e];
+            gr[e] = gscale ? gr[e] * ld_ordered(gscale + col + e) : gr[e];
         }
         stv<VW>(grad_out + q0, gr);
         return;

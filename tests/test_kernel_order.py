@@ -41,3 +41,12 @@ def test_dense_batch_is_read_behind_the_wait():
     assert "cost[" not in body[:wait] and "pack_transpose" not in body[:wait]
     pack = _body("k_dense.cu", "pack_transpose")
     assert pack.count("src") == 1 and "ld_ordered(src" in pack
+
+
+def test_gradient_scale_is_read_behind_the_wait():
+    """The caller's kernel that writes the scale of msat_backward is the one
+    before the variable pass in the stream: every read of it is an ordered
+    load, which stays behind the pass's wait."""
+    text = re.sub(r"//[^\n]*", "", open(os.path.join(CSRC, "k_step.cu")).read())
+    assert not re.search(r"gscale\s*\[|\*\s*gscale\b(?!,|\))", text)
+    assert "ld_ordered(gscale + " in text
