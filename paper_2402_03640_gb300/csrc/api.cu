@@ -186,7 +186,7 @@ extern "C" int msat_create(msat_ctx **out, int32_t n_vars, int64_t n_clauses,
 
 int msat::ctx_create(msat_ctx **out, int32_t n_vars, int64_t n_clauses, const int64_t *clause_off,
                      const int32_t *lits, const int64_t *weights, const msat_config *cfg_in,
-                     cudaStream_t stream, bool pool_alloc) {
+                     cudaStream_t stream, bool pool_alloc, bool dev_prep) {
     if (!out) return fail(MSAT_EINVAL, "msat_create: out is NULL");
     *out = nullptr;
     msat_config cfg;
@@ -211,7 +211,7 @@ int msat::ctx_create(msat_ctx **out, int32_t n_vars, int64_t n_clauses, const in
     const bool use_fstore = cfg.f_mode == MSAT_F_STORE || (cfg.f_mode == MSAT_F_AUTO && auto_store);
     HostCnf hc;
     DevCnf dv(pool_alloc);
-    bool on_dev = use_fstore && m > 0 && dev_cnf_worth(n_vars, m, clause_off[m]) &&
+    bool on_dev = dev_prep && use_fstore && m > 0 && dev_cnf_worth(n_vars, m, clause_off[m]) &&
                   dv.check(n_vars, m, clause_off, lits, weights, stream, hc);
     if (!on_dev) {
         dv.clear();  // what the device path took is the host path's to use

@@ -76,10 +76,11 @@ struct msat_ctx {
 namespace msat {
 
 // msat_create with an explicit stream; pool_alloc: allocate with
-// cudaMallocAsync on that stream (freed with cudaFreeAsync in order).
+// cudaMallocAsync on that stream (freed with cudaFreeAsync in order);
+// dev_prep: instances worth it may be prepared on the device.
 int ctx_create(msat_ctx **out, int32_t n_vars, int64_t n_clauses, const int64_t *clause_off,
                const int32_t *lits, const int64_t *weights, const msat_config *cfg,
-               cudaStream_t stream, bool pool_alloc);
+               cudaStream_t stream, bool pool_alloc, bool dev_prep = true);
 // final evaluation of the current x (best update and capture) on c->stream
 cudaError_t ctx_eval_current(msat_ctx *c);
 // free a context without synchronising (pool contexts: frees ordered on c->stream)

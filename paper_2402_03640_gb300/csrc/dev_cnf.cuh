@@ -62,4 +62,12 @@ inline bool dev_cnf_worth(int32_t n, int64_t m, int64_t raw) {
     return raw >= (1 << 17) && 21LL * n + 4LL * m > 227 * 1024;
 }
 
+// Upper bound of the device bytes that DevCnf::check holds at a time: the
+// uploaded offsets and literals and the variables' counts beside the arrays
+// that stay.  Nothing else of a context is allocated before they are freed;
+// DevCnf::occurrences (without rows) holds less than the context does later.
+inline size_t dev_cnf_check_bytes(int32_t n, int64_t m, int64_t raw, bool weighted) {
+    return 12 * (size_t)(m + 1) + 8 * (size_t)raw + 9 * (size_t)(n + 1) + (weighted ? 8 * (size_t)m : 0) + 16 * 512;
+}
+
 }  // namespace msat

@@ -41,6 +41,7 @@
 #include <nvtx3/nvToolsExt.h>
 
 #include "ctx.cuh"
+#include "dev_cnf.cuh"
 
 using namespace msat;
 using Clock = std::chrono::steady_clock;
@@ -58,6 +59,7 @@ struct SrvRequest {
     Clock::time_point t_submit;
     size_t est = 0;
     int64_t work = 0;  // literal evaluations of one step: nnz x restarts
+    bool dev_prep = false;  // the reservation covers a preparation on the device
 };
 
 struct SrvSlot {
@@ -154,7 +156,8 @@ struct msat_server {
 namespace {
 
 // Upper bound of a context's device bytes (the allocations msat_create makes
-// with f stored, before repeated literals are dropped).
+// with f stored, before repeated literals are dropped; a preparation on the
+// device may hold more for a while, see msat_submit).
 size_t estimate_bytes(int64_t n, int64_t m, int64_t nnz, bool weighted, int B) {
     size_t b = 0;
     b += 4 * (size_t)(m + 1) + 4 * (size_t)nnz + (weighted ? 8 * (size_t)m : 0);  // clause CSR
@@ -252,7 +255,8 @@ void builder_main(msat_server *S, int k) {
         const msat_config cfg = request_config(S, req);
         msat_ctx *c = nullptr;
         const int rc = ctx_create(&c, req.n, req.m, req.off.data(), req.lits.data(),
-                                  req.w.empty() ? nullptr : req.w.data(), &cfg, S->build_st[(size_t)k], true);
+                                  req.w.empty() ? nullptr : req.w.data(), &cfg, S->build_st[(size_t)k], true,
+                                  req.dev_prep);
         if (rc) finish_failed(S, req.ticket, rc, req.t_submit);
         SrvBuilt b;
         b.ctx = rc ? nullptr : c;
@@ -705,6 +709,16 @@ extern "C" int msat_submit(msat_server *S, const msat_request *req, uint64_t *ti
     if (req->weights) r.w.assign(req->weights, req->weights + m);
     r.est = estimate_bytes(r.n, m, nnz, req->weights != nullptr, S->cfg.restarts);
     r.work = nnz * (int64_t)S->cfg.restarts;
+    // the reservation covers the preparation too; where the budget holds the
+    // context but not its preparation on the device, the host prepares it
+    // (with one restart and more than about eight clauses a variable the
+    // preparation is the larger of the two: 5-SAT n=8000, m=168000 8.8 against
+    // 8.5 MB)
+    if (dev_cnf_worth(r.n, m, nnz)) {
+        const size_t prep = dev_cnf_check_bytes(r.n, m, nnz, req->weights != nullptr);
+        r.dev_prep = std::max(prep, r.est) <= S->cfg.hbm_budget;
+        if (r.dev_prep) r.est = std::max(prep, r.est);
+    }
     if (r.est > S->cfg.hbm_budget)
         return fail(MSAT_EBUDGET, "msat_submit: the instance needs about " + std::to_string(r.est) +
                                       " device bytes, above the server budget of " +
