@@ -215,7 +215,7 @@ int msat::ctx_create(msat_ctx **out, int32_t n_vars, int64_t n_clauses, const in
                   dv.check(n_vars, m, clause_off, lits, weights, stream, hc);
     if (!on_dev) {
         dv.clear();  // what the device path took is the host path's to use
-        const int hrc = build_host_cnf(n_vars, m, clause_off, lits, weights, hc);
+        const int hrc = build_host_cnf(n_vars, m, clause_off, lits, weights, dv.off_checked, hc);
         if (hrc) return hrc;
     }
     I32Buf &coff = hc.coff, &lit = hc.lit, &voff = hc.voff, &occ = hc.occ;
@@ -307,7 +307,7 @@ int msat::ctx_create(msat_ctx **out, int32_t n_vars, int64_t n_clauses, const in
         // all (every number above is the same there)
         on_dev = false;
         dv.clear();
-        const int hrc = build_host_cnf(n_vars, m, clause_off, lits, weights, hc);
+        const int hrc = build_host_cnf(n_vars, m, clause_off, lits, weights, dv.off_checked, hc);
         if (hrc) return hrc;
     }
     if (block_rows && !on_dev) {

@@ -359,6 +359,30 @@ struct Temps {
     }
 };
 
+// Up to this many clauses the host looks at the offsets: the pass costs 0.6 us
+// per thousand clauses, the device's its launch, a wait and, where the host
+// path follows, an upload.  msat_create with the host's look / the device's:
+// weighted Zipf m=1e5 4.20 / 4.36 ms, m=3e5 7.42 / 7.55, m=1e6 12.8 / 12.4,
+// 3-SAT m=51600 0.56 / 0.56, m=258000 1.06 / 0.93; in either case the host
+// path then skips its own (Zipf m=1e5 4.15, m=1e6 11.6, m=2e6 17.5 ms; 4.08,
+// 11.9 and 18.3 before there was a device path).
+constexpr int64_t kHostOffsets = 1 << 17;
+
+// Whether every clause has 0 to kMaxCleanLen literals, and the shortest and
+// longest.  off[0] is 0, so differences within that range (taken modulo 2^64)
+// say that the offsets are their sums, below 2^31, and never decrease.
+bool lengths_in_range(int64_t m, const int64_t *off, int &min_len, int &max_len) {
+    int64_t lo = INT_MAX, hi = 0;
+    for (int64_t j = 0; j < m; ++j) {
+        const int64_t d = (int64_t)((uint64_t)off[j + 1] - (uint64_t)off[j]);
+        lo = std::min(lo, d);
+        hi = std::max(hi, d);
+    }
+    min_len = (int)lo;
+    max_len = (int)hi;
+    return lo >= 0 && hi <= kMaxCleanLen;
+}
+
 // Whether a look at a few clauses (offsets checked, at most kMaxCleanLen
 // literals each) already says that the instance is for the host path: a
 // variable twice in one of them, or one so frequent that it has about twice
@@ -442,22 +466,33 @@ bool DevCnf::check(int32_t n_vars, int64_t n_clauses, const int64_t *off, const 
     int64_t *d_off = nullptr;
     int32_t *d_raw = nullptr, *deg = nullptr, *part = nullptr;
     CnfStat *stat = nullptr;
+    CnfStat h{0u, 0, INT_MAX, 0, 0ull, 0ull};
+    const bool host_off = m <= kHostOffsets;
+    if (host_off) {
+        if (!lengths_in_range(m, off, h.min_len, h.max_len)) return false;
+        off_checked = true;
+        if (sample_unfit(m, off, lits)) return false;
+    }
     cudaError_t e = T.get(&d_off, (size_t)m + 1);
     if (!e) e = T.get(&stat, 1);
-    CnfStat h{0u, 0, INT_MAX, 0, 0ull, 0ull};
     if (!e) e = cudaMemcpyAsync(stat, &h, sizeof(h), cudaMemcpyHostToDevice, st);
     if (!e) e = cudaMemcpyAsync(d_off, off, sizeof(int64_t) * (size_t)(m + 1), cudaMemcpyHostToDevice, st);
-    if (!e) {
-        k_off_check<<<grid_for(m), kThreads, 0, st>>>(m, d_off, stat);
-        e = cudaGetLastError();
+    if (!host_off) {
+        if (!e) {
+            k_off_check<<<grid_for(m), kThreads, 0, st>>>(m, d_off, stat);
+            e = cudaGetLastError();
+        }
+        if (!e) e = cudaMemcpyAsync(&h, stat, sizeof(h), cudaMemcpyDeviceToHost, st);
+        if (!e) e = cudaStreamSynchronize(st);
     }
-    if (!e) e = cudaMemcpyAsync(&h, stat, sizeof(h), cudaMemcpyDeviceToHost, st);
-    if (!e) e = cudaStreamSynchronize(st);
     if (e) {
         cudaGetLastError();
         return false;
     }
-    if (h.flags || sample_unfit(m, off, lits)) return false;
+    if (!host_off) {
+        off_checked = (h.flags & 1u) == 0;
+        if (h.flags || sample_unfit(m, off, lits)) return false;
+    }
     read_lits = true;
     e = own(*this, &coff, (size_t)m + 1);
     if (!e) e = own(*this, &lit, (size_t)raw);

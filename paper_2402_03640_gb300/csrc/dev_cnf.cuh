@@ -24,6 +24,7 @@ struct DevCnf {
     int32_t *row = nullptr;  // temporary: clause -> row of the store
     int32_t *plit = nullptr, *pcoff = nullptr;
     int64_t *pw = nullptr;
+    bool off_checked = false;  // check() has seen that the offsets never decrease
     bool read_lits = false;  // the literals were uploaded
 
     explicit DevCnf(bool pool_alloc) : pool(pool_alloc) {}

@@ -50,10 +50,10 @@ int threads_for(int64_t work) {
 }  // namespace
 
 int build_host_cnf(int32_t n, int64_t m, const int64_t *off, const int32_t *lits, const int64_t *w,
-                   HostCnf &out) {
+                   bool off_checked, HostCnf &out) {
     if (off[0] != 0) return fail(MSAT_EINVAL, "msat_create: clause_off[0] must be 0");
     const int Tm = threads_for(m);
-    {
+    if (!off_checked) {
         std::vector<int64_t> bad((size_t)Tm, -1);
         parallel_ranges(m, Tm, [&](int t, int64_t b, int64_t e) {
             for (int64_t j = b; j < e; ++j)

@@ -54,9 +54,10 @@ struct HostCnf {
 // range, weights >= 1, canonical clauses of at most kMaxClauseLen literals)
 // and fills `out` up to the occurrence offsets (voff); MSAT_EINVAL with the
 // message of the first violation in input order.  The work is spread over
-// the host's hardware threads.
+// the host's hardware threads.  off_checked: the offsets are known not to
+// decrease.
 int build_host_cnf(int32_t n, int64_t m, const int64_t *off, const int32_t *lits, const int64_t *w,
-                   HostCnf &out);
+                   bool off_checked, HostCnf &out);
 
 // Rows of the clause pass's store of w*f grouped by the variable pass's
 // light blocks: a clause's home is the block of its first light variable

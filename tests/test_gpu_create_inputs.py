@@ -98,3 +98,35 @@ def test_instances_for_the_host_are_seen_early(pkg, what, want):
     for b in range(3):
         sat = np.bincount(clause[(a[np.abs(lits) - 1, b] > 0) == (lits > 0)], minlength=off.size - 1)
         assert got[b] == (np.ones(off.size - 1, np.int64) if w is None else w)[sat == 0].sum()
+
+
+@pytest.mark.parametrize("m", [(1 << 17) - 1, 1 << 17, (1 << 17) + 1])
+@pytest.mark.parametrize("bad", ["first", "last", "wrap", "none"])
+def test_offsets_on_both_sides_of_the_line(pkg, m, bad):
+    """Offsets checked by the host (up to 2^17 clauses) and by the device: an
+    offset that decreases, at the first clause, the last or by differences
+    that are small modulo 2^64, is refused with the literals behind it
+    untouched; without one the device prepares the instance."""
+    from paper_2402_03640_gb300 import MsatError
+    cnf = uniform_ksat(30000, m, 3, seed=3)
+    off, total = cnf.off.copy(), 64 << 20
+    buf = mmap.mmap(-1, total, flags=mmap.MAP_PRIVATE | mmap.MAP_ANONYMOUS)
+    lits = np.frombuffer(buf, np.int32, count=total // 4)
+    lits[:cnf.lits.size] = cnf.lits
+    if bad == "none":
+        with pkg.Solver(cnf.n, off, lits[:cnf.lits.size], None, restarts=1) as s:
+            assert _route(s) == "device" and s.info()["uniform_len"] == 3
+        return
+    at = {"first": 0, "last": m - 1, "wrap": 1000}[bad]
+    if bad == "first":
+        off[1], off[2:] = -1, total // 4
+        off[-1] = total // 4
+    elif bad == "last":
+        off[m - 1], off[m] = total // 4 + 1, total // 4
+    else:
+        off[at + 1:] = np.iinfo(np.int64).min + 3
+        off[-1] = total // 4
+    with pytest.raises(MsatError) as e:
+        pkg.Solver(cnf.n, off, lits, None, restarts=1)
+    assert "non-decreasing at clause %d" % at in str(e.value)
+    assert _resident(buf, 8 << 20, total) == 0
