@@ -10,6 +10,7 @@
 #include <algorithm>
 #include <chrono>
 #include <cmath>
+#include <future>
 #include <string>
 #include <system_error>
 #include <thread>
@@ -173,6 +174,16 @@ extern "C" int msat_config_default(msat_config *cfg) {
 
 extern "C" const char *msat_last_error(void) { return g_last_error.c_str(); }
 
+static int multiprocessors() {
+    int dev = 0, sms = 0;
+    cudaGetDevice(&dev);
+    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
+        cudaGetLastError();
+        sms = 152;
+    }
+    return sms;
+}
+
 static bool valid_restarts(int32_t B) {
     return B >= 1 && B <= 1024 && (B & (B - 1)) == 0;
 }
@@ -314,16 +325,11 @@ int msat::ctx_create(msat_ctx **out, int32_t n_vars, int64_t n_clauses, const in
         const int rrc = build_block_rows(n_vars, m, kfix, coff, lit, weights, lblk, ro);
         if (rrc) return rrc;
     }
-    // a forced row order is a request for the per-pass kernels
+    // lists of the one-block-per-restart kernel, if it may take this instance
     SoloHost solo;
-    bool use_solo = cfg.row_order != 2 && !on_dev && build_solo(n_vars, m, kfix, max_len, max_deg, hc, solo);
-    if (use_solo) {
-        int dev = 0;
-        cudaGetDevice(&dev);
-        if (cudaDeviceGetAttribute(&solo.dev.sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
-            cudaGetLastError();
-            solo.dev.sms = 152;
-        }
+    auto make_solo = [&, sms = multiprocessors()]() -> bool {
+        if (!build_solo(n_vars, m, kfix, max_len, max_deg, hc, weights, solo)) return false;
+        solo.dev.sms = sms;
         DevInst shape{};
         shape.n = n_vars;
         shape.B = B;
@@ -332,17 +338,33 @@ int msat::ctx_create(msat_ctx **out, int32_t n_vars, int64_t n_clauses, const in
         // for a long call, with room for what the estimate does not know; each
         // call then takes the faster route (the serving engine has only one,
         // and its batch does not start a step for this instance alone)
-        use_solo = solo_pays(solo.dev, shape, nnz, max_len, 1 << 30, pool_alloc ? 1.5 : 2.0);
+        return solo_pays(solo.dev, shape, nnz, max_len, 1 << 30, pool_alloc ? 1.5 : 2.0);
+    };
+    // by a thread of its own beside the rest of the creation, which does not
+    // read them (the serving engine's does), from this many literals on: the
+    // thread costs about 25 us, the lists 3 ns a literal and 196 us at n=5000.
+    // With one upload of the lists and one allocation of the small arrays,
+    // msat_create of 3-SAT n=1000, B=8 361 -> 318, n=5000, B=1 848 -> 640,
+    // weighted Zipf n=3000, B=1 1105 -> 791 us (300, 645 and 785 before there
+    // were such lists)
+    constexpr int64_t kSoloBeside = 1 << 13;
+    bool use_solo = false;
+    std::future<bool> solo_made;  // waits for the thread where an error leaves early
+    if (cfg.row_order != 2 && !on_dev) {  // a forced row order is a request for the per-pass kernels
+        if (!pool_alloc && nnz >= kSoloBeside && solo_fits(n_vars, m, max_deg)) {
+            try {
+                solo_made = std::async(std::launch::async, make_solo);
+            } catch (const std::system_error &) {  // no more threads
+                use_solo = make_solo();
+            }
+        } else {
+            use_solo = make_solo();
+        }
     }
     // the serving engine runs such an instance on that kernel alone: its
     // context holds none of the per-pass kernels' lists and buffers
     const bool solo_only = use_solo && pool_alloc;
     if (!solo_only && !on_dev) scatter_occurrences(n_vars, m, hc, block_rows ? &ro.row : nullptr);
-    std::vector<int64_t> solo_w;
-    if (use_solo && weights && !solo.slot.empty()) {
-        solo_w.resize((size_t)m);
-        for (int64_t j = 0; j < m; ++j) solo_w[(size_t)solo.slot[(size_t)j]] = weights[j];
-    }
     std::vector<int2> occx;
     if (expand) {
         occx.resize((size_t)nnz);
@@ -373,7 +395,6 @@ int msat::ctx_create(msat_ctx **out, int32_t n_vars, int64_t n_clauses, const in
     c->max_len = max_len;
     c->max_deg = max_deg;
     c->wsum = wsum;
-    c->clen = std::move(hc.clen);
     c->taut = std::move(hc.taut);
     if (weights) c->wts.assign(weights, weights + m);
     while (hc.wor >> c->wbits) ++c->wbits;
@@ -381,14 +402,24 @@ int msat::ctx_create(msat_ctx **out, int32_t n_vars, int64_t n_clauses, const in
     const int64_t nB = (int64_t)n_vars * B;
     int rc = MSAT_OK;
     int32_t *d_coff = nullptr, *d_lit = nullptr, *d_voff = nullptr, *d_occ = nullptr;
-    int32_t *d_hvar = nullptr, *d_hch = nullptr, *d_hofc = nullptr;
-    int2 *d_lblk = nullptr, *d_occx = nullptr;
+    int32_t *d_tab = nullptr;
+    int2 *d_occx = nullptr;
     int32_t *d_plit = nullptr, *d_pcoff = nullptr;
     int64_t *d_pw = nullptr;
     int64_t *d_w = nullptr;
     unsigned char *d_slists = nullptr;
-    int32_t *d_sperm = nullptr;
-    int64_t *d_sw = nullptr;
+    // heavy variables, their first chunks, the heavy variable of every chunk
+    // (one load per chunk block) and the light blocks: one array, one upload
+    std::vector<int32_t> tab;
+    auto tab_end = [&] { tab.resize((tab.size() + 3) & ~(size_t)3); return tab.size(); };
+    tab.insert(tab.end(), hvar.begin(), hvar.end());
+    const size_t tab_hch = tab_end();
+    tab.insert(tab.end(), hchunk0.begin(), hchunk0.end());
+    const size_t tab_hofc = tab_end();
+    for (size_t h = 0; h + 1 < hchunk0.size(); ++h) tab.insert(tab.end(), (size_t)(hchunk0[h + 1] - hchunk0[h]), (int32_t)h);
+    const size_t tab_lblk = tab_end();
+    tab.resize(tab_lblk + 2 * lblk.size());
+    if (!lblk.empty()) memcpy(tab.data() + tab_lblk, lblk.data(), sizeof(int2) * lblk.size());
 #define TRY_ALLOC(ptr, count)                          \
     do {                                               \
         rc = dalloc_t(c, &(ptr), (size_t)(count));     \
@@ -415,20 +446,12 @@ int msat::ctx_create(msat_ctx **out, int32_t n_vars, int64_t n_clauses, const in
         TRY_ALLOC(d_occ, nnz);
     }
     if (weights && !on_dev) TRY_ALLOC(d_w, m);
-    TRY_ALLOC(d_hvar, (int64_t)hvar.size());
-    TRY_ALLOC(d_hch, (int64_t)hchunk0.size());
-    TRY_ALLOC(d_hofc, std::max<int64_t>(1, hchunk0.back()));
-    TRY_ALLOC(d_lblk, (int64_t)lblk.size());
+    TRY_ALLOC(d_tab, (int64_t)tab.size());
     if (expand) TRY_ALLOC(d_occx, nnz);
     if (block_rows && !on_dev) {
         TRY_ALLOC(d_plit, nnz);
         if (kfix == 0) TRY_ALLOC(d_pcoff, m + 1);
         if (weights) TRY_ALLOC(d_pw, m);
-    }
-    if (use_solo) {
-        TRY_ALLOC(d_slists, solo.lists.size());
-        TRY_ALLOC(d_sperm, n_vars);
-        if (!solo_w.empty()) TRY_ALLOC(d_sw, m);
     }
     if (use_fstore && !solo_only) TRY_ALLOC(c->S.fstore, (m + 1) * B);
     TRY_ALLOC(c->S.x, nB);
@@ -452,40 +475,43 @@ int msat::ctx_create(msat_ctx **out, int32_t n_vars, int64_t n_clauses, const in
     I.heavy_deg = heavy_deg;
     I.n_heavy = (int32_t)hvar.size();
     I.heavy_chunks = hchunk0.back();
-    I.heavy_var = d_hvar;
-    I.heavy_chunk0 = d_hch;
-    I.heavy_of_chunk = d_hofc;
+    I.heavy_var = d_tab;
+    I.heavy_chunk0 = d_tab + tab_hch;
+    I.heavy_of_chunk = d_tab + tab_hofc;
     I.occ_shift = expand ? 3 : 1;
     I.occx = d_occx;
     I.n_lblk = (int32_t)lblk.size();
     I.task_cap = task_cap;
     I.fwd_vw = fwd_vw;
     I.stage_vw = stage_vw;
-    I.lblk = d_lblk;
+    I.lblk = reinterpret_cast<const int2 *>(d_tab + tab_lblk);
     I.plit = d_plit;
     I.pcoff = d_pcoff;
     I.pw = d_pw;
 
-    if (use_solo) {
-        c->solo = solo.dev;
-        c->solo.lists = d_slists;
-        c->solo.perm = d_sperm;
-        c->solo.w = d_sw ? d_sw : d_w;
-    }
-
     DevStep &D = c->D;
     D.fwd_blocks = cfg.fwd_blocks > 0 ? cfg.fwd_blocks : fwd_grid_blocks(I);
-    TRY_ALLOC(D.sc, 1);
-    TRY_ALLOC(D.wu_acc, (int64_t)kRep * B);
-    TRY_ALLOC(D.cost, B);
-    TRY_ALLOC(D.best, B);
-    TRY_ALLOC(D.best_step, B);
-    TRY_ALLOC(D.improved, B);
-    TRY_ALLOC(D.cscale, B);
-    TRY_ALLOC(D.loss, B);
-    TRY_ALLOC(D.lpart, (int64_t)D.fwd_blocks * B);
-    TRY_ALLOC(D.hpart, std::max<int64_t>(1, I.heavy_chunks) * B);
-    TRY_ALLOC(D.hcount, std::max<int64_t>(1, (int64_t)hvar.size() * G));
+    // the step's scalars and per-restart arrays: one allocation, each from a
+    // 256-byte boundary on; first the two that are uploaded, then those that
+    // start as zero
+    struct StatePart {
+        void **ptr;
+        size_t bytes;
+    };
+    auto part = [](auto *&p, int64_t count) {
+        return StatePart{reinterpret_cast<void **>(&p), (size_t)std::max<int64_t>(1, count) * sizeof(*p)};
+    };
+    const StatePart parts[] = {part(D.sc, 1), part(D.best, B),
+                               part(D.wu_acc, (int64_t)kRep * B), part(D.cost, B), part(D.best_step, B),
+                               part(D.improved, B), part(D.cscale, B), part(D.loss, B),
+                               part(D.hcount, (int64_t)hvar.size() * G),
+                               part(D.lpart, (int64_t)D.fwd_blocks * B), part(D.hpart, I.heavy_chunks * B)};
+    constexpr int kZeroFrom = 2, kZeroTo = 9, kParts = sizeof(parts) / sizeof(parts[0]);
+    size_t state_at[kParts + 1] = {0};
+    for (int k = 0; k < kParts; ++k) state_at[k + 1] = state_at[k] + ((parts[k].bytes + 255) & ~(size_t)255);
+    unsigned char *d_state = nullptr;
+    TRY_ALLOC(d_state, state_at[kParts]);
+    for (int k = 0; k < kParts; ++k) *parts[k].ptr = d_state + state_at[k];
 #undef TRY_ALLOC
 
     cudaStream_t st = c->stream;
@@ -510,7 +536,9 @@ int msat::ctx_create(msat_ctx **out, int32_t n_vars, int64_t n_clauses, const in
     sc.dense = 1;
     sc.wsum = wsum;
     sc.loss_norm = cfg.loss_norm;
-    std::vector<long long> best((size_t)B, (long long)wsum);
+    std::vector<unsigned char> state0(state_at[kZeroFrom]);
+    memcpy(state0.data(), &sc, sizeof(sc));
+    for (int b = 0; b < B; ++b) memcpy(state0.data() + state_at[1] + sizeof(long long) * (size_t)b, &wsum, sizeof(long long));
     cudaError_t e = cudaSuccess;
     const bool lists = !solo_only && !on_dev;
     if (!e && lists) e = up(d_coff, coff.data(), sizeof(int32_t) * coff.size());
@@ -518,33 +546,34 @@ int msat::ctx_create(msat_ctx **out, int32_t n_vars, int64_t n_clauses, const in
     if (!e && weights && !on_dev) e = up(d_w, weights, sizeof(int64_t) * (size_t)m);
     if (!e && lists) e = up(d_voff, voff.data(), sizeof(int32_t) * voff.size());
     if (!e && lists) e = up(d_occ, occ.data(), sizeof(int32_t) * occ.size());
-    if (!e) e = up(d_hvar, hvar.data(), sizeof(int32_t) * hvar.size());
-    if (!e) e = up(d_hch, hchunk0.data(), sizeof(int32_t) * hchunk0.size());
-    // the heavy variable of every chunk (one load per chunk block)
-    std::vector<int32_t> hofc((size_t)std::max<int32_t>(1, hchunk0.back()), 0);
-    for (size_t h = 0; h + 1 < hchunk0.size(); ++h)
-        for (int32_t ch = hchunk0[h]; ch < hchunk0[h + 1]; ++ch) hofc[(size_t)ch] = (int32_t)h;
-    if (!e) e = up(d_hofc, hofc.data(), sizeof(int32_t) * hofc.size());
-    if (!e) e = up(d_lblk, lblk.data(), sizeof(int2) * lblk.size());
+    if (!e) e = up(d_tab, tab.data(), sizeof(int32_t) * tab.size());
     if (!e && expand) e = up(d_occx, occx.data(), sizeof(int2) * occx.size());
     if (!e && block_rows && !on_dev) e = up(d_plit, ro.plit.data(), sizeof(int32_t) * ro.plit.size());
     if (!e && d_pcoff && !on_dev) e = up(d_pcoff, ro.pcoff.data(), sizeof(int32_t) * ro.pcoff.size());
     if (!e && d_pw && !on_dev) e = up(d_pw, ro.pw.data(), sizeof(int64_t) * ro.pw.size());
-    if (!e && use_solo) e = up(d_slists, solo.lists.data(), solo.lists.size());
-    if (!e && use_solo) e = up(d_sperm, solo.perm.data(), sizeof(int32_t) * solo.perm.size());
-    if (!e && d_sw) e = up(d_sw, solo_w.data(), sizeof(int64_t) * solo_w.size());
-    if (!e) e = up(D.sc, &sc, sizeof(sc));
-    if (!e) e = up(D.best, best.data(), sizeof(long long) * best.size());
-    if (!e) e = cudaMemsetAsync(D.best_step, 0, sizeof(long long) * (size_t)B, st);
-    if (!e) e = cudaMemsetAsync(D.wu_acc, 0, sizeof(unsigned long long) * (size_t)kRep * B, st);
-    if (!e) e = cudaMemsetAsync(D.improved, 0, sizeof(int) * (size_t)B, st);
-    if (!e) e = cudaMemsetAsync(D.cost, 0, sizeof(long long) * (size_t)B, st);
-    if (!e) e = cudaMemsetAsync(D.loss, 0, sizeof(float) * (size_t)B, st);
-    if (!e) e = cudaMemsetAsync(D.hcount, 0, sizeof(unsigned) * std::max<size_t>(1, hvar.size() * (size_t)G), st);
+    if (!e) e = up(d_state, state0.data(), state0.size());
+    if (!e) e = cudaMemsetAsync(d_state + state_at[kZeroFrom], 0, state_at[kZeroTo] - state_at[kZeroFrom], st);
     if (!e && !solo_only) e = cudaMemsetAsync(c->S.ubits, 0, sizeof(uint32_t) * (size_t)((m * B + 31) / 32 + 1), st);
     if (!e && c->S.fstore) e = cudaMemsetAsync(c->S.fstore + m * B, 0, sizeof(float) * (size_t)B, st);
     if (!e) e = launch_init(I, c->S, cfg.seed_x, st);
+    if (solo_made.valid()) use_solo = solo_made.get();
+    c->clen = std::move(hc.clen);
+    if (!e && use_solo) {
+        rc = dalloc_t(c, &d_slists, solo.lists.size());
+        if (!rc) {
+            e = up(d_slists, solo.lists.data(), solo.lists.size());
+            c->solo = solo.dev;
+            c->solo.lists = d_slists;
+            c->solo.perm = reinterpret_cast<const int *>(d_slists + solo.perm_at);
+            c->solo.w = solo.w_at ? reinterpret_cast<const int64_t *>(d_slists + solo.w_at) : d_w;
+        }
+    }
     if (!e) e = cudaStreamSynchronize(st);  // host vectors above are freed on return
+    if (rc) {
+        free_all(c);
+        delete c;
+        return rc;
+    }
     if (e) {
         rc = cuda_fail(e, "msat_create: upload / init");
         free_all(c);

@@ -107,7 +107,8 @@ int build_host_cnf(int32_t n, int64_t m, const int64_t *off, const int32_t *lits
     // unsat.  Short clauses compare pairwise; a long one marks literals and
     // variables in the thread's own arrays (marked with the clause index).
     struct Part {
-        std::vector<int32_t> lit;
+        I32Buf lit;       // room for the part's literals as they came
+        size_t n_lit = 0;
         int64_t wsum = 0, wor = 0;
         int32_t max_len = 0;
         int32_t first_len = -1;  // length of the part's first clause
@@ -120,9 +121,10 @@ int build_host_cnf(int32_t n, int64_t m, const int64_t *off, const int32_t *lits
     out.taut.assign((size_t)m, 0);
     parallel_ranges(m, Tm, [&](int t, int64_t b, int64_t e) {
         Part &P = parts[(size_t)t];
-        P.lit.reserve((size_t)(off[e] - off[b]));
+        P.lit.alloc((size_t)(off[e] - off[b]));
+        int32_t *d = P.lit.data();  // where the next literal goes
         for (int64_t j = b; j < e; ++j) {
-            const size_t start = P.lit.size();
+            const int32_t *const c = d;  // the clause so far: [c, d)
             const int64_t len_in = off[j + 1] - off[j];
             bool taut = false;
             if (len_in <= 32) {
@@ -130,11 +132,13 @@ int build_host_cnf(int32_t n, int64_t m, const int64_t *off, const int32_t *lits
                     const int32_t l = lits[p];
                     const int32_t packed = ((std::abs(l) - 1) << 1) | (l < 0 ? 1 : 0);
                     bool dup = false;
-                    for (size_t r = start; r < P.lit.size(); ++r) {
-                        if (P.lit[r] == packed) dup = true;
-                        else if ((P.lit[r] >> 1) == (packed >> 1)) taut = true;
+                    for (const int32_t *r = c; r < d; ++r) {
+                        const int32_t x = *r ^ packed;  // 0: the same literal, 1: the other of its variable
+                        dup |= x == 0;
+                        taut |= x == 1;
                     }
-                    if (!dup) P.lit.push_back(packed);
+                    *d = packed;
+                    d += !dup;
                 }
             } else {
                 if (P.seen.empty()) {
@@ -146,12 +150,12 @@ int build_host_cnf(int32_t n, int64_t m, const int64_t *off, const int32_t *lits
                     const int32_t packed = ((std::abs(l) - 1) << 1) | (l < 0 ? 1 : 0);
                     if (P.seen[(size_t)packed] == (int32_t)j) continue;
                     P.seen[(size_t)packed] = (int32_t)j;
-                    P.lit.push_back(packed);
+                    *d++ = packed;
                     if (P.vseen[(size_t)(packed >> 1)] == (int32_t)j) taut = true;
                     P.vseen[(size_t)(packed >> 1)] = (int32_t)j;
                 }
             }
-            const int32_t len = (int32_t)(P.lit.size() - start);
+            const int32_t len = (int32_t)(d - c);
             if (P.first_len < 0) P.first_len = len;
             P.same_len = P.same_len && len == P.first_len;
             if (len > kMaxClauseLen && P.too_long < 0) P.too_long = j;
@@ -161,6 +165,7 @@ int build_host_cnf(int32_t n, int64_t m, const int64_t *off, const int32_t *lits
             P.wsum += w ? w[j] : 1;
             if (w) P.wor |= w[j];
         }
+        P.n_lit = (size_t)(d - P.lit.data());
     });
     for (const Part &P : parts)
         if (P.too_long >= 0)
@@ -172,7 +177,7 @@ int build_host_cnf(int32_t n, int64_t m, const int64_t *off, const int32_t *lits
     out.wsum = 0;
     out.max_len = 0;
     for (int t = 0; t < Tm; ++t) {
-        lbase[(size_t)t + 1] = lbase[(size_t)t] + (int64_t)parts[(size_t)t].lit.size();
+        lbase[(size_t)t + 1] = lbase[(size_t)t] + (int64_t)parts[(size_t)t].n_lit;
         out.wsum += parts[(size_t)t].wsum;
         out.wor |= parts[(size_t)t].wor;
         out.max_len = std::max(out.max_len, parts[(size_t)t].max_len);
@@ -183,7 +188,7 @@ int build_host_cnf(int32_t n, int64_t m, const int64_t *off, const int32_t *lits
     out.coff[0] = 0;
     parallel_ranges(m, Tm, [&](int t, int64_t b, int64_t e) {
         const Part &P = parts[(size_t)t];
-        std::copy(P.lit.begin(), P.lit.end(), out.lit.data() + lbase[(size_t)t]);
+        std::copy(P.lit.data(), P.lit.data() + P.n_lit, out.lit.data() + lbase[(size_t)t]);
         int64_t at = lbase[(size_t)t];
         for (int64_t j = b; j < e; ++j) {
             at += out.clen[(size_t)j];

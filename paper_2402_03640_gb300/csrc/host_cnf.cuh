@@ -81,15 +81,19 @@ int build_block_rows(int32_t n, int64_t m, int32_t kfix, const I32Buf &coff, con
 void scatter_occurrences(int32_t n, int64_t m, HostCnf &hc, const I32Buf *row);
 
 // Lists of the one-block-per-restart step kernel (k_solo.cu) of a canonical
-// CNF; false where the instance does not fit one SM's shared memory.  dev
-// holds the sizes and offsets (its pointers are set after the upload).
+// CNF; false where the instance does not fit one SM's shared memory (no
+// instance without solo_fits does).  dev holds the sizes and offsets (its
+// pointers are set after the upload); behind the lists, in the same array, lie
+// the internal variable order -> variable table and, where the clauses are in
+// another order, the weights in slot order (w_at 0: there are none).  Reads
+// coff, lit, voff and clen of hc.
 struct SoloHost {
     SoloDev dev;
     std::vector<unsigned char> lists;
-    std::vector<int32_t> perm;  // internal variable order -> variable
-    std::vector<int32_t> slot;  // clause -> slot, empty: clause order
+    size_t perm_at = 0, w_at = 0;
 };
+bool solo_fits(int32_t n, int64_t m, int32_t max_deg);
 bool build_solo(int32_t n, int64_t m, int32_t kfix, int32_t max_len, int32_t max_deg, const HostCnf &hc,
-                SoloHost &out);
+                const int64_t *w, SoloHost &out);
 
 }  // namespace msat

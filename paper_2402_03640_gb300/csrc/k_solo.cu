@@ -516,12 +516,16 @@ struct SoloShape {
 
 }  // namespace
 
-bool build_solo(int32_t n, int64_t m, int32_t kfix, int32_t max_len, int32_t max_deg, const HostCnf &hc,
-                SoloHost &out) {
+bool solo_fits(int32_t n, int64_t m, int32_t max_deg) {
     // 16-bit words: var << 1 | neg with the dummy variable n, slots up to the
     // dummy clause m
-    if (n > 32766 || m > 65534 || max_deg > 32 * 1024) return false;
-    if (solo_smem(n, (int)m, 0, false, 0).total > kSoloSmemMax) return false;
+    return n <= 32766 && m <= 65534 && max_deg <= 32 * 1024 &&
+           solo_smem(n, (int)m, 0, false, 0).total <= kSoloSmemMax;
+}
+
+bool build_solo(int32_t n, int64_t m, int32_t kfix, int32_t max_len, int32_t max_deg, const HostCnf &hc,
+                const int64_t *w, SoloHost &out) {
+    if (!solo_fits(n, m, max_deg)) return false;
     SoloDev &V = out.dev;
     V = SoloDev{};
     const int32_t *coff = hc.coff.data(), *lit = hc.lit.data(), *voff = hc.voff.data();
@@ -529,7 +533,7 @@ bool build_solo(int32_t n, int64_t m, int32_t kfix, int32_t max_len, int32_t max
     // variables: one leaf first (longest first), then several leaves (those a
     // warp combines first)
     auto leaves = [&](int32_t i) { return (voff[i + 1] - voff[i] + 31) / 32; };
-    out.perm.resize((size_t)n);
+    std::vector<int32_t> perm((size_t)n);
     SoloShape sh;
     {
         int32_t cnt[10] = {0};
@@ -549,7 +553,7 @@ bool build_solo(int32_t n, int64_t m, int32_t kfix, int32_t max_len, int32_t max
         for (int32_t i = 0; i < n; ++i) {
             const int32_t d = voff[i + 1] - voff[i];
             const int32_t id = d <= 32 ? at[8 - (d + 3) / 4]++ : leaves(i) > kNarrowLeaves ? wide++ : narrow++;
-            out.perm[(size_t)id] = i;
+            perm[(size_t)id] = i;
         }
     }
     if (solo_smem(n, (int)m, sh.n_mtask, false, 0).total > kSoloSmemMax) return false;
@@ -591,7 +595,7 @@ bool build_solo(int32_t n, int64_t m, int32_t kfix, int32_t max_len, int32_t max
     {
         int32_t k = 0;
         for (int32_t h = 0; h < sh.n_multi; ++h) {
-            const int32_t i = out.perm[(size_t)(sh.n_single + h)];
+            const int32_t i = perm[(size_t)(sh.n_single + h)];
             const int32_t d = voff[i + 1] - voff[i];
             tfirst[(size_t)(sh.n_single + h)] = k;
             mbeg[(size_t)h] = k;
@@ -599,7 +603,7 @@ bool build_solo(int32_t n, int64_t m, int32_t kfix, int32_t max_len, int32_t max
         }
         mbeg[(size_t)sh.n_multi] = k;
         for (int32_t id = 0; id < sh.n_single; ++id) {
-            const int32_t i = out.perm[(size_t)id];
+            const int32_t i = perm[(size_t)id];
             tfirst[(size_t)id] = k;
             tlen[(size_t)k++] = (uint8_t)(voff[i + 1] - voff[i]);
         }
@@ -626,6 +630,11 @@ bool build_solo(int32_t n, int64_t m, int32_t kfix, int32_t max_len, int32_t max
     place(V.off_sgn, sizeof(uint32_t) * (size_t)n_task);
     place(V.off_mbeg, sizeof(int32_t) * mbeg.size());
     V.list_bytes = at;
+    uint32_t perm_at = 0, w_at = 0;
+    place(perm_at, sizeof(int32_t) * (size_t)n);
+    if (w && !slot.empty()) place(w_at, sizeof(int64_t) * (size_t)m);
+    out.perm_at = perm_at;
+    out.w_at = w_at;
     out.lists.assign(at, 0);
     uint16_t *lw = reinterpret_cast<uint16_t *>(out.lists.data() + V.off_lit);
     uint16_t *ow = reinterpret_cast<uint16_t *>(out.lists.data() + V.off_occ);
@@ -644,7 +653,7 @@ bool build_solo(int32_t n, int64_t m, int32_t kfix, int32_t max_len, int32_t max
     auto leaf_at = [&](uint32_t k) { return ((uint32_t)obase[k >> 5] * 32u + (k & 31u)) * 4u; };
     for (int32_t id = 0; id < n; ++id) {
         const uint32_t k = (uint32_t)tfirst[(size_t)id];
-        fill[(size_t)out.perm[(size_t)id]] = Fill{(uint32_t)id << 1, leaf_at(k), k, 0u, 0u};
+        fill[(size_t)perm[(size_t)id]] = Fill{(uint32_t)id << 1, leaf_at(k), k, 0u, 0u};
     }
     const uint32_t pairs = V.pairs ? 1u : 0u;
     for (int64_t j = 0; j < m; ++j) {
@@ -668,7 +677,11 @@ bool build_solo(int32_t n, int64_t m, int32_t kfix, int32_t max_len, int32_t max
         }
     }
     for (const Fill &F : fill) sg[F.task] = F.sgn;
-    out.slot = std::move(slot);
+    std::copy(perm.begin(), perm.end(), reinterpret_cast<int32_t *>(out.lists.data() + perm_at));
+    if (w_at) {
+        int64_t *sw = reinterpret_cast<int64_t *>(out.lists.data() + w_at);
+        for (int64_t j = 0; j < m; ++j) sw[slot[(size_t)j]] = w[j];
+    }
     V.n_single = sh.n_single;
     V.n_multi = sh.n_multi;
     V.n_wide = sh.n_wide;
