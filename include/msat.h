@@ -293,6 +293,13 @@ int msat_selftest_scratch_limit(msat_ctx *ctx, int64_t bytes);
 int msat_selftest_preparation(msat_ctx *ctx, int32_t *route);
 
 /*
+ * Self-test of the two step routes, which give the same bits: whether a call
+ * of n_steps steps (without MSAT_STEP_PER_PASS and kernel timing) takes the
+ * one-block-per-restart kernel (1) or the per-pass kernels (0).
+ */
+int msat_selftest_step_route(msat_ctx *ctx, int64_t n_steps, int32_t *solo);
+
+/*
  * Measured peak of the dense backend's tensor-core instruction (no
  * counterpart in the paper; a benchmark helper): every SM issues `iters`
  * stages of four block-scaled kind::mxf4 MMAs (M = 128 clauses, N =

@@ -668,14 +668,17 @@ static cudaError_t plain_steps(msat_ctx *c, int64_t n_steps) {
     return e;
 }
 
+static bool takes_solo(const msat_ctx *c, int64_t k) {
+    return c->solo.lists && solo_pays(c->solo, c->I, c->nnz, c->max_len, k, 1.0);
+}
+
 // k steps and, if asked, the evaluation of the final x by the fastest route
 // that gives the same bits: the one-block-per-restart kernel for small
 // instances, captured graphs when asked, else plain launches (always plain
 // while kernel timing is on, so every pass is timed).
 static cudaError_t run_steps(msat_ctx *c, int64_t k, uint32_t flags, bool final_eval) {
     cudaError_t e = cudaSuccess;
-    if (!c->prof_on && !(flags & MSAT_STEP_PER_PASS) && c->solo.lists &&
-        solo_pays(c->solo, c->I, c->nnz, c->max_len, k, 1.0)) {
+    if (!c->prof_on && !(flags & MSAT_STEP_PER_PASS) && takes_solo(c, k)) {
         for (int64_t done = 0; !e;) {
             const int64_t now = std::min<int64_t>(k - done, 1 << 30);
             done += now;
@@ -1284,6 +1287,12 @@ extern "C" int msat_selftest_scratch_limit(msat_ctx *c, int64_t bytes) {
 extern "C" int msat_selftest_preparation(msat_ctx *c, int32_t *route) {
     if (!c || !route) return fail(MSAT_EINVAL, "msat_selftest_preparation: NULL argument");
     *route = c->prep_route;
+    return MSAT_OK;
+}
+
+extern "C" int msat_selftest_step_route(msat_ctx *c, int64_t n_steps, int32_t *solo) {
+    if (!c || !solo) return fail(MSAT_EINVAL, "msat_selftest_step_route: NULL argument");
+    *solo = takes_solo(c, n_steps);
     return MSAT_OK;
 }
 

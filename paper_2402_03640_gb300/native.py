@@ -145,6 +145,7 @@ def load(build_if_missing: bool = False) -> ctypes.CDLL:
             "msat_selftest_bounded_wait": ([i64], ctypes.c_int),
             "msat_selftest_scratch_limit": ([P, i64], ctypes.c_int),
             "msat_selftest_preparation": ([P, P], ctypes.c_int),
+            "msat_selftest_step_route": ([P, i64, P], ctypes.c_int),
             "msat_dense_mma_rate": ([i32, i32, P], ctypes.c_int),
             "msat_best_step": ([P, P], ctypes.c_int),
             "msat_profile_enable": ([P, ctypes.c_int], ctypes.c_int),
