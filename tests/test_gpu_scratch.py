@@ -233,3 +233,32 @@ def test_best_without_scratch(pkg):
         for limit in (0, cnf.n * 64 - 1, -1):
             s._lib.msat_selftest_scratch_limit(s._ctx, limit)
             assert np.array_equal(s.best()[0], want), limit
+
+
+@pytest.mark.parametrize("call", ["msat_get_x", "msat_best", "msat_get_state"])
+def test_a_refused_copy_leaves_the_array_alone(pkg, call):
+    """A call that cannot copy (its stream is being captured) gives an error
+    and has not written to the caller's array."""
+    import ctypes
+
+    import torch
+    cnf = uniform_ksat(300000, 1000, 3, seed=5)
+    rt = ctypes.CDLL("libcudart.so.%s" % torch.version.cuda.split(".")[0])
+    st = torch.cuda.Stream()
+    raw = ctypes.c_void_p(st.cuda_stream)
+    with pkg.Solver.from_cnf(cnf, restarts=4, stream=st) as s:
+        a = np.full(4 * cnf.n * (1 if call == "msat_best" else 4), 0x5a, np.uint8)
+        args = {"msat_get_x": (a.ctypes.data,), "msat_best": (a.ctypes.data, None),
+                "msat_get_state": (a.ctypes.data, None, None, None, None, None, None)}[call]
+        fn = getattr(s._lib, call)
+        torch.cuda.synchronize()
+        graph = ctypes.c_void_p()
+        assert rt.cudaStreamBeginCapture(raw, 1) == 0  # this thread's calls
+        rc = fn(s._ctx, *(None if v is None else ctypes.c_void_p(v) for v in args))
+        rt.cudaStreamEndCapture(raw, ctypes.byref(graph))
+        rt.cudaGetLastError()
+        if graph.value:
+            rt.cudaGraphDestroy(graph)
+        assert rc != 0
+        assert (a == 0x5a).all()
+        assert s.x().shape[0] == cnf.n  # and the context goes on
