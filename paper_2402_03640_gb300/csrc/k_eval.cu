@@ -295,8 +295,8 @@ cudaError_t launch_eval_sparse(const DevInst &I, const int8_t *a, const float *x
         }
         return e;
     }
-    for (int b0 = 0; b0 < nb && e == cudaSuccess; b0 += chunk) {
-        const int k = std::min(chunk, nb - b0);
+    for (long long b0 = 0; b0 < nb && e == cudaSuccess; b0 += chunk) {  // past 2^31 behind the last part
+        const int k = (int)std::min<long long>(chunk, nb - b0);
         const int8_t *ak = a ? a + b0 : nullptr;
         const float *xk = a ? nullptr : x + b0;
         unsigned long long *cost = reinterpret_cast<unsigned long long *>(cost_out) + b0;

@@ -50,3 +50,11 @@ def test_gradient_scale_is_read_behind_the_wait():
     text = re.sub(r"//[^\n]*", "", open(os.path.join(CSRC, "k_step.cu")).read())
     assert not re.search(r"gscale\s*\[|\*\s*gscale\b(?!,|\))", text)
     assert "ld_ordered(gscale + " in text
+
+
+def test_parts_of_a_batch_are_counted_in_64_bits():
+    """launch_eval_sparse takes a batch in parts: the position behind the last
+    part of a batch of nearly 2^31 assignments is past 32 bits."""
+    body = _body("k_eval.cu", "cudaError_t launch_eval_sparse")
+    loops = re.findall(r"for \((.*?) b0 = 0;", body)
+    assert loops == ["long long", "long long"]
