@@ -935,7 +935,8 @@ static int sparse_eval(msat_ctx *c, const int8_t *a, const float *x, int32_t nb,
     bool packed = false;
     if (!eval_is_direct(c->nnz, nb) && !captured()) {
         constexpr int kGroup = 128;
-        const int64_t groups = (256LL << 20) / (int64_t)eval_sparse_bytes(c->n, kGroup);
+        // 65535: a launch's limit on the groups of the batch
+        const int64_t groups = std::min<int64_t>(65535, (256LL << 20) / (int64_t)eval_sparse_bytes(c->n, kGroup));
         int chunk = (int)std::min<int64_t>(nb, std::max<int64_t>(1, groups) * kGroup);
         std::lock_guard<std::mutex> lk(c->scratch.mu);
         uint32_t *bits = scratch_take(c, eval_sparse_bytes(c->n, chunk), st);

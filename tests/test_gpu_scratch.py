@@ -139,6 +139,19 @@ def test_captured_evaluation_of_very_many_assignments(pkg):
         assert np.array_equal(out.cpu().numpy(), want)
 
 
+def test_evaluation_past_a_launch_of_packed_groups(pkg):
+    """More groups of 128 assignments than a launch takes."""
+    import torch
+    from synth import Cnf
+    cnf = Cnf.from_clauses(2, [[1, 2], [-1], [1, -2]], weights=[5, 3, 1 << 33])
+    nb = 65535 * 128 + 129
+    a = torch.randint(0, 2, (2, nb), device="cuda", dtype=torch.int8) * 2 - 1
+    t = a > 0
+    want = 5 * (~(t[0] | t[1])).long() + 3 * t[0].long() + (1 << 33) * (~t[0] & t[1]).long()
+    with pkg.Solver.from_cnf(cnf, restarts=1) as s:
+        assert torch.equal(s.evaluate(a, "sparse"), want)
+
+
 def test_evaluation_without_scratch(pkg, batches):
     """Where the packed batch cannot be allocated, 128 assignments' worth of
     it, and where that cannot be had the kernel without scratch, give the same
