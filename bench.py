@@ -996,11 +996,13 @@ def run_serving(args):
     return 0
 
 
-# a kernel's sources and those of the data layout it reads (host_cnf.cu
-# builds the row order of the stored w f)
-KERNEL_SOURCES = {"forward": ("k_step.cu", "step_math.cuh", "msat_internal.cuh", "host_cnf.cu"),
-                  "backward": ("k_step.cu", "step_math.cuh", "msat_internal.cuh", "host_cnf.cu"),
-                  "dense_eval": ("k_dense.cu", "msat_internal.cuh"),
+# a kernel's sources and those of the data layout it reads (dev_cnf.cu and, for
+# the instances it does not take, host_cnf.cu build the row order of the stored
+# w f) and of the overlap of its launches (pdl.cuh)
+STEP_SOURCES = ("k_step.cu", "step_math.cuh", "pdl.cuh", "msat_internal.cuh", "dev_cnf.cu", "host_cnf.cu")
+KERNEL_SOURCES = {"forward": STEP_SOURCES,
+                  "backward": STEP_SOURCES,
+                  "dense_eval": ("k_dense.cu", "bits.cuh", "pdl.cuh", "msat_internal.cuh"),
                   "small_steps": ("k_solo.cu", "step_math.cuh", "msat_internal.cuh")}
 
 

@@ -19,8 +19,9 @@
 // The form before it gave each lane one assignment and read 32 bytes of a
 // per literal and 32 assignments, about 42 instructions for 32 (clause,
 // assignment) pairs where this one takes about 150 for 4096.  Weighted Zipf
-// n=2e5, m=1e6, 100 assignments: 695 -> 53
-// us a call (14 packing, 36 evaluation, the rest launches).
+// n=2e5, m=1e6, 100 assignments: 697 -> 59
+// us a call (14 packing, 36 evaluation, the rest launches and the order among
+// the users of the scratch).
 
 #include <cuda_runtime.h>
 #include <stdint.h>

@@ -6,17 +6,21 @@
 //                     loss partials per restart; the last block to finish
 //                     turns them into cost, best, 2/W_U and the Adam scalars
 //   k_backward_light  variable pass over the transposed CSR for variables
-//                     with few occurrences: occurrence terms staged in shared
-//                     memory, then per variable the fixed-order sum, 1 - t^2,
-//                     fused Adam update, best-assignment capture and tanh
+//                     with few occurrences: a thread sums the terms of one
+//                     32-occurrence leaf straight from their gathers, then
+//                     1 - t^2, fused Adam update, best-assignment capture and
+//                     tanh; the leaves of a longer variable meet in shared
+//                     memory
 //   k_backward_heavy  the same for variables with many occurrences, split
-//                     into 1024-occurrence chunks combined in the fixed order
+//                     into 1024-occurrence chunks, a warp each, combined in
+//                     the fixed order
 //
 // Layouts: x, mom, vel, t are float [n][B] (restart index innermost), so the
 // B values of one variable are one contiguous, vector-loadable row.  A
 // thread owns VW consecutive restarts of one clause, occurrence or variable:
-// up to 8 in the clause pass, up to 16 when staging occurrence terms, up to
-// 4 in the update (where every restart carries x, m, v, t and the sums).
+// up to 8 in the clause pass, 4 of a leaf in the variable pass (up to 16 where
+// the caller's launch shape says so), up to 4 in the update (where every
+// restart carries x, m, v, t and the sums).
 
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -616,7 +620,8 @@ constexpr int kWarps = kThreads / 32;
 
 __host__ __device__ inline int loss_blocks(int B) { return (B + kWarps - 1) / kWarps; }
 
-// s + lo += v, the rounding error of the addition collected in lo.
+// s + lo += v, the rounding error of the addition (Knuth's error-free sum of
+// two floats) collected in lo.
 __device__ __forceinline__ void add_two(float &s, float &lo, float v) {
     const float t = s + v, z = t - s;
     lo += (s - (t - z)) + (v - z);
@@ -659,11 +664,12 @@ __host__ __device__ constexpr bool takes_loss(int VW, int B) { return VW <= 4 &&
 bool probe_takes_loss(const DevInst &I) { return takes_loss(I.fwd_vw, I.B); }
 
 // --------------------------------------------------------------- k_forward
-// One item = (clause j, restart group g of VW restarts).  For VW <= 4 the
-// grid-stride loop is unrolled by two (items base + lane and base + stride +
-// lane; the stride is a multiple of G, so both belong to the thread's
-// restart group), keeping the loads of two clauses in flight; wider groups
-// already have VW/4 row loads per literal in flight.  The unsat bits of 32
+// One item = (clause j, restart group g of VW restarts).  Where the rows of
+// two clauses leave the registers for it (fwd_items: VW <= 4, and for k = 4
+// and 5 VW <= 2) the grid-stride loop is unrolled by two (items base + lane
+// and base + stride + lane; the stride is a multiple of G, so both belong to
+// the thread's restart group), keeping the loads of two clauses in flight;
+// wider groups already have several row loads per literal in flight.  The unsat bits of 32
 // consecutive items are packed with shuffles into whole 32-bit words.
 
 template <int VW, int KFIX>

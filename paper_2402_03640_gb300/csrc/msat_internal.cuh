@@ -300,8 +300,9 @@ cudaError_t launch_backward(const DevInst &I, const DevState &S, const DevStep &
 cudaError_t launch_tanh(const float *x, float *t, int64_t count, cudaStream_t st);
 cudaError_t launch_transpose_u8(const uint8_t *in, uint8_t *out, int rows, int cols, cudaStream_t st);
 // Batched step over nslot instances (all with the same B and launch shape,
-// f stored by the clause pass; variable-length clause path): fwd_start / heavy_start / light_start are device int[nslot+1]
-// block prefixes; totals are the grid sizes.
+// f stored by the clause pass, which takes each instance's common clause
+// length): fwd_start / heavy_start / light_start are device int[nslot+1] block
+// prefixes; totals are the grid sizes.
 cudaError_t launch_step_batch(const SlotDesc *slots, int nslot, const int *fwd_start, int fwd_total,
                               const int *heavy_start, int heavy_total, const int *light_start,
                               int light_total, int B, int fwd_vw, int stage_vw, int task_cap,
