@@ -922,7 +922,7 @@ static int sparse_eval(msat_ctx *c, const int8_t *a, const float *x, int32_t nb,
     const cudaStream_t st = c->stream;
     auto run = [&](int chunk, uint32_t *bits) {
         prof_begin(c, PROF_EVAL);
-        const cudaError_t e = launch_eval_sparse(c->I, a, x, nb, chunk, c->wbits, bits, (long long *)cost_out, st);
+        const cudaError_t e = launch_eval_sparse(c->I, a, x, nb, chunk, c->wbits, c->max_len, bits, (long long *)cost_out, st);
         prof_end(c);
         return e;
     };
@@ -933,7 +933,7 @@ static int sparse_eval(msat_ctx *c, const int8_t *a, const float *x, int32_t nb,
     };
     cudaError_t e = cudaSuccess;
     bool packed = false;
-    if (!eval_is_direct(c->nnz, nb) && !captured()) {
+    if (!eval_is_direct(c->nnz, c->max_len, nb) && !captured()) {
         constexpr int kGroup = 128;
         // 65535: a launch's limit on the groups of the batch
         const int64_t groups = std::min<int64_t>(65535, (256LL << 20) / (int64_t)eval_sparse_bytes(c->n, kGroup));

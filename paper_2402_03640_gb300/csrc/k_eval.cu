@@ -37,6 +37,8 @@ namespace {
 
 constexpr int kEvalWarps = kThreads / 32;
 constexpr int kLitBatch = 4;  // literals whose loads and gathers are in flight together
+// Clauses of more literals are read by the whole warp.
+constexpr int kLongClause = 32;
 
 // What the evaluation reads of an instance (a launch copies its arguments).
 struct EvalInst {
@@ -118,10 +120,33 @@ __global__ void __launch_bounds__(kThreads)
     }
 }
 
-// wbits: bits of the largest clause weight (0: every weight is 1).
+// ors the values of literals L (-1: none) into sat, all their rows in flight.
 template <int VW>
+__device__ __forceinline__ void gather_or(const uint32_t *__restrict__ bits, int wpr, int word0,
+                                          const int (&L)[kLitBatch], uint32_t (&sat)[VW]) {
+    uint32_t row[kLitBatch][VW];
+#pragma unroll
+    for (int k = 0; k < kLitBatch; ++k)
+        if (L[k] >= 0) ld_words<VW>(bits + (long long)(L[k] >> 1) * wpr + word0, row[k]);
+#pragma unroll
+    for (int k = 0; k < kLitBatch; ++k) {
+        if (L[k] < 0) continue;
+        const uint32_t neg = (L[k] & 1) ? 0xffffffffu : 0u;
+#pragma unroll
+        for (int v = 0; v < VW; ++v) sat[v] |= row[k][v] ^ neg;
+    }
+}
+
+// wbits: bits of the largest clause weight (0: every weight is 1).  cpw:
+// clauses a warp takes at a time, in its first lanes.  LONG: there are clauses
+// of more than kLongClause literals, which the warp reads together, its lanes'
+// ors then joined; a lane a clause, they are the longest chain of a call that
+// keeps few warps busy.  300 clauses of 100..300 literals, 100 / 256 assignments
+// 53.7 / 60.0 -> 24.3 / 24.4 us a call (42.9 / 44.8 before batches were packed), one
+// clause of 15000 literals among 40000 of three, 100 assignments 1757 -> 77 (1344).
+template <int VW, bool LONG>
 __global__ void __launch_bounds__(kThreads)
-    k_eval_sparse(EvalInst I, const uint32_t *__restrict__ bits, int wpr, int nb, int wbits,
+    k_eval_sparse(EvalInst I, const uint32_t *__restrict__ bits, int wpr, int nb, int wbits, int cpw,
                   unsigned long long *__restrict__ cost) {
     __shared__ unsigned long long s_acc[kEvalWarps][32 * VW];
     const int lane = threadIdx.x & 31;
@@ -130,10 +155,10 @@ __global__ void __launch_bounds__(kThreads)
     unsigned long long acc[VW];
 #pragma unroll
     for (int v = 0; v < VW; ++v) acc[v] = 0;
-    for (long long j0 = ((long long)blockIdx.x * kEvalWarps + warp) * 32; j0 < I.m;
-         j0 += (long long)gridDim.x * kEvalWarps * 32) {
+    for (long long j0 = ((long long)blockIdx.x * kEvalWarps + warp) * cpw; j0 < I.m;
+         j0 += (long long)gridDim.x * kEvalWarps * cpw) {
         const long long j = j0 + lane;
-        const bool live = j < I.m;
+        const bool live = j < I.m && lane < cpw;
         int beg = 0, end = 0;
         if (live) {
             if (I.kfix > 0) {
@@ -147,23 +172,36 @@ __global__ void __launch_bounds__(kThreads)
         uint32_t sat[VW];
 #pragma unroll
         for (int v = 0; v < VW; ++v) sat[v] = live ? 0u : 0xffffffffu;
-        for (int p0 = beg; p0 < end; p0 += kLitBatch) {
+        const int len = end - beg;
+        const bool joint = LONG && len > kLongClause;
+        for (int p0 = 0; p0 < (joint ? 0 : len); p0 += kLitBatch) {
             int L[kLitBatch];
-            uint32_t row[kLitBatch][VW];
 #pragma unroll
-            for (int k = 0; k < kLitBatch; ++k) L[k] = p0 + k < end ? __ldg(I.lit + p0 + k) : -1;
-#pragma unroll
-            for (int k = 0; k < kLitBatch; ++k)
-                if (L[k] >= 0) ld_words<VW>(bits + (long long)(L[k] >> 1) * wpr + word0, row[k]);
-#pragma unroll
-            for (int k = 0; k < kLitBatch; ++k) {
-                if (L[k] < 0) continue;
-                const uint32_t neg = (L[k] & 1) ? 0xffffffffu : 0u;
-#pragma unroll
-                for (int v = 0; v < VW; ++v) sat[v] |= row[k][v] ^ neg;
-            }
+            for (int k = 0; k < kLitBatch; ++k) L[k] = p0 + k < len ? __ldg(I.lit + beg + p0 + k) : -1;
+            gather_or<VW>(bits, wpr, word0, L, sat);
         }
         __syncwarp();
+        if constexpr (LONG) {
+            for (unsigned todo = __ballot_sync(0xffffffffu, joint); todo; todo &= todo - 1) {
+                const int src = __ffs(todo) - 1;
+                const int cb = __shfl_sync(0xffffffffu, beg, src), cl = __shfl_sync(0xffffffffu, len, src);
+                uint32_t any[VW];
+#pragma unroll
+                for (int v = 0; v < VW; ++v) any[v] = 0u;
+                for (int p0 = lane; p0 < cl; p0 += 32 * kLitBatch) {
+                    int L[kLitBatch];
+#pragma unroll
+                    for (int k = 0; k < kLitBatch; ++k) L[k] = p0 + 32 * k < cl ? __ldg(I.lit + cb + p0 + 32 * k) : -1;
+                    gather_or<VW>(bits, wpr, word0, L, any);
+                }
+                __syncwarp();
+#pragma unroll
+                for (int v = 0; v < VW; ++v) {
+                    const uint32_t r = __reduce_or_sync(0xffffffffu, any[v]);
+                    if (lane == src) sat[v] = r;
+                }
+            }
+        }
         uint32_t un[VW];  // lane b: the unsat bits of the warp's 32 clauses under assignment b
 #pragma unroll
         for (int v = 0; v < VW; ++v) un[v] = transpose_bits32(~sat[v], lane);
@@ -198,9 +236,10 @@ __global__ void __launch_bounds__(kThreads)
 
 // Small batches of small instances, and calls that may not have scratch, in
 // one launch: a lane is one assignment and a warp walks clauses, reading 32
-// entries of a variable's row (of `row` entries, the first nb evaluated) per
-// literal.
-template <typename T>
+// entries of a variable's row per literal.  PART: the first nb entries of rows
+// of `row`; whole batches have a form of their own, which is faster (300
+// clauses of 100..300 literals, 32 assignments 43 us, 52 with the row apart).
+template <typename T, bool PART>
 __global__ void __launch_bounds__(kThreads)
     k_eval_direct(EvalInst I, const T *__restrict__ a, int row, int nb, unsigned long long *__restrict__ cost) {
     __shared__ unsigned long long s_acc[kEvalWarps][32];
@@ -208,6 +247,7 @@ __global__ void __launch_bounds__(kThreads)
     const int warp = threadIdx.x >> 5;
     const int b = blockIdx.y * 32 + lane;
     const bool live = b < nb;
+    const int stride = PART ? row : nb;
     unsigned long long acc = 0;
     for (long long j = (long long)blockIdx.x * kEvalWarps + warp; j < I.m; j += (long long)gridDim.x * kEvalWarps) {
         const int beg = I.kfix > 0 ? (int)j * I.kfix : __ldg(I.coff + j);
@@ -215,7 +255,7 @@ __global__ void __launch_bounds__(kThreads)
         bool sat = false;
         for (int p = beg; p < end; ++p) {
             const int L = __ldg(I.lit + p);
-            const T v = live ? __ldg(a + (long long)(L >> 1) * row + b) : T(0);
+            const T v = live ? __ldg(a + (long long)(L >> 1) * stride + b) : T(0);
             sat |= is_true(v) != (bool)(L & 1);
         }
         if (!sat) acc += I.w ? (unsigned long long)__ldg(I.w + j) : 1ull;
@@ -239,7 +279,11 @@ __global__ void __launch_bounds__(kThreads)
 // 1) 23.0 / 10.9.
 constexpr long long kDirectReads = 96 << 10;
 
-bool eval_is_direct(int64_t nnz, int nb) { return nnz * ((nb + 31) / 32) <= kDirectReads; }
+// Long clauses are read by a whole warp only when packed (300 clauses of 100..300
+// literals, 1 assignment: 35 / 23).
+bool eval_is_direct(int64_t nnz, int max_len, int nb) {
+    return max_len <= kLongClause && nnz * ((nb + 31) / 32) <= kDirectReads;
+}
 
 // Words a lane carries: rows of up to 128 assignments are one load.
 static int eval_vw(int nb) { return nb > 64 ? 4 : nb > 32 ? 2 : 1; }
@@ -254,7 +298,7 @@ size_t eval_sparse_bytes(int n, int nb) { return sizeof(uint32_t) * (size_t)n * 
 
 template <int VW>
 static void launch_eval_vw(const DevInst &I, const int8_t *a, const float *x, int row, int nb, int wbits,
-                           uint32_t *bits, unsigned long long *cost, cudaStream_t st) {
+                           int max_len, uint32_t *bits, unsigned long long *cost, cudaStream_t st) {
     const int wpr = eval_wpr(nb);
     const long long rows4 = ((long long)I.n * VW + 3) / 4;  // warp iterations of the packing
     const unsigned pb = (unsigned)std::min<long long>((rows4 + kEvalWarps - 1) / kEvalWarps, 152LL * 8);
@@ -264,11 +308,17 @@ static void launch_eval_vw(const DevInst &I, const int8_t *a, const float *x, in
     else if (a) k_pack_bits<int8_t, VW, false><<<pb, kThreads, 0, st>>>(a, I.n, row, nb, wpr, bits, cost);
     else k_pack_bits<float, VW, false><<<pb, kThreads, 0, st>>>(x, I.n, row, nb, wpr, bits, cost);
     const int gy = wpr / VW;
-    // about eight blocks per SM in all, or fewer when the clauses do not fill them
-    const long long need = ((long long)I.m + kThreads - 1) / kThreads;
-    const long long gx = std::max<long long>(1, std::min<long long>(need, (152LL * 8 + gy - 1) / gy));
-    k_eval_sparse<VW><<<dim3((unsigned)gx, (unsigned)gy), kThreads, 0, st>>>(
-        EvalInst{I.m, I.kfix, I.coff, I.lit, I.w}, bits, wpr, nb, wbits, cost);
+    // about eight blocks per SM in all, or fewer when the clauses do not fill
+    // them; long clauses are spread over all warps
+    const long long blocks = (152LL * 8 + gy - 1) / gy;
+    const bool lng = max_len > kLongClause;
+    const int cpw = lng ? (int)std::min<long long>(32, (I.m + blocks * kEvalWarps - 1) / (blocks * kEvalWarps)) : 32;
+    const long long need = ((long long)I.m + kEvalWarps * cpw - 1) / (kEvalWarps * cpw);
+    const long long gx = std::max<long long>(1, std::min<long long>(need, blocks));
+    const dim3 grid((unsigned)gx, (unsigned)gy);
+    const EvalInst E{I.m, I.kfix, I.coff, I.lit, I.w};
+    if (lng) k_eval_sparse<VW, true><<<grid, kThreads, 0, st>>>(E, bits, wpr, nb, wbits, cpw, cost);
+    else k_eval_sparse<VW, false><<<grid, kThreads, 0, st>>>(E, bits, wpr, nb, wbits, cpw, cost);
 }
 
 // The batch is a (int8 [n][nb]) or, where a is nullptr, x (float [n][nb],
@@ -276,7 +326,7 @@ static void launch_eval_vw(const DevInst &I, const int8_t *a, const float *x, in
 // eval_sparse_bytes(n, min(nb, chunk)) of scratch, or nullptr for the direct
 // kernel.
 cudaError_t launch_eval_sparse(const DevInst &I, const int8_t *a, const float *x, int nb, int chunk, int wbits,
-                               uint32_t *bits, long long *cost_out, cudaStream_t st) {
+                               int max_len, uint32_t *bits, long long *cost_out, cudaStream_t st) {
     cudaError_t e = cudaSuccess;
     if (I.m == 0 || !bits) {
         e = cudaMemsetAsync(cost_out, 0, sizeof(long long) * (size_t)nb, st);
@@ -290,8 +340,13 @@ cudaError_t launch_eval_sparse(const DevInst &I, const int8_t *a, const float *x
             const int gy = (k + 31) / 32;
             const dim3 grid((unsigned)std::max<long long>(1, std::min<long long>(need, (152LL * 8 + gy - 1) / gy)),
                             (unsigned)gy);
-            if (a) k_eval_direct<int8_t><<<grid, kThreads, 0, st>>>(E, a + b0, nb, k, cost + b0);
-            else k_eval_direct<float><<<grid, kThreads, 0, st>>>(E, x + b0, nb, k, cost + b0);
+            if (k == nb) {
+                if (a) k_eval_direct<int8_t, false><<<grid, kThreads, 0, st>>>(E, a, nb, k, cost);
+                else k_eval_direct<float, false><<<grid, kThreads, 0, st>>>(E, x, nb, k, cost);
+            } else {
+                if (a) k_eval_direct<int8_t, true><<<grid, kThreads, 0, st>>>(E, a + b0, nb, k, cost + b0);
+                else k_eval_direct<float, true><<<grid, kThreads, 0, st>>>(E, x + b0, nb, k, cost + b0);
+            }
             e = cudaGetLastError();
         }
         return e;
@@ -302,9 +357,9 @@ cudaError_t launch_eval_sparse(const DevInst &I, const int8_t *a, const float *x
         const float *xk = a ? nullptr : x + b0;
         unsigned long long *cost = reinterpret_cast<unsigned long long *>(cost_out) + b0;
         switch (eval_vw(k)) {
-            case 4: launch_eval_vw<4>(I, ak, xk, nb, k, wbits, bits, cost, st); break;
-            case 2: launch_eval_vw<2>(I, ak, xk, nb, k, wbits, bits, cost, st); break;
-            default: launch_eval_vw<1>(I, ak, xk, nb, k, wbits, bits, cost, st); break;
+            case 4: launch_eval_vw<4>(I, ak, xk, nb, k, wbits, max_len, bits, cost, st); break;
+            case 2: launch_eval_vw<2>(I, ak, xk, nb, k, wbits, max_len, bits, cost, st); break;
+            default: launch_eval_vw<1>(I, ak, xk, nb, k, wbits, max_len, bits, cost, st); break;
         }
         e = cudaGetLastError();
     }

@@ -318,9 +318,9 @@ cudaError_t launch_solo_steps(const SoloDev &V, const DevInst &I, const DevState
                               int n_steps, bool final_eval, cudaStream_t st);
 bool solo_pays(const SoloDev &V, const DevInst &I, int64_t nnz, int max_len, int64_t steps, double slack);
 size_t eval_sparse_bytes(int n, int nb);
-bool eval_is_direct(int64_t nnz, int nb);
+bool eval_is_direct(int64_t nnz, int max_len, int nb);
 cudaError_t launch_eval_sparse(const DevInst &I, const int8_t *a, const float *x, int nb, int chunk, int wbits,
-                               uint32_t *bits, long long *cost_out, cudaStream_t st);
+                               int max_len, uint32_t *bits, long long *cost_out, cudaStream_t st);
 cudaError_t launch_heuristic_gap(const DevInst &I, const float *x, long long *heur_unsat,
                                  long long *disagree, cudaStream_t st);
 int dense_tile_n(int nb);

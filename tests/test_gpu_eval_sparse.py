@@ -90,3 +90,31 @@ def test_captured_evaluation_outlives_the_buffer(pkg):
             g.replay()
             torch.cuda.synchronize()
             assert np.array_equal(out.cpu().numpy(), _want(cnf, a.cpu().numpy()))
+
+
+@pytest.mark.parametrize("count", [1, 300, 30000, 330000])
+@pytest.mark.parametrize("nb", [1, 33, 65, 130])
+def test_long_clauses_are_read_by_the_warp(pkg, count, nb):
+    """Clauses at the edges of 32 literals and of the warp's batches of 128,
+    alone and among short and empty ones, for one to 32 clauses a warp."""
+    import torch
+    rng = np.random.default_rng(count + nb)
+    n = 5000
+    lens = rng.integers(0, 4, size=count)
+    at = rng.choice(count, size=min(count, 40), replace=False)
+    lens[at] = rng.choice([32, 33, 64, 65, 127, 128, 129, 160, 161, 4000], size=at.size)
+    lens[at[0]] = 129
+    off = np.concatenate([[0], np.cumsum(lens)]).astype(np.int64)
+    lits = ((rng.integers(0, n, size=off[-1]) + 1) * rng.choice([-1, 1], size=off[-1])).astype(np.int32)
+    a = rng.choice(np.array([-1, 1], np.int8), size=(n, nb))
+    # long clauses that one assignment leaves unsat, and some with one true literal
+    for i, j in enumerate(at):
+        lits[off[j]:off[j + 1]] = np.abs(lits[off[j]:off[j + 1]]) * -a[np.abs(lits[off[j]:off[j + 1]]) - 1, i % nb]
+        if i % 3 == 1:
+            k = off[j] + rng.integers(lens[j])
+            lits[k] = -lits[k]
+    for w in (None, rng.integers(1, 1 << 40, size=count)):
+        cnf = Cnf(n, off, lits, w)
+        with pkg.Solver.from_cnf(cnf, restarts=1) as s:
+            got = s.evaluate(torch.from_numpy(a).cuda(), "sparse").cpu().numpy()
+        assert np.array_equal(got, _want(cnf, a))
