@@ -770,6 +770,11 @@ cudaError_t launch_solo_steps(const SoloDev &V, const DevInst &I, const DevState
 // 36), for clauses that are not all of three literals 2 + 0.15 per literal of
 // the longest, or 0.3 with four or more restarts (ordering principle, B=8:
 // 20.5), and then 12 for a launch of heavy variables (Zipf n=3000, B=4: 37).
+// An evaluation alone (no steps) is half a step here, reads one of the three
+// state arrays and writes none, and the two passes may cost 1.1 times their
+// estimate, which counts none of the host's launches.  Whole calls, passes /
+// here: 5-SAT n=1200, B=16 35.7 / 46.6 us, weighted Zipf n=3000, B=1 38.0 /
+// 46.2, 4-SAT n=800, B=1024 92.8 / 76.5, 3-SAT n=1000, B=16 37.2 / 35.1.
 // slack: factor allowed to this kernel.
 bool solo_pays(const SoloDev &V, const DevInst &I, int64_t nnz, int max_len, int64_t steps, double slack) {
     const double waves = (I.B + V.sms - 1) / V.sms;
@@ -777,7 +782,8 @@ bool solo_pays(const SoloDev &V, const DevInst &I, int64_t nnz, int max_len, int
     const double passes = 10.0 + 1.5e-6 * (double)nnz * I.B +
                           (I.kfix == 3 ? 0.0 : 2.0 + (I.B < 4 ? 0.15 : 0.3) * max_len) +
                           (I.n_heavy > 0 && I.B >= 4 ? 12.0 : 0.0);
-    return (double)steps * solo + 8.0 + 7e-5 * (double)I.n * I.B <= slack * (double)std::max<int64_t>(steps, 1) * passes;
+    if (steps == 0) return 0.5 * solo + 8.0 + 2e-5 * (double)I.n * I.B <= 1.1 * slack * passes;
+    return (double)steps * solo + 8.0 + 7e-5 * (double)I.n * I.B <= slack * (double)steps * passes;
 }
 
 }  // namespace msat

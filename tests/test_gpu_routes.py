@@ -7,7 +7,7 @@ import ctypes
 import numpy as np
 import pytest
 
-from synth import Cnf, uniform_ksat
+from synth import Cnf, uniform_ksat, zipf_weighted
 
 pytestmark = pytest.mark.gpu
 
@@ -165,3 +165,21 @@ def test_heavy_variable_of_several_chunks(pkg, oracle, k, B, shape):
         cost = [s.step(1, want_loss=False, per_pass=True)[1] for _ in range(S)]
         assert np.array_equal(np.stack(cost), ref["cost_hist"][1:])
         assert np.array_equal(s.x().astype(np.float64), ref["x_final"])
+
+
+@pytest.mark.parametrize("make,B,solo", [(lambda: uniform_ksat(1200, 25200, 5, seed=1), 16, False),
+                                         (lambda: zipf_weighted(3000, 15000, seed=1), 1, False),
+                                         (lambda: uniform_ksat(800, 7900, 4, seed=1), 1024, True),
+                                         (lambda: uniform_ksat(1000, 4300, 3, seed=1), 16, True)])
+def test_route_of_an_evaluation_alone(pkg, make, B, solo):
+    """A call without steps takes the route that its evaluation alone is faster
+    on; both give the same costs and best assignments."""
+    cnf = make()
+    got = []
+    for per_pass in (False, True):
+        with pkg.Solver.from_cnf(cnf, restarts=B, lr=1e-2) as s:
+            assert _solo(s, 0) == solo
+            s.step(2, want_loss=False, per_pass=True)
+            got.append((s.step(0, want_loss=False, per_pass=per_pass)[1], *s.best()))
+    for u, v in zip(*got):
+        assert np.array_equal(u, v)
