@@ -55,18 +55,22 @@ struct NvtxRange {
 // The array is usually fresh from the allocator, and a copy into pages that
 // the host has not touched yet costs far more than the touching: 16 MB of
 // fresh heap 14 ms, after one write a page 0.7 (64 MB, eight cores: 2.9 ->
-// 1.8).  The writes keep what is there: work of the stream that is still to run
-// may read or write the array, and a copy that fails leaves it as it was.
+// 1.8).  The stream is waited for first: work still to run may read the
+// array, and a call that cannot wait (its stream is being captured) leaves it
+// as it was.  Touching that keeps what is there costs more: 64 MB 1.2 ms by
+// writes, 1.7 by madvise, 25 by atomics, whose first fault is a read's.
 static cudaError_t copy_out(void *dst, const void *src, size_t bytes, cudaStream_t st) {
     cudaPointerAttributes at{};
     const bool plain = bytes >= (1 << 20) && cudaPointerGetAttributes(&at, dst) == cudaSuccess &&
                        at.type == cudaMemoryTypeUnregistered;
     cudaGetLastError();
     if (plain) {  // pinned, managed or device memory has its pages
+        const cudaError_t e = cudaStreamSynchronize(st);
+        if (e) return e;
         const size_t page = (size_t)sysconf(_SC_PAGESIZE);
-        char *d = static_cast<char *>(dst);
+        volatile char *d = static_cast<volatile char *>(dst);
         auto touch = [=](size_t b, size_t e) {
-            for (size_t q = b; q < e; q += page) __atomic_fetch_or(d + q, 0, __ATOMIC_RELAXED);
+            for (size_t q = b; q < e; q += page) d[q] = 0;
         };
         const int T = (int)std::max<size_t>(1, std::min<size_t>(8, bytes >> 23));
         std::thread th[8];
@@ -77,7 +81,7 @@ static cudaError_t copy_out(void *dst, const void *src, size_t bytes, cudaStream
             touch(bytes * t / T, bytes);
         }
         touch(0, bytes / T);
-        __atomic_fetch_or(d + bytes - 1, 0, __ATOMIC_RELAXED);
+        d[bytes - 1] = 0;
         for (std::thread &x : th)
             if (x.joinable()) x.join();
     }
