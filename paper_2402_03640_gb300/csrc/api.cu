@@ -189,6 +189,15 @@ static int multiprocessors() {
     return sms;
 }
 
+// Occurrences of the longest variable that a light block takes: its leaves
+// times the restart groups are at most the block's tasks.
+static int32_t heavy_limit(const msat_config &cfg) {
+    const int32_t B = cfg.restarts, vw = cfg.stage_vw > 0 ? std::min(cfg.stage_vw, B) : auto_stage_vw(B);
+    const int32_t GS = std::max(1, B / vw);
+    const int32_t task_cap = std::max(cfg.light_rows > 0 ? cfg.light_rows : kTaskCap, GS);
+    return std::min(cfg.heavy_deg > 0 ? cfg.heavy_deg : kLightMaxDeg, std::min(32 * (task_cap / GS), kLightMaxDeg));
+}
+
 static bool valid_restarts(int32_t B) {
     return B >= 1 && B <= 1024 && (B & (B - 1)) == 0;
 }
@@ -227,7 +236,20 @@ int msat::ctx_create(msat_ctx **out, int32_t n_vars, int64_t n_clauses, const in
     const bool use_fstore = cfg.f_mode == MSAT_F_STORE || (cfg.f_mode == MSAT_F_AUTO && auto_store);
     HostCnf hc;
     DevCnf dv(pool_alloc);
-    bool on_dev = dev_prep && use_fstore && m > 0 && dev_cnf_worth(n_vars, m, clause_off[m]) &&
+    // rows of the store are grouped by the variable pass's light blocks: by
+    // default when the store is above 32 MiB and so mostly gathered from HBM;
+    // never for the serving engine's contexts (their batched kernels read
+    // clause order)
+    const bool grouped = use_fstore && !pool_alloc &&
+                         (cfg.row_order == 2 ||
+                          (cfg.row_order == 0 && (double)m * cfg.restarts * sizeof(float) > 32.0 * (1 << 20)));
+    // where that leaves more clauses of heavy variables alone than the device
+    // sorts, which is certain once the average variable is heavy, the host
+    // prepares the instance from the start (7-SAT n=3000, m=250000, B=64 9.4 ->
+    // 8.5 ms, 5-SAT n=3000, m=63000, B=1024 3.5 -> 2.8; 8.2 and 2.9 before there
+    // was a device path)
+    const bool all_heavy = grouped && m > 0 && clause_off[m] / n_vars > heavy_limit(cfg);
+    bool on_dev = dev_prep && use_fstore && m > 0 && !all_heavy && dev_cnf_worth(n_vars, m, clause_off[m]) &&
                   dv.check(n_vars, m, clause_off, lits, weights, stream, hc);
     if (!on_dev) {
         dv.clear();  // what the device path took is the host path's to use
@@ -268,9 +290,7 @@ int msat::ctx_create(msat_ctx **out, int32_t n_vars, int64_t n_clauses, const in
     if (cfg.loss_norm < MSAT_LOSS_MEAN_UNSAT || cfg.loss_norm > MSAT_LOSS_MEAN_ALL)
         return fail(MSAT_EINVAL, "msat_create: unknown loss_norm");
     if (cfg.row_order < 0 || cfg.row_order > 2) return fail(MSAT_EINVAL, "msat_create: unknown row_order");
-    const int32_t leaf_room = 32 * (task_cap / GS);  // occurrences of the longest light variable
-    const int32_t heavy_deg = std::min(cfg.heavy_deg > 0 ? cfg.heavy_deg : kLightMaxDeg,
-                                       std::min(leaf_room, kLightMaxDeg));
+    const int32_t heavy_deg = heavy_limit(cfg);
     std::vector<int32_t> hvar, hchunk0(1, 0);
     std::vector<int2> lblk;
     {
@@ -309,14 +329,8 @@ int msat::ctx_create(msat_ctx **out, int32_t n_vars, int64_t n_clauses, const in
     // expanded occurrence record streamed with the occurrence list
     const bool expand = cfg.f_mode == MSAT_F_EXPANDED ||
                         (cfg.f_mode == MSAT_F_AUTO && !use_fstore && kfix == 3 && m < (1LL << 28));
-    // rows of the store grouped by the variable pass's light blocks (the
-    // occurrence words carry rows; every sum keeps its order): by default
-    // when the store is above 32 MiB and so mostly gathered from HBM;
-    // never for the serving engine's contexts (their batched kernels read
-    // clause order)
-    const bool block_rows = use_fstore && !expand && !pool_alloc &&
-                            (cfg.row_order == 2 ||
-                             (cfg.row_order == 0 && (double)m * B * sizeof(float) > 32.0 * (1 << 20)));
+    // with grouped rows the occurrence words carry rows; every sum keeps its order
+    const bool block_rows = grouped && !expand;
     RowOrder ro;
     if (on_dev && ((block_rows && !dv.rows(lblk)) || !dv.occurrences())) {
         // a row group past the device sort, or no memory: the host path after

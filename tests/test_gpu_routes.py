@@ -183,3 +183,17 @@ def test_route_of_an_evaluation_alone(pkg, make, B, solo):
             got.append((s.step(0, want_loss=False, per_pass=per_pass)[1], *s.best()))
     for u, v in zip(*got):
         assert np.array_equal(u, v)
+
+
+@pytest.mark.parametrize("B,want", [(1, "device"), (1024, "host")])
+def test_instance_of_heavy_variables_is_prepared_by_the_host(pkg, B, want):
+    """With grouped rows (B=1024) and an average variable past the light
+    blocks' reach, nearly every clause has heavy variables alone."""
+    import torch
+    cnf = uniform_ksat(3000, 63000, 5, seed=1)
+    a = np.random.default_rng(1).choice(np.array([-1, 1], np.int8), size=(cnf.n, 2))
+    with pkg.Solver.from_cnf(cnf, restarts=B) as s:
+        assert _prep(s) == want
+        got = s.evaluate(torch.from_numpy(a).cuda(), "sparse").cpu().numpy()
+    sat = ((a[np.abs(cnf.lits) - 1] > 0) == (cnf.lits > 0)[:, None]).reshape(cnf.m, 5, 2).any(axis=1)
+    assert np.array_equal(got, (~sat).sum(axis=0))
