@@ -347,17 +347,23 @@ int msat::ctx_create(msat_ctx **out, int32_t n_vars, int64_t n_clauses, const in
     // lists of the one-block-per-restart kernel, if it may take this instance
     SoloHost solo;
     auto make_solo = [&, sms = multiprocessors()]() -> bool {
-        if (!build_solo(n_vars, m, kfix, max_len, max_deg, hc, weights, solo)) return false;
+        auto pays = [&](const SoloDev &V) {
+            SoloDev v = V;
+            v.sms = sms;
+            DevInst shape{};
+            shape.n = n_vars;
+            shape.B = B;
+            shape.kfix = kfix;
+            shape.n_heavy = (int32_t)hvar.size();
+            // for a long call, with room for what the estimate does not know;
+            // each call then takes the faster route (the serving engine has
+            // only one, and its batch does not start a step for this instance
+            // alone)
+            return solo_pays(v, shape, nnz, max_len, 1 << 30, pool_alloc ? 1.5 : 2.0);
+        };
+        const bool ok = build_solo(n_vars, m, kfix, max_len, max_deg, hc, weights, pays, solo);
         solo.dev.sms = sms;
-        DevInst shape{};
-        shape.n = n_vars;
-        shape.B = B;
-        shape.kfix = kfix;
-        shape.n_heavy = (int32_t)hvar.size();
-        // for a long call, with room for what the estimate does not know; each
-        // call then takes the faster route (the serving engine has only one,
-        // and its batch does not start a step for this instance alone)
-        return solo_pays(solo.dev, shape, nnz, max_len, 1 << 30, pool_alloc ? 1.5 : 2.0);
+        return ok;
     };
     // by a thread of its own beside the rest of the creation, which does not
     // read them (the serving engine's does), from this many literals on: the
@@ -578,9 +584,9 @@ int msat::ctx_create(msat_ctx **out, int32_t n_vars, int64_t n_clauses, const in
     if (solo_made.valid()) use_solo = solo_made.get();
     c->clen = std::move(hc.clen);
     if (!e && use_solo) {
-        rc = dalloc_t(c, &d_slists, solo.lists.size());
+        rc = dalloc_t(c, &d_slists, solo.bytes);
         if (!rc) {
-            e = up(d_slists, solo.lists.data(), solo.lists.size());
+            e = up(d_slists, solo.lists.get(), solo.bytes);
             c->solo = solo.dev;
             c->solo.lists = d_slists;
             c->solo.perm = reinterpret_cast<const int *>(d_slists + solo.perm_at);

@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <functional>
 #include <memory>
 #include <vector>
 
@@ -85,15 +86,16 @@ void scatter_occurrences(int32_t n, int64_t m, HostCnf &hc, const I32Buf *row);
 // instance without solo_fits does).  dev holds the sizes and offsets (its
 // pointers are set after the upload); behind the lists, in the same array, lie
 // the internal variable order -> variable table and, where the clauses are in
-// another order, the weights in slot order (w_at 0: there are none).  Reads
+// another order, the weights in slot order (w_at 0: there are none).  pays:
+// asked with the sizes before the lists are filled; false ends there.  Reads
 // coff, lit, voff and clen of hc.
 struct SoloHost {
     SoloDev dev;
-    std::vector<unsigned char> lists;
-    size_t perm_at = 0, w_at = 0;
+    std::unique_ptr<unsigned char[]> lists;
+    size_t bytes = 0, perm_at = 0, w_at = 0;
 };
 bool solo_fits(int32_t n, int64_t m, int32_t max_deg);
 bool build_solo(int32_t n, int64_t m, int32_t kfix, int32_t max_len, int32_t max_deg, const HostCnf &hc,
-                const int64_t *w, SoloHost &out);
+                const int64_t *w, const std::function<bool(const SoloDev &)> &pays, SoloHost &out);
 
 }  // namespace msat

@@ -33,6 +33,9 @@
 #include <stdint.h>
 
 #include <algorithm>
+#include <functional>
+#include <future>
+#include <system_error>
 #include <vector>
 
 #include "host_cnf.cuh"
@@ -524,7 +527,7 @@ bool solo_fits(int32_t n, int64_t m, int32_t max_deg) {
 }
 
 bool build_solo(int32_t n, int64_t m, int32_t kfix, int32_t max_len, int32_t max_deg, const HostCnf &hc,
-                const int64_t *w, SoloHost &out) {
+                const int64_t *w, const std::function<bool(const SoloDev &)> &pays, SoloHost &out) {
     if (!solo_fits(n, m, max_deg)) return false;
     SoloDev &V = out.dev;
     V = SoloDev{};
@@ -559,31 +562,30 @@ bool build_solo(int32_t n, int64_t m, int32_t kfix, int32_t max_len, int32_t max
     if (solo_smem(n, (int)m, sh.n_mtask, false, 0).total > kSoloSmemMax) return false;
 
     // clauses: slots by falling length (all equal: clause order)
-    std::vector<int32_t> slot, of;  // clause -> slot, slot -> clause
+    I32Buf slot;  // clause -> slot
+    const int64_t nsl = (m + 31) / 32;
+    std::vector<int32_t> lbase((size_t)nsl + 1, 0);
     if (kfix == 0 && m > 0) {
-        slot.resize((size_t)m);
-        of.resize((size_t)m);
-        const int32_t top = (max_len + 3) / 4;
+        slot.alloc((size_t)m);
+        const int32_t top = (max_len + 3) / 4;  // bucket k: clauses of top - k rows
         std::vector<int32_t> at((size_t)top + 2, 0);
         for (int64_t j = 0; j < m; ++j) ++at[(size_t)(top - (hc.clen[(size_t)j] + 3) / 4) + 1];
         for (int32_t k = 0; k <= top; ++k) at[(size_t)k + 1] += at[(size_t)k];
-        for (int64_t j = 0; j < m; ++j) {
-            const int32_t s = at[(size_t)(top - (hc.clen[(size_t)j] + 3) / 4)]++;
-            slot[(size_t)j] = s;
-            of[(size_t)s] = (int32_t)j;
+        int32_t k = 0;
+        for (int64_t s = 0; s < nsl; ++s) {  // a slice's first clause is its longest
+            while (at[(size_t)k + 1] <= 32 * s) ++k;
+            lbase[(size_t)s + 1] = lbase[(size_t)s] + std::max(1, top - k);
         }
+        for (int64_t j = 0; j < m; ++j)
+            slot[(size_t)j] = at[(size_t)(top - (hc.clen[(size_t)j] + 3) / 4)]++;
+    } else {
+        for (int64_t s = 0; s < nsl; ++s) lbase[(size_t)s + 1] = lbase[(size_t)s] + std::max(1, (kfix + 3) / 4);
     }
     V.kind = kfix == 3 ? 0 : max_len <= 32 ? 1 : 2;
     // signed pairs of w*f where they fit: an occurrence word is then slot <<
     // 1 | neg, else the slot, with the signs apart (m + 1 pairs fit only for
     // m < 32767)
     V.pairs = V.kind < 2 && solo_smem(n, (int)m, sh.n_mtask, true, 0).total <= kSoloSmemMax;
-    const int64_t nsl = (m + 31) / 32;
-    std::vector<int32_t> lbase((size_t)nsl + 1, 0);
-    for (int64_t s = 0; s < nsl; ++s) {
-        const int32_t len = kfix > 0 ? kfix : m > 0 ? hc.clen[(size_t)of[(size_t)(32 * s)]] : 0;
-        lbase[(size_t)s + 1] = lbase[(size_t)s] + std::max(1, (len + 3) / 4);
-    }
     sh.lit_rows = lbase[(size_t)nsl];
 
     // leaf tasks: those of the variables of several leaves in (variable,
@@ -616,6 +618,12 @@ bool build_solo(int32_t n, int64_t m, int32_t kfix, int32_t max_len, int32_t max
         obase[(size_t)s + 1] = obase[(size_t)s] + std::max(1, (mx + 3) / 4);
     }
     sh.occ_rows = obase[(size_t)ntsl];
+    V.n_single = sh.n_single;
+    V.n_multi = sh.n_multi;
+    V.n_wide = sh.n_wide;
+    V.n_mtask = sh.n_mtask;
+    V.rows = (int)(sh.lit_rows + sh.occ_rows);
+    if (!pays(V)) return false;
 
     // one array: literal rows, occurrence rows, then the small tables
     uint32_t at = 0;
@@ -632,61 +640,78 @@ bool build_solo(int32_t n, int64_t m, int32_t kfix, int32_t max_len, int32_t max
     V.list_bytes = at;
     uint32_t perm_at = 0, w_at = 0;
     place(perm_at, sizeof(int32_t) * (size_t)n);
-    if (w && !slot.empty()) place(w_at, sizeof(int64_t) * (size_t)m);
+    if (w && slot.size() > 0) place(w_at, sizeof(int64_t) * (size_t)m);
     out.perm_at = perm_at;
     out.w_at = w_at;
-    out.lists.assign(at, 0);
-    uint16_t *lw = reinterpret_cast<uint16_t *>(out.lists.data() + V.off_lit);
-    uint16_t *ow = reinterpret_cast<uint16_t *>(out.lists.data() + V.off_occ);
-    uint32_t *sg = reinterpret_cast<uint32_t *>(out.lists.data() + V.off_sgn);
-    std::copy(lbase.begin(), lbase.end(), reinterpret_cast<int32_t *>(out.lists.data() + V.off_lit_base));
-    std::copy(obase.begin(), obase.end(), reinterpret_cast<int32_t *>(out.lists.data() + V.off_occ_base));
-    std::copy(mbeg.begin(), mbeg.end(), reinterpret_cast<int32_t *>(out.lists.data() + V.off_mbeg));
-    std::fill(lw, lw + sh.lit_rows * 128, (uint16_t)(n << 1));
-    std::fill(ow, ow + sh.occ_rows * 128, (uint16_t)(V.pairs ? 2 * m : m));
-    // per variable: its word, where its current leaf's words go, the leaf
-    // task and the occurrences and signs placed in it
+    out.bytes = at;
+    out.lists.reset(new unsigned char[at]);
+    // every byte but the gaps between the tables is written below
+    uint16_t *lw = reinterpret_cast<uint16_t *>(out.lists.get() + V.off_lit);
+    uint16_t *ow = reinterpret_cast<uint16_t *>(out.lists.get() + V.off_occ);
+    uint32_t *sg = reinterpret_cast<uint32_t *>(out.lists.get() + V.off_sgn);
+    std::copy(lbase.begin(), lbase.end(), reinterpret_cast<int32_t *>(out.lists.get() + V.off_lit_base));
+    std::copy(obase.begin(), obase.end(), reinterpret_cast<int32_t *>(out.lists.get() + V.off_occ_base));
+    std::copy(mbeg.begin(), mbeg.end(), reinterpret_cast<int32_t *>(out.lists.get() + V.off_mbeg));
+    // the words of the clauses, by a thread of their own where they are many
+    // (a thread costs about 25 us, the words 1 to 2 ns each)
+    constexpr int64_t kApart = 1 << 15;
+    std::vector<int32_t> id_of((size_t)n);
+    for (int32_t id = 0; id < n; ++id) id_of[(size_t)perm[(size_t)id]] = id;
+    auto slot_at = [&](int64_t j) { return (uint32_t)(kfix > 0 ? j : slot[(size_t)j]); };
+    auto lit_words = [&] {
+        std::fill(lw, lw + sh.lit_rows * 128, (uint16_t)(n << 1));
+        for (int64_t j = 0; j < m; ++j) {
+            const uint32_t s = slot_at(j);
+            uint16_t *l0 = lw + ((size_t)lbase[s >> 5] * 32 + (s & 31u)) * 4;
+            const int32_t *c = lit + coff[j];
+            const int32_t len = coff[j + 1] - coff[j];
+            for (int32_t r = 0; r < len; ++r)
+                l0[(r >> 2) * 128 + (r & 3)] = (uint16_t)((id_of[(size_t)(c[r] >> 1)] << 1) | (c[r] & 1));
+        }
+    };
+    std::future<void> apart;
+    if (hc.nnz >= kApart) {
+        try {
+            apart = std::async(std::launch::async, lit_words);
+        } catch (const std::system_error &) {  // no more threads
+        }
+    }
+    if (!apart.valid()) lit_words();
+    // per variable: where its current leaf's words go, the leaf task and the
+    // occurrences and signs placed in it
     struct Fill {
-        uint32_t word, at, task, cnt, sgn;
+        uint32_t at, task, cnt, sgn;
     };
     std::vector<Fill> fill((size_t)n);
     auto leaf_at = [&](uint32_t k) { return ((uint32_t)obase[k >> 5] * 32u + (k & 31u)) * 4u; };
     for (int32_t id = 0; id < n; ++id) {
         const uint32_t k = (uint32_t)tfirst[(size_t)id];
-        fill[(size_t)perm[(size_t)id]] = Fill{(uint32_t)id << 1, leaf_at(k), k, 0u, 0u};
+        fill[(size_t)perm[(size_t)id]] = Fill{leaf_at(k), k, 0u, 0u};
     }
     const uint32_t pairs = V.pairs ? 1u : 0u;
+    std::fill(ow, ow + sh.occ_rows * 128, (uint16_t)(V.pairs ? 2 * m : m));
     for (int64_t j = 0; j < m; ++j) {
-        const uint32_t s = (uint32_t)(kfix > 0 ? j : slot[(size_t)j]);
-        uint16_t *l0 = lw + ((size_t)lbase[s >> 5] * 32 + (s & 31u)) * 4;
-        const int32_t *c = lit + coff[j];
-        const int32_t len = coff[j + 1] - coff[j];
-        for (int32_t r = 0; r < len; ++r) {
-            const uint32_t neg = (uint32_t)c[r] & 1u;
-            Fill &F = fill[(size_t)(c[r] >> 1)];
+        const uint32_t s = slot_at(j);
+        for (int32_t p = coff[j]; p < coff[j + 1]; ++p) {
+            const uint32_t neg = (uint32_t)lit[p] & 1u;
+            Fill &F = fill[(size_t)(lit[p] >> 1)];
             if (F.cnt == 32u) {
                 sg[F.task] = F.sgn;
                 ++F.task;
                 F.at = leaf_at(F.task);
                 F.cnt = F.sgn = 0u;
             }
-            l0[(r >> 2) * 128 + (r & 3)] = (uint16_t)(F.word | neg);
             ow[F.at + (F.cnt >> 2) * 128u + (F.cnt & 3u)] = (uint16_t)((s << pairs) | (neg & pairs));
             F.sgn |= neg << F.cnt;
             ++F.cnt;
         }
     }
     for (const Fill &F : fill) sg[F.task] = F.sgn;
-    std::copy(perm.begin(), perm.end(), reinterpret_cast<int32_t *>(out.lists.data() + perm_at));
+    std::copy(perm.begin(), perm.end(), reinterpret_cast<int32_t *>(out.lists.get() + perm_at));
     if (w_at) {
-        int64_t *sw = reinterpret_cast<int64_t *>(out.lists.data() + w_at);
+        int64_t *sw = reinterpret_cast<int64_t *>(out.lists.get() + w_at);
         for (int64_t j = 0; j < m; ++j) sw[slot[(size_t)j]] = w[j];
     }
-    V.n_single = sh.n_single;
-    V.n_multi = sh.n_multi;
-    V.n_wide = sh.n_wide;
-    V.n_mtask = sh.n_mtask;
-    V.rows = (int)(sh.lit_rows + sh.occ_rows);
     return true;
 }
 
