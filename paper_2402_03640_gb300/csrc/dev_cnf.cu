@@ -13,7 +13,8 @@
 // What bounds it: the upload of the caller's arrays (86 MB at n=1e6,
 // m=4.3e6) and one host pass over the occurrence offsets (the partition into
 // light blocks); the kernels are random 4-byte atomics and gathers, about 13
-// million a pass.  3-SAT n=1e6, m=4.3e6, B=16: msat_create 43.7 -> 5.8 ms.
+// million a pass, 0.9 ms in all (k_row_sort 0.21, k_occ_sort 0.19, k_occ_scatter
+// 0.16 ms).  3-SAT n=1e6, m=4.3e6, B=1: msat_create 32 -> 5.3 ms.
 
 #include <cuda_runtime.h>
 #include <limits.h>
